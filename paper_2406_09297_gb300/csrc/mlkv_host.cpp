@@ -862,6 +862,7 @@ static int fused_issue(mlkv_cache_t c, const void *Q, void *out, int n_q_layers,
     p.G = c->G;
     p.s_max = c->max_seq;
     p.slot = slot0;
+    p.sm_count = c->sm_count;
     p.head_pairs = 0;
     p.fused_L = L;
     p.fused_L1 = L1;
@@ -1859,6 +1860,7 @@ int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const 
     p.G = c->G;
     p.s_max = s_max;
     p.slot = c->slot[layer];
+    p.sm_count = c->sm_count;
     p.fused_L = p.fused_L1 = 0;
     for (int beta = 0; beta < c->b; ++beta)
         p.prompt_len[beta] = prompt_lens[beta];

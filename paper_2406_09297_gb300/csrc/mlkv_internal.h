@@ -103,6 +103,7 @@ struct PrefillParams {
     int *err;                 // device error word
     float scale_log2;         // log2(e) / sqrt(D)
     int b, h, g, G, s_max, slot, n_units, head_pairs;
+    int sm_count;             // the launch's persistent CTAs: one or two per SM, at most n_units
     // Cross-layer fused decode (mlkv_decode_block_fused, and mlkv_decode_step's fused form): every
     // block has L layers, L1 of them in tile B (the rest in tile A); prompt_len holds the sequence
     // lengths.  Both 0 for prefill.  A unit's block blk (fused_nblk blocks in all) reads slot

@@ -5,14 +5,19 @@
 // attention, Eqs. 2-3 with the MLKV maps of Eqs. 13-18).  Owner layers first store the prompt's
 // K/V in their slot (mlkv_host.cpp); every layer of the block then attends over it.
 //
-// Work unit (one CTA), head_dim 128: two query tiles A and B of 128 prompt positions that read the
+// Persistent CTAs: the grid is at most one wave, and CTA c takes units c, 2P - 1 - c, 2P + c, ... of
+// the longest-first list (P CTAs).  All roles run on over the units: while a unit's last tile is in
+// its softmax and its output is stored, the next unit's queries and first K/V tiles arrive and its
+// first S is computed.  With a CTA per unit, every unit paid ~7,500 cycles outside its key tiles
+// (barriers, TMEM, tensor-map fetch, first loads, output); now ~3,000.
+//
+// Work unit, head_dim 128: two query tiles A and B of 128 prompt positions that read the
 // same KV head, so that every K/V tile is loaded once for both.  With an even group size G they are
 // two heads of one group at the same positions (identical causal triangles); otherwise they are the
 // blocks 2p and 2p+1 of one head (B sees one tile more; a last block without a partner runs alone
 // as B).  Prefill at head_dim 64: one query tile (as B) per CTA and two CTAs per SM, each with half
-// the tensor memory; the two CTAs' starts, first loads and outputs overlap each other's key-tile
-// loops (measured 8% faster than two tiles per CTA, although every K/V tile is then fetched once
-// per query tile).  Units that see the most keys run first.
+// the tensor memory, so that one CTA's output overlaps the other's key tiles (although every K/V
+// tile is then fetched once per query tile).  Units that see the most keys run first.
 //
 // Fused decode (one new token per sequence, every layer of an owner block at once, Sec. 3): the
 // query rows of a unit are the G heads of KV head j in each of the block's L layers, row = layer * G
@@ -26,7 +31,9 @@
 //   S_X = Q_X K_t^T  M = 128 queries (A = Q_X, K-major, 128-byte swizzle as TMA wrote it),
 //                    N = 128 keys (B = the K tile), K = head_dim; one query row per TMEM lane.
 //   softmax          a warpgroup per query tile, one thread per row: the thread owns its row's
-//                    128 scores, so the running maximum needs no exchange between threads.  The
+//                    128 scores, so the running maximum needs no exchange between threads; the
+//                    tensor-memory load returns it with the scores (tcgen05.ld.red), so S's
+//                    columns are free for the next S before the weights are formed.  The
 //                    reference maximum is raised only when a score exceeds it by more than 2^8
 //                    (then the thread rescales its O row in TMEM); p = 2^(s log2(e)/sqrt(d) - m)
 //                    goes back to TMEM as bf16 pairs.
@@ -37,7 +44,15 @@
 // TMEM (512 columns, 256 with one query tile): S per tile (128 columns), O per tile (head_dim).
 // For head_dim 64, P has columns of its own (so S of the next tile can be computed while P of this
 // one is being written); for head_dim 128, P overwrites the first 64 columns of its S (tcgen05.mma
-// of one thread execute in order, so S of the next tile is written after P V has read P).
+// of one thread execute in order, so S of the next tile is written after P V has read P), and the
+// product of the first 64 keys starts while the softmax forms the weights of the last 64.
+//
+// What bounds it, per key tile and query tile of an SM: the tensor core (head_dim 64: 4 x 66 cycles
+// of S and 8 x 34 of P V; head_dim 128: 16 x 66) and the softmax warps' issue slots (~690 cycles:
+// 128 exponentials, and paired multiply-adds, sums and conversions that take two slots each).
+// Measured on GB300 (two layers, before -> after the persistent form with early S columns and
+// elected issuing threads): 8 x 2048 positions x 12 heads, head_dim 64, 168.6 -> 132.1 us; 4 x 2048
+// x 32 heads, head_dim 128, 313.8 -> 240.6 us; 32 prompts of 1 to 777 positions 103.7 -> 83.0 us.
 //
 // The diagonal tile masks keys after the query; keys past the prompt's end only meet such masked
 // scores, and their V rows are zeroed in shared memory so that 0 * V stays 0.
@@ -45,10 +60,11 @@
 // Warp roles: 4 softmax warps per query tile (warps 0-3 tile A, 4-7 tile B; the one-tile CTA's
 // warps 0-3 take its tile), then the TMA producer (query tiles, then K_0, V_0, K_1, V_1, ...
 // through a ring), the MMA issuer (for head_dim 64 only of S, the next warp issuing the P V
-// products), the rest idle.  Registers: the two-tile block launches with 168 a thread and its last
-// warpgroup gives registers back (72 or 88) to the softmax warpgroups (216 or 208, head_dim 64 or
-// 128): 128 * low + 256 * high <= 384 * 168; the one-tile block launches with 128 (two blocks per
-// SM) and splits 56 / 200: 128 * 56 + 128 * 200 = 256 * 128.
+// products), and last a warp that loads queries held in host memory (else idle).  Registers: the
+// two-tile block launches with 168 a thread and its last warpgroup gives registers back (72 or 88)
+// to the softmax warpgroups (216 or 208, head_dim 64 or 128): 128 * low + 256 * high <= 384 * 168;
+// the one-tile block launches with 128 (two blocks per SM) and splits 40 / 216: 128 * 40 +
+// 128 * 216 = 256 * 128.
 // Every wait is bounded; on expiry the kernel records an error bit, stops, lets its copies and MMAs
 // land and frees its TMEM.
 #include <type_traits>
@@ -84,24 +100,33 @@ struct PrefillPlan {
     static constexpr int kMinBlocks = kForm == kOneTile ? 2 : 1;
     // registers at launch, then the other warps' share and the softmax warps' (setmaxnreg)
     static constexpr int kRegsLaunch = kForm == kOneTile ? 128 : 168;
-    static constexpr int kRegsLow = kForm == kOneTile ? 56 : (D == 64 ? 72 : 88);
-    static constexpr int kRegsHigh = kForm == kOneTile ? 200 : (D == 64 ? 216 : 208);
+    static constexpr int kRegsLow = kForm == kOneTile ? 40 : (D == 64 ? 72 : 88);
+    static constexpr int kRegsHigh = kForm == kOneTile ? 216 : (D == 64 ? 216 : 208);
     static constexpr int kProducer = kSoftWarps, kMma = kSoftWarps + 1;
     static constexpr int kSub = D / 64;                      // 64-channel blocks of a row
     static constexpr int kTileBytes = 128 * D * 2;           // 128 rows of Q, K or V
     // K_t and V_t alternate in the ring
     static constexpr int kRingTiles = kForm == kOneDeep ? 12 : kOne ? 5 : (D == 64 ? 8 : 4);
-    static constexpr int kQ = 0;                             // [kTiles] query tiles
-    static constexpr int kRing = kQ + kTiles * kTileBytes;
-    static constexpr int kFlags = kRing + kRingTiles * kTileBytes;   // int [4], TMEM base at +16
-    // u64 barriers: q, full[R], empty[R], s_ready[2], s_free[2], p_ready[2], pv_done[2], fin[2]
-    // (s_ready and s_free per query tile, or per S buffer in the deep form)
+    // Query tiles: two sets where shared memory allows it, so that a unit's queries arrive while
+    // the unit before it still runs.
+    static constexpr int kQBufs = D == 64 && kForm != kOneDeep ? 2 : 1;
+    static constexpr int kQ = 0;                             // [kQBufs][kTiles] query tiles
+    static constexpr int kRing = kQ + kQBufs * kTiles * kTileBytes;
+    // Outputs are staged for coalesced stores in the unit's own query tile (head_dim 64), else in
+    // 4 KB per softmax warp.
+    static constexpr bool kStageInQ = D == 64;
+    static constexpr int kStage = kRing + kRingTiles * kTileBytes;
+    static constexpr int kFlags = kStage + (kStageInQ ? 0 : kSoftWarps * 4096);
+                                                             // int [4], TMEM base at +16
+    // u64 barriers: q[2], q_free[2], full[R], empty[R], s_ready[2], s_free[2], p_half[2],
+    // p_ready[2], pv_done[2], fin[2] (s_ready and s_free per query tile, or per S buffer in the
+    // deep form)
     static constexpr int kBars = kFlags + 32;
-    static constexpr int kNumBars = 1 + 2 * kRingTiles + 8 + 2;
+    static constexpr int kNumBars = 4 + 2 * kRingTiles + 10 + 2;
     // the second warpgroup's running maximum and sum per row, for the merge (two buffers)
     static constexpr int kML = kBars + kNumBars * 8;
     static constexpr int kBytes = kML + (kSBuf == 2 ? 128 * 8 : 0);
-    static constexpr int kAlloc = kBytes + 1024;             // base aligned up to 1024
+    static constexpr int kAlloc = kBytes;
     static_assert(kMinBlocks * (kAlloc + 1024) <= 228 * 1024, "shared memory of the resident CTAs");
     static constexpr int kTmemCols = kForm == kOneTile ? 256 : 512;
     static constexpr bool kPSep = D == 64;                   // P in columns of its own
@@ -138,6 +163,62 @@ __device__ __forceinline__ float max3f(float a, float b, float c)
     return d;
 }
 
+// A work unit as its CTA's warps see it (see PrefillParams::units).
+struct Unit {
+    int beta, S;          // sequence; its prompt length, or (fused decode) its length
+    int chunk, blk;       // fused decode: context chunk and owner block (both 0 for prefill)
+    int kt0;              // first key tile (128 positions) of the unit
+    int n_a, n_b;         // key tiles of query tiles A (0: no tile A) and B, n_a <= n_b
+    int qb_b;             // prefill: tile B's query block
+    int head_a, head_b, j;
+    int zk, zv;           // rows of the cache's tensor map: K and V of (slot, sequence, KV head)
+    bool has_end;         // the unit holds the sequence's last key tile
+};
+
+template <bool kFused, int kTiles>
+__device__ __forceinline__ Unit unit_of(const PrefillParams &p, int i)
+{
+    Unit x;
+    const uint32_t u = p.units[i];
+    x.beta = static_cast<int>(u & 0x3FFu);
+    const int sel = static_cast<int>(u >> 24);
+    x.S = p.prompt_len[x.beta];
+    if (kFused) {
+        // every query row sees positions [0, S); the unit takes key tiles [kt0, kt0 + n_b)
+        const int n_kt = (x.S + 127) / 128;
+        x.chunk = static_cast<int>((u >> 10) & 0xFFu);
+        x.blk = static_cast<int>((u >> 18) & 0x3Fu);
+        x.kt0 = x.chunk * p.fused_kc;
+        const int kt1 = min(x.kt0 + p.fused_kc, n_kt);
+        x.has_end = kt1 == n_kt;
+        x.n_b = kt1 - x.kt0;
+        x.n_a = kTiles == 2 && p.fused_L > p.fused_L1 ? x.n_b : 0;
+        x.qb_b = 0;
+        x.head_a = x.head_b = x.j = sel;
+    } else {
+        x.chunk = x.blk = x.kt0 = 0;
+        x.has_end = true;
+        x.qb_b = static_cast<int>((u >> 10) & 0x3FFFu);
+        x.n_b = x.qb_b + 1;
+        x.n_a = kTiles == 1 ? 0 : p.head_pairs ? x.n_b : ((x.qb_b & 1) ? x.qb_b : 0);
+        x.head_a = p.head_pairs ? 2 * sel : sel;
+        x.head_b = p.head_pairs ? 2 * sel + 1 : sel;
+        x.j = x.head_b / p.G;   // Eq. 15
+    }
+    x.zk = (((p.slot + x.blk) * 2 + 0) * p.b + x.beta) * p.g + x.j;
+    x.zv = x.zk + p.b * p.g;
+    return x;
+}
+
+// The CTA's k-th unit, or -1 past its last: a snake deal of the units (longest first) to the
+// persistent CTAs, which evens out their key tiles.
+__device__ __forceinline__ int unit_index(const PrefillParams &p, int k)
+{
+    const int P = static_cast<int>(gridDim.x), c = static_cast<int>(blockIdx.x);
+    const int i = k * P + ((k & 1) ? P - 1 - c : c);
+    return i < p.n_units ? i : -1;
+}
+
 template <int D, bool kFused, int kForm>
 __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
                                   PrefillPlan<D, kForm>::kMinBlocks)
@@ -147,56 +228,40 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
 {
     using PL = PrefillPlan<D, kForm>;
     constexpr bool kSplit = PL::kSBuf == 2;   // key tiles alternate between two warpgroups
+    constexpr int NQ = PL::kQBufs;
+    constexpr int R = PL::kRingTiles;
     // Query tile g's shared-memory slot and tensor-memory columns (the only tile of a one-tile CTA
     // is tile B, in slot 0).
     auto slot_of = [](int g) { return PL::kTiles == 1 ? 0 : g; };
-    constexpr int R = PL::kRingTiles;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    extern __shared__ __align__(1024) uint8_t smem[];   // swizzled tiles: 1024-byte aligned
     const uint32_t sbase = smem_addr(smem);
-    const uint32_t bar_q = sbase + PL::kBars;
-    const uint32_t bar_full = bar_q + 8;
+    const uint32_t bar_q = sbase + PL::kBars;             // [NQ] query tiles loaded
+    const uint32_t bar_q_free = bar_q + 8 * 2;            // [NQ] query tiles read for the last time
+    const uint32_t bar_full = bar_q_free + 8 * 2;
     const uint32_t bar_empty = bar_full + 8 * R;
-    const uint32_t bar_s_ready = bar_empty + 8 * R;   // [2] per query tile
+    const uint32_t bar_s_ready = bar_empty + 8 * R;       // [2] per query tile or S buffer
     const uint32_t bar_s_free = bar_s_ready + 16;
-    const uint32_t bar_p_ready = bar_s_free + 16;
+    const uint32_t bar_p_half = bar_s_free + 16;          // P of the tile's first 64 keys (P over S)
+    const uint32_t bar_p_ready = bar_p_half + 16;
     const uint32_t bar_pv_done = bar_p_ready + 16;
-    const uint32_t bar_fin = bar_pv_done + 16;   // [2]: one per issuing thread
+    const uint32_t bar_fin = bar_pv_done + 16;            // [2]: one per issuing thread
     volatile int *flags = reinterpret_cast<volatile int *>(smem + PL::kFlags);
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    // The unit: sequence, last query block of B, head pair or head (see PrefillParams::units).
-    // Fused decode: sequence, KV head j and owner block blk; S is then the sequence length, every
-    // query row sees positions [0, S), and the tiles hold the block's layers [0, L1) (B) and
-    // [L1, L) (A).
-    const uint32_t u = p.units[blockIdx.x];
-    const int beta = static_cast<int>(u & 0x3FFu);
-    const int sel = static_cast<int>(u >> 24);
-    const int S = p.prompt_len[beta];
-    // Fused decode: key tiles [kt0, kt0 + n_b) of the sequence (a chunk of p.fused_kc tiles).
-    const int chunk = static_cast<int>((u >> 10) & (kFused ? 0xFFu : 0x3FFFu));
-    const int blk = kFused ? static_cast<int>((u >> 18) & 0x3Fu) : 0;
-    const int n_kt = (S + 127) / 128;
-    const int kt0 = kFused ? chunk * p.fused_kc : 0;
-    const int kt1 = kFused ? min(kt0 + p.fused_kc, n_kt) : 0;
-    const bool has_end = !kFused || kt1 == n_kt;   // the unit holds the sequence's last tile
-    const int qb_b = kFused ? kt1 - kt0 - 1 : chunk;
-    const int head_a = p.head_pairs ? 2 * sel : sel;
-    const int head_b = p.head_pairs ? 2 * sel + 1 : sel;
-    const int n_b = qb_b + 1;                                   // key tiles 0 .. qb_b
-    const int n_a = PL::kTiles == 1 ? 0
-                    : kFused ? (p.fused_L > p.fused_L1 ? n_b : 0)
-                             : (p.head_pairs ? n_b : ((qb_b & 1) ? qb_b : 0));   // 0: no tile A
-    const int j = kFused ? sel : head_b / p.G;                  // Eq. 15
-    const int zk = (((p.slot + blk) * 2 + 0) * p.b + beta) * p.g + j;
-    const int zv = zk + p.b * p.g;
-
+    if ((sbase & 1023u) != 0) {   // the swizzled tiles need it; never seen
+        if (threadIdx.x == 0)
+            atomicOr(p.err, kErrDrain);
+        return;
+    }
     if (threadIdx.x == 0) {
-        // the query tiles' barrier: the producer's tensor-map copy, or every softmax warp's share
-        // of the rows read from host memory
-        mbar_init(bar_q, (kFused && p.q_host != nullptr) ? PL::kSoftWarps : 1);
+        for (int q = 0; q < NQ; ++q) {
+            // the query tiles' barrier: the producer's tensor-map copy, or the last warp's loads
+            // from host memory; freed by the unit's last S and, where the outputs are staged in
+            // the query tiles, by the softmax warps
+            mbar_init(bar_q + 8 * q, 1);
+            mbar_init(bar_q_free + 8 * q, 1 + (PL::kStageInQ ? PL::kSoftWarps : 0));
+        }
         for (int s = 0; s < R; ++s) {
             mbar_init(bar_full + 8 * s, 1);
             mbar_init(bar_empty + 8 * s, 1);
@@ -204,6 +269,7 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
         for (int g = 0; g < 2; ++g) {
             mbar_init(bar_s_ready + 8 * g, 1);
             mbar_init(bar_s_free + 8 * g, 4);
+            mbar_init(bar_p_half + 8 * g, 4);
             mbar_init(bar_p_ready + 8 * g, 4);
             mbar_init(bar_pv_done + 8 * g, 1);
         }
@@ -223,7 +289,7 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    if (kFused && warp < PL::kSoftWarps) {
+    if (kFused && warp < 4 * PL::kTiles) {   // one warpgroup per query tile
         // The tiles' rows past the loaded ones (the TMA box, G x min(L1, L) rows) are never
         // written; zero them so that their (discarded) scores stay finite.
         const int grp = PL::kTiles == 1 ? 1 : warp >> 2, r = threadIdx.x & 127;
@@ -231,12 +297,14 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
         // rows the load writes: the box (tensor map), or tile A's own rows (read from host)
         const int keep = (p.q_host != nullptr && grp == 0) ? (p.fused_L - p.fused_L1) * p.G
                                                            : box_rows;
-        if (r >= keep && warp < 4 * PL::kTiles) {   // one warpgroup per query tile
-            uint8_t *qrow = smem + PL::kQ + slot_of(grp) * PL::kTileBytes;
+        if (r >= keep) {
+            for (int q = 0; q < NQ; ++q) {
+                uint8_t *qrow = smem + PL::kQ + (q * PL::kTiles + slot_of(grp)) * PL::kTileBytes;
 #pragma unroll
-            for (int c = 0; c < 8 * PL::kSub; ++c)
-                *reinterpret_cast<uint4 *>(qrow + (c >> 3) * 16384 + r * 128 +
-                                           (((c & 7) ^ (r & 7)) << 4)) = make_uint4(0, 0, 0, 0);
+                for (int c = 0; c < 8 * PL::kSub; ++c)
+                    *reinterpret_cast<uint4 *>(qrow + (c >> 3) * 16384 + r * 128 +
+                                               (((c & 7) ^ (r & 7)) << 4)) = make_uint4(0, 0, 0, 0);
+            }
             fence_proxy_async_smem();
         }
     }
@@ -256,83 +324,114 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
     grid_dependents_launch();
     if (warp == PL::kProducer) {
         // ------------------------------------ producer ------------------------------------------
+        // Lane 0 waits and announces the bytes; the copies of a tile go out from different lanes
+        // (one thread completes about one bulk copy per 0.4 us, different lanes side by side).
         setmaxnreg_dec<PL::kRegsLow>();
-        if (lane == 0) {
-            bool waited = !early;
-            // mode 2: the cache tiles that hold no new row first, as far as the ring goes
-            int idx_pre = 0;
-            if (early && !q_early) {
-                const int n_pre = 2 * n_b < R ? 2 * n_b : R;
-                for (; idx_pre < n_pre; ++idx_pre) {
-                    if (has_end && (idx_pre >> 1) + kt0 == n_kt - 1)
-                        break;
-                    const uint32_t fb = bar_full + 8 * idx_pre;
-                    mbar_arrive_expect_tx(fb, PL::kTileBytes);
-                    const uint32_t dst = sbase + PL::kRing + idx_pre * PL::kTileBytes;
-                    const int z = (idx_pre & 1) ? zv : zk;
-#pragma unroll
-                    for (int sub = 0; sub < PL::kSub; ++sub)
-                        tma_load_3d(dst + sub * 16384, &tmap_kv, fb, sub * 64,
-                                    ((idx_pre >> 1) + kt0) * 128, z);
-                }
-                grid_dependency_wait();   // the step's inputs are in place
-                waited = true;
-            }
-            if (kFused && p.q_host != nullptr) {
-                // the softmax warps read the queries from host memory
-            } else if (kFused) {
-                // Q [layers][b][h][D] as (channel, head in group, group, sequence, layer): a box
-                // of min(L1, L) layers x G heads = the tile's rows, layer-major (row = layer*G + i),
-                // from the block's first layer (tile B) and its layer L1 (tile A).
-                const int box_rows = (p.fused_L < p.fused_L1 ? p.fused_L : p.fused_L1) * p.G;
-                const int lay0 = blk * p.fused_L;
-                mbar_arrive_expect_tx(bar_q, (n_a > 0 ? 2 : 1) * PL::kSub * box_rows * 128);
-#pragma unroll
-                for (int sub = 0; sub < PL::kSub; ++sub) {
-                    if (n_a > 0)
-                        tma_load_5d(sbase + PL::kQ + sub * 16384, &tmap_q, bar_q, sub * 64, 0, j,
-                                    beta, lay0 + p.fused_L1);
-                    tma_load_5d(sbase + PL::kQ + slot_of(1) * PL::kTileBytes + sub * 16384,
-                                &tmap_q, bar_q, sub * 64, 0, j, beta, lay0);
-                }
-            } else {
-                mbar_arrive_expect_tx(bar_q, (n_a > 0 ? 2 : 1) * PL::kTileBytes);
-#pragma unroll
-                for (int sub = 0; sub < PL::kSub; ++sub) {
-                    if (n_a > 0)
-                        tma_load_4d(sbase + PL::kQ + sub * 16384, &tmap_q, bar_q, sub * 64,
-                                    head_a, (n_a - 1) * 128, beta);
-                    tma_load_4d(sbase + PL::kQ + slot_of(1) * PL::kTileBytes + sub * 16384, &tmap_q,
-                                bar_q, sub * 64, head_b, qb_b * 128, beta);
-                }
-            }
-            const int n_idx = 2 * n_b;   // K_0, V_0, K_1, V_1, ...
-            int idx = idx_pre;
-            for (; idx < n_idx; ++idx) {
-                const int s = idx % R;
+        bool waited = !early;
+        int idx = 0;   // ring tiles sent so far: K_0, V_0, K_1, V_1, ... over all units
+        int uc = 0;    // units whose queries were sent
+        auto agreed = [&](int ok) { return __shfl_sync(0xffffffffu, ok, 0) != 0; };
+        // Ring tile k of unit x (K of key tile k / 2 if k is even, else V).
+        auto send_kv = [&](const Unit &x, int k) {
+            const int s = idx % R;
+            int ok = 1;
+            if (lane == 0) {
                 if (idx >= R && !flags[0] &&
                     !mbar_wait(bar_empty + 8 * s, ((idx / R) & 1) ^ 1)) {
                     flags[0] = 1;
                     atomicOr(p.err, kErrWaitEmpty);
                 }
-                if (flags[0])
-                    break;
-                if (!waited && has_end && (idx >> 1) + kt0 == n_kt - 1) {
-                    grid_dependency_wait();   // the tile that holds the new row
-                    waited = true;
-                }
-                const uint32_t fb = bar_full + 8 * s;
-                mbar_arrive_expect_tx(fb, PL::kTileBytes);
-                const uint32_t dst = sbase + PL::kRing + s * PL::kTileBytes;
-                const int z = (idx & 1) ? zv : zk;
-#pragma unroll
-                for (int sub = 0; sub < PL::kSub; ++sub)
-                    tma_load_3d(dst + sub * 16384, &tmap_kv, fb, sub * 64,
-                                ((idx >> 1) + kt0) * 128, z);
+                ok = !flags[0];
             }
-            // No copy may still be in flight when the CTA exits.
-            if (!mbar_wait(bar_q, 0))
-                atomicOr(p.err, kErrDrain);
+            if (!agreed(ok))
+                return false;
+            if (!waited && x.has_end && (k >> 1) == x.n_b - 1) {
+                grid_dependency_wait();   // the tile that holds the new row
+                waited = true;
+            }
+            const uint32_t fb = bar_full + 8 * s;
+            if (lane == 0)
+                mbar_arrive_expect_tx(fb, PL::kTileBytes);
+            __syncwarp();
+            const int sub = lane - (idx & 7) * 2;   // the lanes take turns
+            if (sub >= 0 && sub < PL::kSub)
+                tma_load_3d(sbase + PL::kRing + s * PL::kTileBytes + sub * 16384, &tmap_kv, fb,
+                            sub * 64, ((k >> 1) + x.kt0) * 128, (k & 1) ? x.zv : x.zk);
+            ++idx;
+            return true;
+        };
+        auto send_q = [&](const Unit &x) {
+            const int qb = uc % NQ;
+            if (kFused && p.q_host != nullptr) {
+                ++uc;   // the last warp reads the queries from host memory
+                return true;
+            }
+            int ok = 1;
+            if (lane == 0) {
+                if (uc >= NQ && !flags[0] &&
+                    !mbar_wait(bar_q_free + 8 * qb, ((uc / NQ) & 1) ^ 1)) {
+                    flags[0] = 1;
+                    atomicOr(p.err, kErrWaitEmpty);
+                }
+                ok = !flags[0];
+            }
+            if (!agreed(ok))
+                return false;
+            const uint32_t qbar = bar_q + 8 * qb;
+            const uint32_t dst = sbase + PL::kQ + qb * PL::kTiles * PL::kTileBytes;
+            const int n_tiles = x.n_a > 0 ? 2 : 1;
+            // fused: Q [layers][b][h][D] as (channel, head in group, group, sequence, layer); a
+            // box of min(L1, L) layers x G heads = the tile's rows, layer-major (row = layer*G + i),
+            // from the block's first layer (tile B) and its layer L1 (tile A)
+            const int box_rows =
+                kFused ? (p.fused_L < p.fused_L1 ? p.fused_L : p.fused_L1) * p.G : 128;
+            if (lane == 0)
+                mbar_arrive_expect_tx(qbar, n_tiles * PL::kSub * box_rows * 128);
+            __syncwarp();
+            const int sub = lane & 1, g = 1 - ((lane >> 1) & 1);
+            if (lane < 2 * n_tiles && sub < PL::kSub) {
+                const uint32_t d = dst + slot_of(g) * PL::kTileBytes + sub * 16384;
+                if (kFused)
+                    tma_load_5d(d, &tmap_q, qbar, sub * 64, 0, x.j, x.beta,
+                                x.blk * p.fused_L + (g ? 0 : p.fused_L1));
+                else
+                    tma_load_4d(d, &tmap_q, qbar, sub * 64, g ? x.head_b : x.head_a,
+                                (g ? x.qb_b : x.n_a - 1) * 128, x.beta);
+            }
+            ++uc;
+            return true;
+        };
+        bool ok = true;
+        for (int n = 0; ok; ++n) {
+            const int i = unit_index(p, n);
+            if (i < 0)
+                break;
+            const Unit x = unit_of<kFused, PL::kTiles>(p, i);
+            const int n_idx = 2 * x.n_b;
+            int k = 0;
+            if (n == 0 && early && !q_early) {
+                // mode 2: the cache tiles that hold no new row first, as far as the ring goes
+                const int n_pre = n_idx < R ? n_idx : R;
+                while (ok && k < n_pre && !(x.has_end && (k >> 1) == x.n_b - 1))
+                    ok = send_kv(x, k++);
+                grid_dependency_wait();   // the step's inputs are in place
+                waited = true;
+            }
+            // a later unit's first key tile can go before its queries' slot is free
+            if (n > 0 && NQ == 1)
+                ok = ok && send_kv(x, k++);
+            ok = ok && send_q(x);
+            while (ok && k < n_idx)
+                ok = send_kv(x, k++);
+            if (kSplit)
+                break;   // one unit per CTA
+        }
+        // No copy may still be in flight when the CTA exits.
+        if (lane == 0) {
+            if (!(kFused && p.q_host != nullptr))
+                for (int k = uc > NQ ? uc - NQ : 0; k < uc; ++k)
+                    if (!mbar_wait(bar_q + 8 * (k % NQ), (k / NQ) & 1))
+                        atomicOr(p.err, kErrDrain);
             for (int k = idx > R ? idx - R : 0; k < idx; ++k)
                 if (!mbar_wait(bar_full + 8 * (k % R), (k / R) & 1))
                     atomicOr(p.err, kErrDrain);
@@ -346,9 +445,9 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
         // issuing both spent about a third of each key tile on barrier checks while the tensor core
         // ran dry.)  With P over S (head_dim 128) one thread issues both, in order.
         setmaxnreg_dec<PL::kRegsLow>();
-        const bool do_s = warp == PL::kMma, do_pv = !PL::kPSep || warp == PL::kMma + 1;
+        const bool do_s = warp == PL::kMma;
         const uint32_t my_fin = bar_fin + (warp == PL::kMma ? 0 : 8);
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t kIdS = umma_idesc(128, 128, 0, 0);
             constexpr uint32_t kIdPV = umma_idesc(128, D, 0, 1);
             constexpr uint32_t kSlot = PL::kTileBytes >> 4;   // one ring slot in descriptor units
@@ -356,7 +455,7 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
             // 64-channel block only moves the start-address field (shared addresses < 256 KB), so
             // each MMA's descriptors are one add away; the tensor core queues little, and any
             // latency between two MMAs of this thread leaves it idle.
-            const uint64_t dq = umma_desc(sbase + PL::kQ, 16, 1024, kLayoutSw128);
+            const uint64_t dq0 = umma_desc(sbase + PL::kQ, 16, 1024, kLayoutSw128);
             const uint64_t dk = umma_desc(sbase + PL::kRing, 16, 1024, kLayoutSw128);
             const uint64_t dv = umma_desc(sbase + PL::kRing, 16384, 1024, kLayoutSw128);
             bool ok = true;
@@ -378,10 +477,10 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
                 }
                 return ok;
             };
-            auto issue_s = [&](int g, int t) {
+            // S of key tile kt (counted over the CTA's units) into buffer sb
+            auto issue_s = [&](int g, int kt, int sb, uint64_t dq) {
                 const uint64_t qa = dq + slot_of(g) * kSlot;
-                const uint64_t kb = dk + ((2 * t) % R) * kSlot;
-                const int sb = kSplit ? (t & 1) : g;   // S buffer and its barrier
+                const uint64_t kb = dk + ((2 * kt) % R) * kSlot;
 #pragma unroll
                 for (int k = 0; k < D / 16; ++k) {
                     const uint32_t off = (k >> 2) * 1024 + (k & 3) * 2;   // 16384 B, 32 B
@@ -390,78 +489,109 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
                 }
                 umma_commit(bar_s_ready + 8 * sb);
             };
-            auto issue_pv = [&](int g, int t, bool last) {
-                const uint64_t vb = dv + ((2 * t + 1) % R) * kSlot;
-                const int sg = slot_of(g);
-                const int ob = kSplit ? (t & 1) : sg;   // P and O buffer (warpgroup t mod 2)
+            // keys [64 h0, 64 h1) of O += P V of key tile kt into buffer pb
+            auto issue_pv = [&](int kt, int pb, bool first, int h0, int h1) {
+                const uint64_t vb = dv + ((2 * kt + 1) % R) * kSlot;
+                const int ob = kSplit ? pb : slot_of(pb);   // P and O columns
                 const uint32_t pc =
-                    tmem + (PL::kPSep ? PL::kColP + 64 * ob : PL::kColS + 128 * sg);
-                const bool first = kSplit ? t < 2 : t == 0;   // the buffer's first product
+                    tmem + (PL::kPSep ? PL::kColP + 64 * ob : PL::kColS + 128 * ob);
 #pragma unroll
                 for (int k = 0; k < 8; ++k)   // 16 keys = 2048 B of V, 8 TMEM columns of P
-                    umma_f16_ts(tmem + PL::kColO + D * ob, pc + 8 * k, vb + k * 128, kIdPV,
-                                (!first || k > 0) ? 1 : 0);
-                // With P over S, the next S's completion already implies this product's.
-                if (PL::kPSep || last)
-                    umma_commit(bar_pv_done + 8 * (kSplit ? (t & 1) : g));
+                    if (k >= 4 * h0 && k < 4 * h1)
+                        umma_f16_ts(tmem + PL::kColO + D * ob, pc + 8 * k, vb + k * 128, kIdPV,
+                                    (!first || k > 0) ? 1 : 0);
             };
-            if (do_s && wait(bar_q, 0) && tile_full(0)) {
-                tmem_fence_after();
-                if (n_a > 0)
-                    issue_s(0, 0);
-                issue_s(1, 0);
-            }
             // Ring slots are released by tile B's softmax warps (they see every MMA that read them
             // complete), not by commits: a commit costs the tensor pipe about as much as a short MMA.
-            for (int t = 0; ok && t < n_b; ++t) {
-                if (PL::kPSep) {
-                    // S issuer: both tiles' next S as soon as each tile's S has been read (early in
-                    // its softmax).  P V issuer: both P V as their P arrive.
+            int kb = 0;             // key tiles of the units before
+            int used[2] = {0, 0};   // products issued so far per S (or P) buffer
+            for (int n = 0; ok; ++n) {
+                const int i = unit_index(p, n);
+                if (i < 0)
+                    break;
+                const Unit x = unit_of<kFused, PL::kTiles>(p, i);
+                const int qb = n % NQ;
+                const uint64_t dq = dq0 + static_cast<uint32_t>(qb * PL::kTiles) * kSlot;
+                if (PL::kPSep && do_s) {
+                    // S(t) once its columns are free, i.e. the previous scores of the buffer have
+                    // been read (right after they arrived).
+                    if (!wait(bar_q + 8 * qb, n / NQ))
+                        break;
+                    for (int t = 0; ok && t < x.n_b; ++t) {
 #pragma unroll
-                    for (int g = 0; g < 2; ++g) {
-                        const int ng = g ? n_b : n_a;
-                        if (!do_s || !ok || t + 1 >= ng)
-                            continue;
-                        // S(t + 1) once its columns are free: tile t's S read (one buffer), or
-                        // tile t - 1's (two buffers: S(t + 1) then runs during tile t's softmax)
-                        if (kSplit ? (t >= 1 && !wait(bar_s_free + 8 * ((t + 1) & 1), (t - 1) >> 1))
-                                   : !wait(bar_s_free + 8 * g, t))
-                            break;
-                        if (!tile_full(2 * t + 2))
-                            break;
-                        tmem_fence_after();
-                        issue_s(g, t + 1);
+                        for (int g = 2 - PL::kTiles; g < 2; ++g) {
+                            if (!ok || t >= (g ? x.n_b : x.n_a))
+                                continue;
+                            const int sb = kSplit ? (t & 1) : g;
+                            if (used[sb] > 0 && !wait(bar_s_free + 8 * sb, used[sb] - 1))
+                                break;
+                            if (!tile_full(2 * (kb + t)))
+                                break;
+                            tmem_fence_after();
+                            issue_s(g, kb + t, sb, dq);
+                            ++used[sb];
+                        }
                     }
+                    umma_commit(bar_q_free + 8 * qb);
+                } else if (PL::kPSep) {
+                    for (int t = 0; ok && t < x.n_b; ++t) {
 #pragma unroll
-                    for (int g = 0; g < 2; ++g) {
-                        const int ng = g ? n_b : n_a;
-                        if (!do_pv || !ok || t >= ng)
-                            continue;
-                        if (!tile_full(2 * t + 1) ||
-                            !wait(bar_p_ready + 8 * (kSplit ? (t & 1) : g), kSplit ? (t >> 1) : t))
-                            break;
-                        tmem_fence_after();
-                        issue_pv(g, t, t + 1 >= ng);
+                        for (int g = 2 - PL::kTiles; g < 2; ++g) {
+                            if (!ok || t >= (g ? x.n_b : x.n_a))
+                                continue;
+                            const int pb = kSplit ? (t & 1) : g;
+                            if (!tile_full(2 * (kb + t) + 1) ||
+                                !wait(bar_p_ready + 8 * pb, used[pb]))
+                                break;
+                            tmem_fence_after();
+                            issue_pv(kb + t, pb, kSplit ? t < 2 : t == 0, 0, 2);
+                            umma_commit(bar_pv_done + 8 * pb);
+                            ++used[pb];
+                        }
                     }
-                    continue;
+                } else {
+                    // P over S: the first S of the unit (the P V products that read these columns
+                    // were issued before), then per key tile and query tile the P V product in two
+                    // halves as the halves of P arrive, and the next S right behind it.
+                    if (!wait(bar_q + 8 * qb, n / NQ) || !tile_full(2 * kb))
+                        break;
+                    tmem_fence_after();
+                    if (x.n_a > 0)
+                        issue_s(0, kb, 0, dq);
+                    issue_s(1, kb, 1, dq);
+                    if (x.n_b == 1)
+                        umma_commit(bar_q_free + 8 * qb);
+                    for (int t = 0; ok && t < x.n_b; ++t) {
+#pragma unroll
+                        for (int g = 0; g < 2; ++g) {
+                            const int ng = g ? x.n_b : x.n_a;
+                            if (!ok || t >= ng)
+                                continue;
+                            const bool next = t + 1 < ng;
+                            if (!tile_full(2 * (kb + t) + 1) ||
+                                (next && !tile_full(2 * (kb + t) + 2)) ||
+                                !wait(bar_p_half + 8 * g, used[g]))
+                                break;
+                            tmem_fence_after();
+                            issue_pv(kb + t, g, t == 0, 0, 1);
+                            if (!wait(bar_p_ready + 8 * g, used[g]))
+                                break;
+                            tmem_fence_after();
+                            issue_pv(kb + t, g, t == 0, 1, 2);
+                            ++used[g];
+                            // the next S's completion implies this product's
+                            if (!next)
+                                umma_commit(bar_pv_done + 8 * g);
+                            else
+                                issue_s(g, kb + t + 1, g, dq);
+                            if (g == 1 && t + 2 == x.n_b)
+                                umma_commit(bar_q_free + 8 * qb);   // that was the unit's last S
+                        }
+                    }
                 }
-#pragma unroll
-                for (int g = 0; g < 2; ++g) {
-                    const int ng = g ? n_b : n_a;
-                    if (!ok || t >= ng)
-                        continue;
-                    const bool next = t + 1 < ng;
-                    {
-                        // Everything first, then P V and the next S back to back.
-                        if (!tile_full(2 * t + 1) || (next && !tile_full(2 * t + 2)) ||
-                            !wait(bar_p_ready + 8 * g, t))
-                            break;
-                        tmem_fence_after();
-                        issue_pv(g, t, !next);
-                        if (next)
-                            issue_s(g, t + 1);
-                    }
-                }
+                kb += x.n_b;
+                if (kSplit)
+                    break;   // one unit per CTA
             }
             if (!ok) {
                 flags[0] = 1;
@@ -478,9 +608,6 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
         const int grp = PL::kTiles == 1 ? 1 : warp >> 2;   // 0: query tile A, 1: query tile B
         const int r = threadIdx.x & 127;            // query row of the tile = TMEM lane
         const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16;
-        const int n_g = grp ? n_b : n_a;
-        const int head = grp ? head_b : head_a;
-        const int q0 = (kt0 + n_g - 1) * 128;       // first position of the unit's last tile
         const int sg = slot_of(grp);
         // the warpgroup's buffer: the tile's own, or (split keys) this warpgroup's tiles t = wg,
         // wg + 2, ... with S, P and O buffer wg
@@ -492,122 +619,101 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
             tmem + lane_off +
             (PL::kPSep ? PL::kColP + 64 * (kSplit ? wg : sg) : PL::kColS + 128 * sg);
         const uint32_t s_ready = bar_s_ready + 8 * bsel, s_free = bar_s_free + 8 * bsel;
-        const uint32_t p_ready = bar_p_ready + 8 * bsel, pv_done = bar_pv_done + 8 * bsel;
+        const uint32_t p_half = bar_p_half + 8 * bsel, p_ready = bar_p_ready + 8 * bsel;
+        const uint32_t pv_done = bar_pv_done + 8 * bsel;
         constexpr int kStep = kSplit ? 2 : 1;   // tiles between this warpgroup's
-        // The prompt's last block holds keys past its end; the first tile to reach it zeroes them.
-        const bool zero_v = n_g > 0 && (kFused ? has_end : n_g == (S + 127) / 128) &&
-                            (grp == 0 || n_a != n_b);
+        // Tile B's first warp frees ring slots whose readers have all completed: K_t once S_B(t)
+        // is done (S_A(t) was issued before it by the same thread); V_{t-1} once S_B(t) (P over
+        // S: issued after P V_{t-1}) or P_B V_{t-1} (own P) is done.
+        const bool releaser = grp == 1 && (warp & 3) == 0 && lane == 0;
         const float scale = p.scale_log2;
         const float NEG_INF = -__int_as_float(0x7f800000);
         auto wait = [&](uint32_t bar, int parity) {
-            if (!flags[0] && !mbar_wait(bar, static_cast<uint32_t>(parity) & 1u)) {
+            const uint32_t par = static_cast<uint32_t>(parity) & 1u;
+            if (!mbar_test_wait(bar, par) && !flags[0] && !mbar_wait(bar, par)) {
                 flags[0] = 1;
                 atomicOr(p.err, kErrWaitFull);
             }
         };
-        if (kFused && p.q_host != nullptr) {
-            // The unit's query rows from page-locked host memory through its device-mapped
-            // address (16 bytes a load, four in flight per thread), written into the query tiles
-            // the way the tensor map would have (128-byte swizzle); rows past them stay zero.
-            const int nth = 32 * PL::kSoftWarps;
-            const int L1r = p.fused_L < p.fused_L1 ? p.fused_L : p.fused_L1;
-            const int rows_b = L1r * p.G;
-            const int rows_a = n_a > 0 ? (p.fused_L - p.fused_L1) * p.G : 0;
-            constexpr int kC = D / 8;   // 16-byte chunks of a row
-            const int total = (rows_b + rows_a) * kC;
-            for (int k0 = threadIdx.x; k0 < total; k0 += 4 * nth) {
-                uint4 v[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int k = k0 + u * nth;
-                    if (k < total) {
-                        const int rr = k / kC, c = k - rr * kC;
-                        const bool in_b = rr < rows_b;
-                        const int rw = in_b ? rr : rr - rows_b;
-                        const int lay = blk * p.fused_L + (in_b ? 0 : p.fused_L1) + rw / p.G;
-                        v[u] = *reinterpret_cast<const uint4 *>(
-                            p.q_host + ((static_cast<size_t>(lay) * p.b + beta) * p.h + j * p.G +
-                                        rw % p.G) * D + c * 8);
-                    }
+        int kb = 0;     // key tiles of the units before
+        int used = 0;   // score tiles this warpgroup has taken
+        int outs = 0;   // units it has finished (P over S: phases of pv_done)
+        for (int n = 0;; ++n) {
+            const int i = unit_index(p, n);
+            if (i < 0 || (!kSplit && __any_sync(0xffffffffu, flags[0])))
+                break;
+            const Unit x = unit_of<kFused, PL::kTiles>(p, i);
+            const int qb = n % NQ;
+            const int n_g = grp ? x.n_b : x.n_a;
+            const int q0 = (x.kt0 + n_g - 1) * 128;       // first position of the unit's last tile
+            // The prompt's last block holds keys past its end; the first tile to reach it zeroes
+            // them.
+            const bool zero_v = n_g > 0 && (kFused ? x.has_end : n_g == (x.S + 127) / 128) &&
+                                (grp == 0 || x.n_a != x.n_b);
+            uint8_t *q_slot = smem + PL::kQ + (qb * PL::kTiles + sg) * PL::kTileBytes;
+            float m_run = NEG_INF, l_run = 0.f;
+            for (int t = wg; t < n_g; t += kStep, ++used) {
+                wait(s_ready, used);
+                if (releaser) {
+                    mbar_arrive(bar_empty + 8 * ((2 * (kb + t)) % R));   // K_t
+                    if (!PL::kPSep && t > 0)
+                        mbar_arrive(bar_empty + 8 * ((2 * (kb + t) - 1) % R));   // V_{t-1}
                 }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int k = k0 + u * nth;
-                    if (k < total) {
-                        const int rr = k / kC, c = k - rr * kC;
-                        const bool in_b = rr < rows_b;
-                        const int rw = in_b ? rr : rr - rows_b;
-                        *reinterpret_cast<uint4 *>(smem + PL::kQ +
-                                                   slot_of(in_b ? 1 : 0) * PL::kTileBytes +
-                                                   (c >> 3) * 16384 + rw * 128 +
-                                                   (((c & 7) ^ (rw & 7)) << 4)) = v[u];
-                    }
-                }
-            }
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0)
-                mbar_arrive(bar_q);
-        }
-        float m_run = NEG_INF, l_run = 0.f;
-        for (int t = wg; t < n_g; t += kStep) {
-            const int u = kSplit ? t >> 1 : t;   // this warpgroup's use of its buffers
-            wait(s_ready, u);
-            // Tile B's first warp frees ring slots whose readers have all completed: K_t once S_B(t)
-            // is done (S_A(t) was issued before it by the same thread); V_{t-1} once S_B(t) (P over
-            // S: issued after P V_{t-1}) or P_B V_{t-1} (own P) is done.
-            const bool releaser = grp == 1 && (warp & 3) == 0 && lane == 0;
-            if (releaser && (t == 0 || PL::kPSep))   // K_t
-                mbar_arrive(bar_empty + 8 * ((2 * t) % R));
-            if (releaser && t > 0 && !PL::kPSep) {
-                mbar_arrive(bar_empty + 8 * ((2 * t - 1) % R));
-                mbar_arrive(bar_empty + 8 * ((2 * t) % R));
-            }
-            const bool diag = t == n_g - 1 && has_end;
-            // This tile's scores, with the causal (or sequence-end) mask of the last tile.
-            float sv[4][32];
-            auto load_scores = [&]() {
+                const bool diag = t == n_g - 1 && x.has_end;
+                // This tile's scores and the row's maximum, which the load returns with them.
+                float sv[4][32], mx[4];
+                uint32_t w[2][32];
                 tmem_fence_after();
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
-                    tmem_ld32_nowait(col_s + c * 32, sv[c]);
+                    tmem_ld32_max_nowait(col_s + c * 32, sv[c], mx[c]);
                 tmem_wait_ld();
+                asm volatile("" : "+f"(mx[0]), "+f"(mx[1]), "+f"(mx[2]), "+f"(mx[3]));
+                if (PL::kPSep) {
+                    // S's columns may take the next scores.
+                    tmem_fence_before();
+                    __syncwarp();
+                    if (lane == 0)
+                        mbar_arrive(s_free);
+                }
+                if (diag && zero_v && q0 + r >= x.S) {
+                    // Key q0 + r lies past the prompt: its V row may hold anything; zero it.
+                    const int idx = 2 * (kb + t) + 1;
+                    wait(bar_full + 8 * (idx % R), idx / R);
+                    uint8_t *vrow = smem + PL::kRing + (idx % R) * PL::kTileBytes;
+#pragma unroll
+                    for (int c = 0; c < 8 * PL::kSub; ++c)
+                        *reinterpret_cast<uint4 *>(vrow + (c >> 3) * 16384 + r * 128 +
+                                                   (((c & 7) ^ (r & 7)) << 4)) = make_uint4(0, 0, 0, 0);
+                    fence_proxy_async_smem();
+                }
                 if (diag) {
                     // Keys [0, lim) of the tile are visible: up to the sequence's end (fused
-                    // decode) or to the query's own position (causal mask).
-                    const int lim = kFused ? S - q0 : r + 1;
+                    // decode) or to the query's own position (causal mask); the maximum is
+                    // taken again over those.
+                    const int lim = kFused ? x.S - q0 : r + 1;
 #pragma unroll
-                    for (int c = 0; c < 4; ++c)
+                    for (int c = 0; c < 4; ++c) {
+                        mx[c] = NEG_INF;
 #pragma unroll
-                        for (int k = 0; k < 32; ++k)
+                        for (int k = 0; k < 32; ++k) {
                             if (c * 32 + k >= lim)
                                 sv[c][k] = NEG_INF;
-                }
-            };
-            // Raises the reference maximum to the tile's when a score exceeds it by more than 2^8
-            // (the thread then rescales its O row in TMEM).
-            auto raise_to_tile_max = [&]() {
-                float mx[4];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    float a = max3f(sv[c][0], sv[c][1], sv[c][2]);
-                    float b = max3f(sv[c][3], sv[c][4], sv[c][5]);
-#pragma unroll
-                    for (int k = 6; k < 30; k += 4) {
-                        a = max3f(a, sv[c][k], sv[c][k + 1]);
-                        b = max3f(b, sv[c][k + 2], sv[c][k + 3]);
+                            mx[c] = fmaxf(mx[c], sv[c][k]);
+                        }
                     }
-                    mx[c] = max3f(a, b, fmaxf(sv[c][30], sv[c][31]));
                 }
+                // The reference maximum is raised to the tile's when a score exceeds it by more
+                // than 2^8 (the thread then rescales its O row in TMEM).
                 const float m_tile = max3f(mx[0], mx[1], fmaxf(mx[2], mx[3])) * scale;
                 const bool raise = (m_run == NEG_INF) || (m_tile > m_run + 8.f);
                 if (__any_sync(0xffffffffu, raise)) {
                     const float m_new = raise ? fmaxf(m_run, m_tile) : m_run;
                     const float alpha = fast_exp2(m_run - m_new);   // 0 while nothing is summed
-                    if (u > 0) {
+                    if (t > wg) {
                         // Rescale this row of O once the previous tile's product has landed.
                         if (PL::kPSep)
-                            wait(pv_done, u - 1);
+                            wait(pv_done, used - 1);
                         tmem_fence_after();
 #pragma unroll
                         for (int c = 0; c < D / 32; ++c) {
@@ -623,154 +729,134 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
                     l_run *= alpha;
                     m_run = m_new;
                 }
-            };
-            const float2 sc2 = make_float2(scale, scale);
-            float2 acc[4];
-            uint32_t w[2][32];
-            // p = 2^(s log2(e)/sqrt(d) - m) as bf16 pairs, and the row's sum in fp32.
-            auto weights = [&]() {
+                // p = 2^(s log2(e)/sqrt(d) - m) as bf16 pairs, and the row's sum in fp32.
+                const float2 sc2 = make_float2(scale, scale);
                 const float m_use = m_run == NEG_INF ? 0.f : m_run;   // all masked so far: p = 0
                 const float2 nm2 = make_float2(-m_use, -m_use);
+                float2 acc[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                     acc[q] = make_float2(0.f, 0.f);
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        const int c = half * 64 + 2 * i;   // keys c, c + 1
-                        const float2 x = __ffma2_rn(
+                    for (int e = 0; e < 32; ++e) {
+                        const int c = half * 64 + 2 * e;   // keys c, c + 1
+                        const float2 y = __ffma2_rn(
                             make_float2(sv[c >> 5][c & 31], sv[c >> 5][(c & 31) + 1]), sc2, nm2);
-                        const float2 pr = make_float2(fast_exp2(x.x), fast_exp2(x.y));
-                        acc[i & 3] = __fadd2_rn(acc[i & 3], pr);
-                        w[half][i] = pack_bf16x2(pr.x, pr.y);
+                        const float2 pr = make_float2(fast_exp2(y.x), fast_exp2(y.y));
+                        acc[e & 3] = __fadd2_rn(acc[e & 3], pr);
+                        w[half][e] = pack_bf16x2(pr.x, pr.y);
+                    }
+                    if (!PL::kPSep) {
+                        tmem_st32_nowait(col_p + 32 * half, w[half]);
+                        if (half == 0) {
+                            // the first 64 keys' product may start
+                            tmem_wait_st();
+                            tmem_fence_before();
+                            __syncwarp();
+                            if (lane == 0)
+                                mbar_arrive(p_half);
+                        }
                     }
                 }
-            };
-            load_scores();
-            if (__any_sync(0xffffffffu, m_run == NEG_INF)) {
-                raise_to_tile_max();
-                weights();
-            } else {
-                // Most tiles: the weights against the current reference, without the tile's
-                // maximum.  A row whose weights add up to more than 2^8 (or overflow) may hold one
-                // above 2^8: the scores are read again (S is still in TMEM: its columns are freed
-                // only below) and the reference raised as above.
-                weights();
                 const float2 s01 = __fadd2_rn(acc[0], acc[1]), s23 = __fadd2_rn(acc[2], acc[3]);
                 const float2 s4 = __fadd2_rn(s01, s23);
-                if (__any_sync(0xffffffffu, !(s4.x + s4.y <= 256.f))) {
-                    load_scores();
-                    raise_to_tile_max();
-                    weights();
+                // The P buffer of the previous tile must have been read by its P V; the weights
+                // above were computed while that product ran.
+                if (PL::kPSep && t > wg) {
+                    wait(pv_done, used - 1);
+                    if (releaser)   // V of this warpgroup's previous tile
+                        mbar_arrive(bar_empty + 8 * ((2 * (kb + t - kStep) + 1) % R));
                 }
-            }
-            if (PL::kPSep) {
-                // S's columns may now take the next tile's scores.
+                if (PL::kPSep) {
+                    tmem_fence_after();
+                    tmem_st32_nowait(col_p, w[0]);
+                    tmem_st32_nowait(col_p + 32, w[1]);
+                }
+                l_run += s4.x + s4.y;
+                tmem_wait_st();
                 tmem_fence_before();
                 __syncwarp();
                 if (lane == 0)
-                    mbar_arrive(s_free);
+                    mbar_arrive(p_ready);
             }
-            // The P buffer of the previous tile must have been read by its P V; the weights above
-            // were computed while that product ran.
-            if (PL::kPSep && u > 0) {
-                wait(pv_done, u - 1);
-                if (releaser)   // V of this warpgroup's previous tile
-                    mbar_arrive(bar_empty + 8 * ((2 * (t - kStep) + 1) % R));
+            // ---------------- the tile's output: o = O / l ----------------
+            if (early)
+                grid_dependency_wait();   // earlier kernels of the stream have finished with out
+            // The unit's fields that only the output needs, read again: they need no registers
+            // during the loop.
+            int i_out = i;
+            asm volatile("" : "+r"(i_out));
+            const Unit y = unit_of<kFused, PL::kTiles>(p, i_out);
+            // The unit's last product, and with it the last reader of its last V.
+            const int n_mine = kSplit ? (n_g - wg + 1) / 2 : n_g;   // this warpgroup's tiles
+            if (n_mine > 0) {
+                wait(pv_done, PL::kPSep ? used - 1 : outs);
+                ++outs;
+                if (releaser)
+                    mbar_arrive(bar_empty +
+                                8 * ((2 * (kb + (kSplit ? wg + 2 * (n_mine - 1) : n_g - 1)) + 1) % R));
             }
-            tmem_fence_after();
-            tmem_st32_nowait(col_p, w[0]);
-            tmem_st32_nowait(col_p + 32, w[1]);
-            const float2 s01 = __fadd2_rn(acc[0], acc[1]), s23 = __fadd2_rn(acc[2], acc[3]);
-            const float2 s4 = __fadd2_rn(s01, s23);
-            l_run += s4.x + s4.y;
-            tmem_wait_st();
-            if (diag && zero_v && q0 + r >= S) {
-                // Key q0 + r lies past the prompt: its V row may hold anything; zero it.
-                const int idx = 2 * t + 1;
-                wait(bar_full + 8 * (idx % R), idx / R);
-                uint8_t *vrow = smem + PL::kRing + (idx % R) * PL::kTileBytes;
-#pragma unroll
-                for (int c = 0; c < 8 * PL::kSub; ++c)
-                    *reinterpret_cast<uint4 *>(vrow + (c >> 3) * 16384 + r * 128 +
-                                               (((c & 7) ^ (r & 7)) << 4)) = make_uint4(0, 0, 0, 0);
-                fence_proxy_async_smem();
-            }
-            tmem_fence_before();
-            __syncwarp();
-            if (lane == 0)
-                mbar_arrive(p_ready);
-        }
-        // ---------------- the tile's output: o = O / l ----------------
-        if (early)
-            grid_dependency_wait();   // earlier kernels of the stream have finished with out
-        // Split keys: the second warpgroup hands its running maximum and sum to the first, which
-        // merges the two O buffers row by row (O = O_0 2^(m_0 - M) + O_1 2^(m_1 - M), likewise l).
-        const int n_mine = kSplit ? (n_g - wg + 1) / 2 : n_g;   // this warpgroup's tiles
-        float a0 = 1.f, a1 = 0.f;
-        if (kSplit) {
-            if (n_mine > 0)
-                wait(pv_done, n_mine - 1);
-            float2 *ml = reinterpret_cast<float2 *>(smem + PL::kML);
-            if (wg == 1)
-                ml[r] = make_float2(m_run, l_run);
-            asm volatile("bar.sync 1, %0;" ::"n"(8 * 32) : "memory");
-            if (wg == 1)
-                m_run = NEG_INF;   // done: nothing to store
-            else {
-                const float2 o1 = ml[r];
-                if (o1.y > 0.f) {
-                    const float mx = fmaxf(m_run, o1.x);
-                    a0 = fast_exp2(m_run - mx);
-                    a1 = fast_exp2(o1.x - mx);
-                    l_run = l_run * a0 + o1.y * a1;
-                    m_run = mx;
+            // Split keys: the second warpgroup hands its running maximum and sum to the first, which
+            // merges the two O buffers row by row (O = O_0 2^(m_0 - M) + O_1 2^(m_1 - M), likewise l).
+            float a0 = 1.f, a1 = 0.f;
+            if (kSplit) {
+                float2 *ml = reinterpret_cast<float2 *>(smem + PL::kML);
+                if (wg == 1)
+                    ml[r] = make_float2(m_run, l_run);
+                asm volatile("bar.sync 1, %0;" ::"n"(8 * 32) : "memory");
+                if (wg == 0) {
+                    const float2 o1 = ml[r];
+                    if (o1.y > 0.f) {
+                        const float mxx = fmaxf(m_run, o1.x);
+                        a0 = fast_exp2(m_run - mxx);
+                        a1 = fast_exp2(o1.x - mxx);
+                        l_run = l_run * a0 + o1.y * a1;
+                        m_run = mxx;
+                    }
                 }
             }
-        }
-        // O of this row, 32 columns at c: this warpgroup's buffer, merged with the second's
-        auto load_o = [&](int c, float (&ov)[32]) {
-            tmem_ld32_nowait(col_o + c * 32, ov);
-            if (kSplit && a1 > 0.f) {
-                float o1[32];
-                tmem_ld32_nowait(col_o + D + c * 32, o1);
-                tmem_wait_ld();
+            // O of this row, 32 columns at c: this warpgroup's buffer, merged with the second's
+            auto load_o = [&](int c, float (&ov)[32]) {
+                tmem_ld32_nowait(col_o + c * 32, ov);
+                if (kSplit && a1 > 0.f) {
+                    float o1[32];
+                    tmem_ld32_nowait(col_o + D + c * 32, o1);
+                    tmem_wait_ld();
 #pragma unroll
-                for (int k = 0; k < 32; ++k)
-                    ov[k] = ov[k] * a0 + o1[k] * a1;
-            } else {
-                tmem_wait_ld();
-            }
-        };
-        if (n_g > 0 && wg == 0) {
-            if (!kSplit)
-                wait(pv_done, PL::kPSep ? n_g - 1 : 0);   // with P over S only the last P V commits
-            tmem_fence_after();
-            const float inv = fast_rcp(l_run);
-            bool valid;
-            __nv_bfloat16 *orow;
-            if (kFused) {
-                // Row r: layer (grp ? 0 : L1) + r / G of the block, head j*G + r % G; out
-                // [layers][b][h][D], the block's first layer blk * L.
-                const int L1 = p.fused_L < p.fused_L1 ? p.fused_L : p.fused_L1;
-                valid = r < (grp ? L1 : p.fused_L - p.fused_L1) * p.G;
-                const int layer = (grp ? 0 : p.fused_L1) + r / p.G;
-                orow = p.out + ((static_cast<size_t>(blk * p.fused_L + layer) * p.b + beta) * p.h +
-                                j * p.G + r % p.G) * D;
-                if (p.fused_cmax > 1) {
+                    for (int k = 0; k < 32; ++k)
+                        ov[k] = ov[k] * a0 + o1[k] * a1;
+                } else {
+                    tmem_wait_ld();
+                }
+            };
+            if (n_g > 0 && wg == 0) {
+                tmem_fence_after();
+                const float inv = fast_rcp(l_run);
+                const int stop = flags[0];
+                // Row r of the tile.  Prefill: position q0 + r of the head.  Fused: layer
+                // (grp ? 0 : L1) + r / G of the block, head j*G + r % G; out [layers][b][h][D].
+                const int lay0 = y.blk * p.fused_L + (grp ? 0 : p.fused_L1);
+                const int n_rows =
+                    !kFused ? min(128, y.S - q0)
+                            : (grp ? (p.fused_L < p.fused_L1 ? p.fused_L : p.fused_L1)
+                                   : p.fused_L - p.fused_L1) * p.G;
+                if (kFused && p.fused_cmax > 1) {
                     // One chunk of the context: o = O / l and lse = m + log2(l) for the merge.
-                    const size_t row = (((static_cast<size_t>(blk) * p.b + beta) * p.g + j) *
-                                            p.fused_cmax + chunk) * (p.fused_L * p.G) +
+                    const bool valid = r < n_rows && !stop;
+                    const int layer = (grp ? 0 : p.fused_L1) + r / p.G;
+                    const size_t row = (((static_cast<size_t>(y.blk) * p.b + y.beta) * p.g + y.j) *
+                                            p.fused_cmax + y.chunk) * (p.fused_L * p.G) +
                                        layer * p.G + r % p.G;
                     float *prow = p.part + row * D;
-                    if (valid && !flags[0])
+                    if (valid)
                         p.part_lse[row] = m_run + log2f(l_run);
 #pragma unroll
                     for (int c = 0; c < D / 32; ++c) {
                         float ov[32];
                         load_o(c, ov);
-                        if (valid && !flags[0]) {
+                        if (valid) {
 #pragma unroll
                             for (int k = 0; k < 32; k += 4)
                                 *reinterpret_cast<float4 *>(prow + c * 32 + k) =
@@ -778,70 +864,137 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
                                                 ov[k + 3] * inv);
                         }
                     }
-                    valid = false;   // nothing more to store for this row
                 } else {
-                    // The warp's 32 rows go through this tile's query slot (its last S has
-                    // completed), 16-byte chunks swizzled by row, and out 16 bytes a lane: the G
-                    // heads of a layer are contiguous rows of out, so the stores coalesce, which
-                    // matters most when out is page-locked host memory.
-                    uint8_t *stage = smem + PL::kQ + sg * PL::kTileBytes;
-                    constexpr int kChunks = D * 2 / 16;   // 16-byte chunks of a row
-#pragma unroll
-                    for (int c = 0; c < D / 32; ++c) {
-                        float ov[32];
-                        load_o(c, ov);
-#pragma unroll
-                        for (int k = 0; k < 32; k += 8)
-                            *reinterpret_cast<uint4 *>(stage + r * (D * 2) +
-                                                       ((((c * 32 + k) >> 3) ^ (r & 7)) << 4)) =
-                                make_uint4(pack_bf16x2(ov[k] * inv, ov[k + 1] * inv),
-                                           pack_bf16x2(ov[k + 2] * inv, ov[k + 3] * inv),
-                                           pack_bf16x2(ov[k + 4] * inv, ov[k + 5] * inv),
-                                           pack_bf16x2(ov[k + 6] * inv, ov[k + 7] * inv));
-                    }
-                    __syncwarp();
+                    // The warp's 32 rows go through shared memory, 64 channels at a time (16-byte
+                    // chunks swizzled by row), and out 16 bytes a lane, 8 lanes a row: coalesced
+                    // stores, which matters most when out is page-locked host memory.  At head_dim
+                    // 64 the stage is the unit's own query tile (its last S has completed).
                     const int rw0 = (warp & 3) * 32;
-                    const int n_rows = (grp ? L1 : p.fused_L - p.fused_L1) * p.G;
+                    uint8_t *stage = PL::kStageInQ ? q_slot + rw0 * 128
+                                                   : smem + PL::kStage + warp * 4096;
 #pragma unroll
-                    for (int it = 0; it < kChunks; ++it) {
-                        const int cidx = it * 32 + lane;
-                        const int rr = rw0 + cidx / kChunks, ch = cidx % kChunks;
-                        if (rr < n_rows && !flags[0]) {
-                            const int lay = (grp ? 0 : p.fused_L1) + rr / p.G;
-                            __nv_bfloat16 *o =
-                                p.out + ((static_cast<size_t>(blk * p.fused_L + lay) * p.b + beta) *
-                                             p.h + j * p.G + rr % p.G) * D;
-                            *reinterpret_cast<uint4 *>(o + ch * 8) = *reinterpret_cast<const uint4 *>(
-                                stage + rr * (D * 2) + ((ch ^ (rr & 7)) << 4));
+                    for (int cb = 0; cb < PL::kSub; ++cb) {
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            float ov[32];
+                            load_o(2 * cb + c, ov);
+                            if (r < n_rows) {
+#pragma unroll
+                                for (int k = 0; k < 32; k += 8)
+                                    *reinterpret_cast<uint4 *>(
+                                        stage + lane * 128 + ((((c * 32 + k) >> 3) ^ (lane & 7)) << 4)) =
+                                        make_uint4(pack_bf16x2(ov[k] * inv, ov[k + 1] * inv),
+                                                   pack_bf16x2(ov[k + 2] * inv, ov[k + 3] * inv),
+                                                   pack_bf16x2(ov[k + 4] * inv, ov[k + 5] * inv),
+                                                   pack_bf16x2(ov[k + 6] * inv, ov[k + 7] * inv));
+                            }
+                        }
+                        __syncwarp();
+                        const int ch = lane & 7;
+                        uint4 line[8];   // every load first: shared memory is busy with the MMAs
+#pragma unroll
+                        for (int it = 0; it < 8; ++it) {
+                            const int rl = it * 4 + (lane >> 3);
+                            line[it] = *reinterpret_cast<const uint4 *>(stage + rl * 128 +
+                                                                        ((ch ^ (rl & 7)) << 4));
+                        }
+                        __syncwarp();
+#pragma unroll
+                        for (int it = 0; it < 8; ++it) {
+                            const int rr = rw0 + it * 4 + (lane >> 3);
+                            if (rr < n_rows && !stop) {
+                                size_t row;   // of out, in units of D
+                                if (kFused)
+                                    row = (static_cast<size_t>(lay0 + rr / p.G) * p.b + y.beta) * p.h +
+                                          y.j * p.G + rr % p.G;
+                                else
+                                    row = (static_cast<size_t>(y.beta) * p.s_max + (q0 + rr)) * p.h +
+                                          (grp ? y.head_b : y.head_a);
+                                *reinterpret_cast<uint4 *>(p.out + row * D + cb * 64 + ch * 8) =
+                                    line[it];
+                            }
                         }
                     }
-                    valid = false;
                 }
-            } else {
-                valid = q0 + r < S;
-                orow = p.out + ((static_cast<size_t>(beta) * p.s_max + (q0 + r)) * p.h + head) * D;
+                tmem_fence_before();
             }
-#pragma unroll
-            for (int c = 0; c < (kFused ? 0 : D / 32); ++c) {   // the prefill's rows
-                float ov[32];
-                tmem_ld32_nowait(col_o + c * 32, ov);
-                tmem_wait_ld();
-                if (valid && !flags[0]) {
-#pragma unroll
-                    for (int k = 0; k < 32; k += 8)
-                        *reinterpret_cast<uint4 *>(orow + c * 32 + k) = make_uint4(
-                            pack_bf16x2(ov[k] * inv, ov[k + 1] * inv),
-                            pack_bf16x2(ov[k + 2] * inv, ov[k + 3] * inv),
-                            pack_bf16x2(ov[k + 4] * inv, ov[k + 5] * inv),
-                            pack_bf16x2(ov[k + 6] * inv, ov[k + 7] * inv));
-                }
+            if (PL::kStageInQ) {
+                // the next queries may be written over the stage
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0)
+                    mbar_arrive(bar_q_free + 8 * qb);
             }
-            tmem_fence_before();
+            kb += x.n_b;
+            if (kSplit)
+                break;   // one unit per CTA
         }
     } else {
-        setmaxnreg_dec<PL::kRegsLow>();   // warp 11 (and 10 with head_dim 128): no role
+        setmaxnreg_dec<PL::kRegsLow>();
+        if (kFused && p.q_host != nullptr && warp == PL::kSoftWarps + 3) {
+            // The last warp: each unit's query rows from page-locked host memory through its
+            // device-mapped address (16 bytes a load, several in flight per lane), written into the
+            // query tiles the way the tensor map would have (128-byte swizzle); rows past them stay
+            // zero.
+            constexpr int kFly = PL::kRegsLow >= 72 ? 10 : 4;
+            constexpr int kC = D / 8;   // 16-byte chunks of a row
+            const int rows_b = (p.fused_L < p.fused_L1 ? p.fused_L : p.fused_L1) * p.G;
+            for (int n = 0;; ++n) {
+                const int i = unit_index(p, n);
+                if (i < 0)
+                    break;
+                const Unit x = unit_of<kFused, PL::kTiles>(p, i);
+                const int qb = n % NQ;
+                int ok = 1;
+                if (lane == 0 && n >= NQ && !flags[0] &&
+                    !mbar_wait(bar_q_free + 8 * qb, ((n / NQ) & 1) ^ 1)) {
+                    flags[0] = 1;
+                    atomicOr(p.err, kErrWaitEmpty);
+                }
+                if (lane == 0)
+                    ok = !flags[0];
+                if (!__shfl_sync(0xffffffffu, ok, 0))
+                    break;
+                uint8_t *dst = smem + PL::kQ + qb * PL::kTiles * PL::kTileBytes;
+                const int total = (rows_b + (x.n_a > 0 ? (p.fused_L - p.fused_L1) * p.G : 0)) * kC;
+                for (int k0 = lane; k0 < total; k0 += 32 * kFly) {
+                    uint4 v[kFly];
+#pragma unroll
+                    for (int u = 0; u < kFly; ++u) {
+                        const int k = k0 + u * 32;
+                        if (k < total) {
+                            const int rr = k / kC, c = k - rr * kC;
+                            const int rw = rr < rows_b ? rr : rr - rows_b;
+                            const int lay = x.blk * p.fused_L + (rr < rows_b ? 0 : p.fused_L1) +
+                                            rw / p.G;
+                            v[u] = *reinterpret_cast<const uint4 *>(
+                                p.q_host + ((static_cast<size_t>(lay) * p.b + x.beta) * p.h +
+                                            x.j * p.G + rw % p.G) * D + c * 8);
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kFly; ++u) {
+                        const int k = k0 + u * 32;
+                        if (k < total) {
+                            const int rr = k / kC, c = k - rr * kC;
+                            const int rw = rr < rows_b ? rr : rr - rows_b;
+                            *reinterpret_cast<uint4 *>(
+                                dst + slot_of(rr < rows_b ? 1 : 0) * PL::kTileBytes +
+                                (c >> 3) * 16384 + rw * 128 + (((c & 7) ^ (rw & 7)) << 4)) = v[u];
+                        }
+                    }
+                }
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0)
+                    mbar_arrive(bar_q + 8 * qb);
+                if (kSplit)
+                    break;   // one unit per CTA
+            }
+        }
     }
 
+    tmem_fence_before();
     __syncthreads();
     if (warp == PL::kMma) {
         tmem_fence_after();
@@ -1013,7 +1166,9 @@ cudaError_t launch(int head_dim, bool fused, int form, const CUtensorMap *tmap_q
                    const CUtensorMap *tmap_kv, const PrefillParams &p, cudaStream_t stream)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(p.n_units));
+    // persistent CTAs: at most one wave, each taking units in turn (unit_index)
+    cfg.gridDim = dim3(static_cast<unsigned>(
+        min(p.n_units, p.sm_count * (form == kOneTile ? 2 : 1))));
     cfg.blockDim = dim3(static_cast<unsigned>(threads_of(head_dim, form)));
     cfg.dynamicSmemBytes = smem_of(head_dim, form);
     cfg.stream = stream;

@@ -75,6 +75,22 @@ def test_prefill_long_prompts(d):
         _prefill_model(owner, h, g, d, b, [2048, 1500], s_max, s_max, 52, cache, ref, nthreads=2)
 
 
+@pytest.mark.parametrize("h,g,d,b,s_max", [
+    (12, 1, 64, 23, 385),     # 1,104 units and fewer: several per persistent CTA, uneven rounds
+    (12, 4, 128, 37, 300),    # groups of 3: blocks in pairs, units with and without a tile A
+    (16, 4, 128, 40, 200),    # head pairs
+    (5, 5, 64, 61, 129),      # 305 heads of prompts: one CTA takes a second unit
+])
+def test_prefill_units_beyond_one_wave(h, g, d, b, s_max):
+    # More units than resident CTAs (152 SMs, two per SM at head_dim 64): every CTA runs several
+    # units on one set of barriers, query buffers and tensor-memory columns.
+    import paper_2406_09297_gb300 as mlkv
+    lens = [s_max if i % 3 == 0 else 1 + (i * 97) % s_max for i in range(b)]
+    with mlkv.MLKVCache(1, h, d, [0], g, b, s_max) as cache:
+        ref = oracle.OracleCache([0], h, g, d, b, s_max)
+        _prefill_model([0], h, g, d, b, lens, s_max, s_max, 55, cache, ref, nthreads=8)
+
+
 def test_prefill_long_prompt_every_row():
     # A 6000-position prompt: 47 key tiles per query block, units of very different lengths.
     import paper_2406_09297_gb300 as mlkv

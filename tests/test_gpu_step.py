@@ -497,3 +497,43 @@ def test_fused_step_host_buffers(chunked):
             assert mx <= MAX_ABS and mean <= MEAN_ABS, (n, mx, mean)
         cache.sync_status()
         cache2.sync_status()
+
+
+@pytest.mark.parametrize("owner,h,g,d,b", [
+    ([0, 0, 0, 3, 3, 3], 12, 4, 64, 47),    # one query tile, two CTAs per SM
+    ([0] * 12, 12, 1, 64, 160),             # 144 rows: two query tiles at head_dim 64
+    ([0, 0, 2, 2], 32, 8, 128, 11),         # head_dim 128
+])
+def test_fused_step_host_buffers_beyond_one_wave(owner, h, g, d, b):
+    # More units than resident CTAs, queries read from page-locked host memory: each persistent CTA
+    # loads its next unit's queries while the unit before still runs.  Equal, bit for bit, to the
+    # step on device buffers, and to the oracle within the tolerance.
+    import torch
+
+    import paper_2406_09297_gb300 as mlkv
+    l, L = len(owner), 300
+    lens = np.array([1 + (i * 131) % L for i in range(b)], dtype=np.int32)
+    with mlkv.MLKVCache(l, h, d, owner, g, b, L) as cache, \
+            mlkv.MLKVCache(l, h, d, owner, g, b, L) as cache2:
+        ref = oracle.OracleCache(owner, h, g, d, b, L)
+        qb, kn, vn = _inputs(owner, h, g, d, b, lens, L, 91, cache, ref)
+        _inputs(owner, h, g, d, b, lens, L, 91, cache2, None)
+        for c in (cache, cache2):
+            c.set_option("step_fused", 2)
+        Q, K, V = to_dev(qb), to_dev(kn), to_dev(vn)
+        want = torch.empty((l, b, h, d), dtype=torch.bfloat16, device="cuda")
+        cache2.decode_step(Q, K, V, want, lens)
+        hq, hk, hv = Q.cpu().pin_memory(), K.cpu().pin_memory(), V.cpu().pin_memory()
+        out = torch.full((l, b, h, d), float("nan"), dtype=torch.bfloat16).pin_memory()
+        cache.decode_step_host(hq, hk, hv, out, lens)
+        torch.cuda.synchronize()
+        assert cache.get_option("last_step_fused") == 1
+        assert torch.equal(out, want.cpu())
+        owners = sorted(set(owner))
+        for n in range(l):
+            if owner[n] == n:
+                k = owners.index(n)
+                ref.append(n, gen.bf16_bits_to_f64(kn[k]), gen.bf16_bits_to_f64(vn[k]), lens)
+            mx, mean = errors(from_dev(out[n]), ref.decode(n, gen.bf16_bits_to_f64(qb[n]), lens))
+            assert mx <= MAX_ABS and mean <= MEAN_ABS, (n, mx, mean)
+        cache.sync_status()
