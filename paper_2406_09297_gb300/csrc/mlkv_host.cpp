@@ -556,7 +556,7 @@ static int decode_impl(mlkv_cache_t c, int layer, const void *K_new, const void 
     // be better for a small layer: whole segments per CTA (no merge at all), or each segment in k
     // equal pieces run as one k-CTA cluster and merged over DSMEM.  They are chosen with a cost
     // model in units of one tile's consumer work (~0.5 us on GB300 when the tile is in L2):
-    // a DSMEM cluster merge costs ~2 tiles, the last-CTA merge of up to 4 partial records ~6 (a
+    // a DSMEM cluster merge costs ~2 tiles, the last-CTA merge of up to 8 partial records ~6 (a
     // global write, an atomic and the reads, after the previous layer has finished) and the
     // separate combine launch ~7.
     const long long wave = std::min<long long>(

@@ -241,8 +241,11 @@ int max_pieces_per_segment(const DecodeParams &p, int T, int grid);
 cudaError_t launch_combine(const DecodeParams &p, int head_dim, cudaStream_t stream,
                            bool pdl = true);
 
-// Pieces per segment above which the decode launch defers its merges to combine_kernel.
-constexpr int kInlineMergeMaxPieces = 4;
+// Pieces per segment above which the decode launch defers its merges to combine_kernel.  Up to 8
+// the last finisher's merge is one round trip to L2 (every record's loads in flight together); the
+// separate launch costs ~3 us a layer (8 sequences of up to 3000 positions, 8 KV heads of 128, 6
+// pieces at most: 529 -> 505 us for 32 layers when the bound went from 4 to 8).
+constexpr int kInlineMergeMaxPieces = 8;
 // combine_kernel keeps one weight per piece in shared memory.
 constexpr int kCombineMaxPiecesHost = 1024;
 

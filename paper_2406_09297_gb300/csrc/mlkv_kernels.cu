@@ -21,8 +21,12 @@
 //   update
 //   O += P V run on the tensor cores (mma.sync m16n8k16, bf16 in, fp32 accumulate) with the
 //   query group padded to M = 16 rows; the softmax is online, in fp32, base 2 with the 1/sqrt(d)
-//   scale folded into the exponent, with quad shuffles for row maxima.  The warps' states are
-//   merged through shared memory at the end of each piece.
+//   scale folded into the exponent, with quad shuffles for row maxima.  At the end of a piece each
+//   warp leaves its raw sums in shared memory and goes on; the epilogue warp merges them (the
+//   CTA's last piece: all consumer warps, after one barrier).  With the former tree over the
+//   consumer warps, a barrier a level, a piece boundary cost ~2 us at head_dim 128 (measured, 64
+//   uneven segments over 138 CTAs: layer calls 16.2 -> 13.4 us with the merge of up to 8 records
+//   in the launch, below).
 //
 //   Launch.  Programmatic dependent launch: barrier set-up overlaps the previous kernel of the
 //   stream, and no global memory is touched before griddepcontrol.wait.
@@ -59,16 +63,21 @@ struct Plan {
     static constexpr int kTW = T / NCW;               // positions per warp per tile
     static constexpr int kTileBytes = T * D * 2;      // one K (or V) tile
     static constexpr int kStageBytes = 2 * kTileBytes;
-    static constexpr int kWarpFrag = D * 64;          // one warp's O fragments: D/8*4 f32 x 32
-    static constexpr int kResO = 16 * D * 4;          // a piece's result: o[16][D] f32
-    static constexpr int kResBytes = kResO + 16 * 4 + 32;   // + lse[16] + 8 ints of metadata
-    static constexpr int kMerge = STAGES * kStageBytes;                 // [NCW/2][kWarpFrag]
-    static constexpr int kRes = kMerge + (NCW / 2) * kWarpFrag;        // [2][kResBytes]
-    static constexpr int kEpiW = kRes + 2 * kResBytes;                 // f32 [kEpiCap] weights
-    static constexpr int kEpiCap = 512;
-    static constexpr int kRedM = kEpiW + kEpiCap * 4;                  // f32 [NCW][16]
-    static constexpr int kRedL = kRedM + NCW * 16 * 4;                 // f32 [NCW][16]
-    static constexpr int kFlags = kRedL + NCW * 16 * 4;                // int [4]
+    static constexpr int kResO = 16 * D * 4;          // a cluster rank's result: o[16][D] f32
+    static constexpr int kResBytes = kResO + 16 * 4 + 32;   // + lse[16] (cluster slots)
+    // A finished piece: every warp's raw sums o[NCW][16][kRawRow] f32 (rows padded so that the
+    // fragment stores of a warp's 8 rows fall in distinct banks), its row maxima and sums
+    // [2][16][NCW], 8 ints of metadata and, in a cluster's leader, lse[16].
+    static constexpr int kRawRow = D + 8;
+    static constexpr int kRawO = NCW * 16 * kRawRow * 4;
+    static constexpr int kRawMeta = kRawO + 2 * 16 * NCW * 4;
+    static constexpr int kRawLse = kRawMeta + 32;
+    static constexpr int kRawBytes = kRawLse + 64;
+    // Two buffers where shared memory has room for them beside the ring.
+    static constexpr int kRawBufs = (D == 128 && T == 128) ? 2 : 1;
+    static constexpr int kRaw = STAGES * kStageBytes;                  // [kRawBufs][kRawBytes]
+    static constexpr int kEpiCap = 512;   // weights of the inline merge, behind a merged piece
+    static constexpr int kFlags = kRaw + kRawBufs * kRawBytes;         // int [4]
     // u64 full[S], empty[S], res_full[2], res_empty[2], cluster
     static constexpr int kBars = kFlags + 16;
     // Dynamic tail: per-sequence tables (lengths differ) or, in cluster mode, the leader's
@@ -80,15 +89,14 @@ struct Plan {
     static constexpr int kQ = (kBars + (2 * STAGES + 5) * 8 + 8 + 127) / 128 * 128;
     static constexpr int kTables = kQ + STAGES * kQSlot;
     static constexpr int kBytes = kTables;
-    static constexpr int kFinRow = D + 8;             // row stride (f32) of the last piece's sums
     static constexpr int kAlloc = kBytes + 1024;      // base aligned up to 1024 in the kernel
     static_assert(kTW % 16 == 0, "each warp takes whole 16-position mma steps");
     static_assert(NCW == 4 || NCW == 8, "tree merge over 4 or 8 warps");
     static_assert(D == 64 || D == 128, "head_dim 64 or 128");
     static_assert(T <= 256, "TMA box height");
     static_assert(kResBytes % 16 == 0, "result slots stay 16-byte aligned");
-    static_assert((NCW * 16 * kFinRow + 16) * 4 <= STAGES * kStageBytes,
-                  "the last piece's per-warp sums fit in the stage ring");
+    static_assert((16 * D + kEpiCap) * 4 <= kRawO, "a merged piece and its weights");
+    static_assert(kRawBytes % 16 == 0 && kRawMeta % 16 == 0, "raw buffers stay 16-byte aligned");
 };
 
 
@@ -292,7 +300,7 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
     }
     if (threadIdx.x == 0) {
         for (int r = 0; r < 2; ++r) {
-            mbar_init(bar_res_full + 8 * r, 1);
+            mbar_init(bar_res_full + 8 * r, NCW);
             mbar_init(bar_res_empty + 8 * r, 1);
         }
         mbar_init(bar_cluster, 1);
@@ -401,11 +409,14 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
 
     // -------------------------------- epilogue warp --------------------------------------------
     if (warp == PL::kEpilogue) {
-        float *s_w = reinterpret_cast<float *>(smem + PL::kEpiW);
+        // Merges the consumer warps' raw sums of every piece but the CTA's last while the
+        // consumers go on with the next piece: row by row m* = max_w m_w, l* = sum_w l_w 2^(m_w -
+        // m*), o = sum_w 2^(m_w - m*) o_w / l*, lse = m* + log2 l*.
+        constexpr int FS = PL::kRawRow;
         for (int k = 0;; ++k) {
-            const int rb = k & 1;
+            const int rb = k % PL::kRawBufs;
             int ok = 1;
-            if (lane == 0 && !mbar_wait(bar_res_full + 8 * rb, (k >> 1) & 1)) {
+            if (lane == 0 && !mbar_wait(bar_res_full + 8 * rb, (k / PL::kRawBufs) & 1)) {
                 flags[0] = 1;
                 atomicOr(p.err, kErrWaitFull);
                 ok = 0;
@@ -413,16 +424,71 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok)
                 break;
-            const uint8_t *slot = smem + PL::kRes + rb * PL::kResBytes;
-            const int *meta = reinterpret_cast<const int *>(slot + PL::kResO + 64);
+            uint8_t *slot = smem + PL::kRaw + rb * PL::kRawBytes;
+            const int *meta = reinterpret_cast<const int *>(slot + PL::kRawMeta);
             if (meta[kMetaStop])
                 break;
             if (early && k == 0)
                 grid_dependency_wait();   // records and merges use the shared scratch
-            if (!flags[0])
-                epilogue_piece<D>(p, reinterpret_cast<const float *>(slot),
-                                  reinterpret_cast<const float *>(slot + PL::kResO), meta, s_w,
-                                  PL::kEpiCap, lane, cta);
+            if (!flags[0]) {
+                float *raw = reinterpret_cast<float *>(slot);
+                float *st_m = reinterpret_cast<float *>(slot + PL::kRawO);   // [16][NCW]
+                float *st_l = st_m + 16 * NCW;
+                float *rlse = reinterpret_cast<float *>(slot + PL::kRawLse);
+                if (lane < p.G) {
+                    // lane r: row r's factors 2^(m_w - m*) / l* in place of m_w
+                    float mw[NCW], lw[NCW];
+#pragma unroll
+                    for (int w = 0; w < NCW; ++w) {
+                        mw[w] = st_m[lane * NCW + w];
+                        lw[w] = st_l[lane * NCW + w];
+                    }
+                    float ms = mw[0];
+#pragma unroll
+                    for (int w = 1; w < NCW; ++w)
+                        ms = fmaxf(ms, mw[w]);   // finite: the piece holds a visible position
+                    float ls = 0.f;
+#pragma unroll
+                    for (int w = 0; w < NCW; ++w) {
+                        mw[w] = fast_exp2(mw[w] - ms);
+                        ls = fmaf(lw[w], mw[w], ls);
+                    }
+                    const float inv = fast_rcp(ls);
+#pragma unroll
+                    for (int w = 0; w < NCW; ++w)
+                        st_m[lane * NCW + w] = mw[w] * inv;
+                    rlse[lane] = ms + fast_log2(ls);
+                }
+                __syncwarp();
+                // Compact result [G][D] over warp 0's rows: row r ends before raw row r + 1 starts.
+                constexpr int E = D / 32;   // columns per lane
+                for (int r = 0; r < p.G; ++r) {
+                    float f[NCW], v[E];
+#pragma unroll
+                    for (int w = 0; w < NCW; ++w)
+                        f[w] = st_m[r * NCW + w];
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        v[e] = 0.f;
+#pragma unroll
+                    for (int w = 0; w < NCW; ++w) {
+                        const float *src = raw + (w * 16 + r) * FS + lane * E;
+#pragma unroll
+                        for (int e = 0; e < E; e += 2) {
+                            const float2 x = *reinterpret_cast<const float2 *>(src + e);
+                            v[e] = fmaf(f[w], x.x, v[e]);
+                            v[e + 1] = fmaf(f[w], x.y, v[e + 1]);
+                        }
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int e = 0; e < E; e += 2)
+                        *reinterpret_cast<float2 *>(raw + r * D + lane * E + e) =
+                            make_float2(v[e], v[e + 1]);
+                }
+                __syncwarp();
+                epilogue_piece<D>(p, raw, rlse, meta, raw + 16 * D, PL::kEpiCap, lane, cta);
+            }
             __syncwarp();
             if (lane == 0)
                 mbar_arrive(bar_res_empty + 8 * rb);
@@ -434,9 +500,6 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
     }
 
     // -------------------------------- consumer warps -------------------------------------------
-    float *merge = reinterpret_cast<float *>(smem + PL::kMerge);
-    float *red_m = reinterpret_cast<float *>(smem + PL::kRedM);
-    float *red_l = reinterpret_cast<float *>(smem + PL::kRedL);
     const int qr = lane >> 2;              // fragment row (query head within the group)
     const int qc = (lane & 3) * 2;         // fragment column pair
     const int G = p.G;
@@ -694,130 +757,56 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
             wk.next(p, s_len, s_start);
         }
 
-        // ---------------- end of piece: merge the warps (no atomics) ----------------
-        // Row statistics of every warp -> per-row maximum m* and total l*; each warp's
-        // accumulators are weighted by 2^(m_w - m*) / l* and the warps summed.
-        const float l_run[2] = {la[0], la[2]};
-        if ((lane & 3) == 0) {
-            red_m[warp * 16 + qr] = m_run[0];
-            red_m[warp * 16 + qr + 8] = m_run[1];
-            red_l[warp * 16 + qr] = l_run[0];
-            red_l[warp * 16 + qr + 8] = l_run[1];
+        // ---------------- end of piece: every warp's raw sums to the piece's buffer -------------
+        // Pieces before the CTA's last go to the epilogue warp, and each warp goes straight on to
+        // the next piece (a tree over the warps with a barrier per level held all of them up for
+        // ~2 us a piece at head_dim 128).
+        constexpr int FS = PL::kRawRow;
+        const int rb = nhand % PL::kRawBufs;
+        uint8_t *slot_raw = smem + PL::kRaw + rb * PL::kRawBytes;
+        if (nhand >= PL::kRawBufs && !flags[0] &&
+            !mbar_wait(bar_res_empty + 8 * rb, ((nhand / PL::kRawBufs) & 1) ^ 1)) {
+            flags[0] = 1;
+            atomicOr(p.err, kErrWaitEmpty);
         }
-        // The barrier also guarantees that every warp is done with the ring's tiles.
-        consumer_bar_sync<NCW>();
+        float *fbuf = reinterpret_cast<float *>(slot_raw);                       // [NCW][16][FS]
+        float *red_m = reinterpret_cast<float *>(slot_raw + PL::kRawO);          // [16][NCW]
+        float *red_l = red_m + 16 * NCW;
+        float *flse = reinterpret_cast<float *>(slot_raw + PL::kRawLse);         // [16]
+#pragma unroll
+        for (int hr = 0; hr < 2; ++hr) {
+            const int row = qr + 8 * hr;
+            if (row < G) {
+#pragma unroll
+                for (int n = 0; n < NO; ++n)
+                    *reinterpret_cast<float2 *>(fbuf + (warp * 16 + row) * FS + n * 8 + qc) =
+                        make_float2(o[n][2 * hr], o[n][2 * hr + 1]);
+                if (qc == 0) {
+                    red_m[row * NCW + warp] = m_run[hr];
+                    red_l[row * NCW + warp] = la[2 * hr];
+                }
+            }
+        }
         if (piece_end != tile_hi) {
-            // A piece before the CTA's last: tree over warps, result to the epilogue warp, and
-            // the consumers go straight on to the next piece.
-            float lse[2];
-    #pragma unroll
-            for (int hr = 0; hr < 2; ++hr) {
-                const int row = qr + 8 * hr;
-                // every piece holds at least one visible position, so mstar is finite
-                float mstar = NEG_INF;
-    #pragma unroll
-                for (int w = 0; w < NCW; ++w)
-                    mstar = fmaxf(mstar, red_m[w * 16 + row]);
-                float lsum = 0.f;
-    #pragma unroll
-                for (int w = 0; w < NCW; ++w)
-                    lsum += red_l[w * 16 + row] * fast_exp2(red_m[w * 16 + row] - mstar);
-                const float f = fast_exp2(m_run[hr] - mstar) * fast_rcp(lsum);
-                lse[hr] = mstar + fast_log2(lsum);
-    #pragma unroll
-                for (int n = 0; n < NO; ++n) {
-                    o[n][2 * hr] *= f;
-                    o[n][2 * hr + 1] *= f;
-                }
+            if (warp == 0 && lane == 0) {
+                int *meta = reinterpret_cast<int *>(slot_raw + PL::kRawMeta);
+                meta[kMetaBeta] = beta;
+                meta[kMetaJ] = j;
+                meta[kMetaSeg] = seg;
+                meta[kMetaWhole] =
+                    (piece_first == seg_first && piece_end == seg_end && !part) ? 1 : 0;
+                meta[kMetaFirst] = ml ? rec : cta_of_tile(seg_first, N, P);
+                meta[kMetaLast] = cta_of_tile(seg_end - 1, N, P);
+                meta[kMetaStop] = 0;
+                meta[kMetaLayer] = layer;
             }
-            // Tree over warps with NCW/2 slots.  First level: warp w in [NCW/2, NCW) writes slot
-            // w - NCW/2 and warp r < NCW/2 adds slot r.  Later levels (half < NCW/2): warp w in
-            // [half, 2 half) writes slot w and warp r < half adds slot r + half.  Every slot is
-            // rewritten only by the warp that read it last, so one barrier per level suffices.
-    #pragma unroll
-            for (int half = NCW / 2; half >= 1; half >>= 1) {
-                const bool first = (half == NCW / 2);
-                if (warp >= half && warp < 2 * half) {
-                    float *dst = merge + (first ? warp - half : warp) * (NO * 4 * 32);
-    #pragma unroll
-                    for (int n = 0; n < NO; ++n)
-    #pragma unroll
-                        for (int c = 0; c < 4; ++c)
-                            dst[(n * 4 + c) * 32 + lane] = o[n][c];
-                }
-                consumer_bar_sync<NCW>();
-                if (warp < half) {
-                    const float *src = merge + (first ? warp : warp + half) * (NO * 4 * 32);
-    #pragma unroll
-                    for (int n = 0; n < NO; ++n)
-    #pragma unroll
-                        for (int c = 0; c < 4; ++c)
-                            o[n][c] += src[(n * 4 + c) * 32 + lane];
-                }
-            }
-
-            // Warp 0 hands the piece to the epilogue warp through a double-buffered slot and the
-            // consumers move on to the next piece at once.
-            if (warp == 0) {
-                const int rb = nhand & 1;
-                if (nhand >= 2 && !flags[0] &&
-                    !mbar_wait(bar_res_empty + 8 * rb, ((nhand >> 1) - 1) & 1)) {
-                    flags[0] = 1;
-                    atomicOr(p.err, kErrWaitEmpty);
-                }
-                uint8_t *slot = smem + PL::kRes + rb * PL::kResBytes;
-                float *ro = reinterpret_cast<float *>(slot);
-                float *rlse = reinterpret_cast<float *>(slot + PL::kResO);
-                int *meta = reinterpret_cast<int *>(slot + PL::kResO + 64);
-    #pragma unroll
-                for (int hr = 0; hr < 2; ++hr) {
-                    const int row = qr + 8 * hr;
-                    if (row < G) {
-    #pragma unroll
-                        for (int n = 0; n < NO; ++n)
-                            *reinterpret_cast<float2 *>(ro + row * D + n * 8 + qc) =
-                                make_float2(o[n][2 * hr], o[n][2 * hr + 1]);
-                        if (qc == 0)
-                            rlse[row] = lse[hr];
-                    }
-                }
-                if (lane == 0) {
-                    meta[kMetaBeta] = beta;
-                    meta[kMetaJ] = j;
-                    meta[kMetaSeg] = seg;
-                    meta[kMetaWhole] =
-                        (piece_first == seg_first && piece_end == seg_end && !part) ? 1 : 0;
-                    meta[kMetaFirst] = ml ? rec : cta_of_tile(seg_first, N, P);
-                    meta[kMetaLast] = cta_of_tile(seg_end - 1, N, P);
-                    meta[kMetaStop] = 0;
-                    meta[kMetaLayer] = layer;
-                }
-                __syncwarp();
-                if (lane == 0)
-                    mbar_arrive(bar_res_full + 8 * rb);
-            }
+            __syncwarp();
+            if (lane == 0)
+                mbar_arrive(bar_res_full + 8 * rb);
             ++nhand;
         } else {
-            // ---- the CTA's last piece: every tile has been consumed and no copy is pending, so
-            // the stage ring is free.  Each warp stores its raw accumulators there; after one
-            // barrier each consumer warp finishes one row per pass from every warp's statistics
-            // of the row: m* = max_w m_w, l* = sum_w l_w 2^(m_w - m*), o = sum_w 2^(m_w - m*) o_w
-            // / l*, lse = m* + log2 l*.
-            // Rows padded to D + 8 floats: the fragment stores of a warp's 8 rows then fall in
-            // distinct banks.
-            constexpr int FS = PL::kFinRow;
-            float *fbuf = reinterpret_cast<float *>(smem);         // [NCW][16][FS] f32
-            float *flse = fbuf + NCW * 16 * FS;                     // [16]
-#pragma unroll
-            for (int hr = 0; hr < 2; ++hr) {
-                const int row = qr + 8 * hr;
-                if (row < G) {
-#pragma unroll
-                    for (int n = 0; n < NO; ++n)
-                        *reinterpret_cast<float2 *>(fbuf + (warp * 16 + row) * FS + n * 8 + qc) =
-                            make_float2(o[n][2 * hr], o[n][2 * hr + 1]);
-                }
-            }
+            // ---- the CTA's last piece: after one barrier each consumer warp finishes one row per
+            // pass from every warp's statistics of the row (as the epilogue warp does).
             if (p.cluster_k > 1)
                 cluster_wait();   // the partner CTAs' barriers exist
             consumer_bar_sync<NCW>();
@@ -848,8 +837,8 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
                 float mw[NCW], lw[NCW];
 #pragma unroll
                 for (int w = 0; w < NCW; ++w) {
-                    mw[w] = red_m[w * 16 + row];
-                    lw[w] = red_l[w * 16 + row];
+                    mw[w] = red_m[row * NCW + w];
+                    lw[w] = red_l[row * NCW + w];
                 }
                 float ms = mw[0];   // finite: the piece holds a visible position
 #pragma unroll
@@ -938,7 +927,7 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
                 }
                 consumer_bar_sync<NCW>();
                 if (flags[1]) {
-                    // Last finisher of the segment: merge its <= 4 records (own included).
+                    // Last finisher of the segment: merge its <= 8 records (own included).
                     const int np = c_last - c_first + 1;
                     const size_t rec0 = static_cast<size_t>(seg + c_first);
 #pragma unroll 1
@@ -978,18 +967,16 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
     }
     if (early)
         grid_dependency_wait();   // no-op if already waited; this grid ends after the previous
-    // Tell the epilogue warp that no piece follows.
-    if (warp == 0) {
-        const int rb = nhand & 1;
-        if (nhand >= 2 && !flags[0] && !mbar_wait(bar_res_empty + 8 * rb, ((nhand >> 1) - 1) & 1)) {
-            flags[0] = 1;
-            atomicOr(p.err, kErrWaitEmpty);
-        }
-        if (lane == 0) {
-            int *meta = reinterpret_cast<int *>(smem + PL::kRes + rb * PL::kResBytes + PL::kResO + 64);
-            meta[kMetaStop] = 1;
+    // Tell the epilogue warp that no piece follows (the buffer is this piece's own; with no tiles at
+    // all it was never used).
+    {
+        const int rb = nhand % PL::kRawBufs;
+        if (warp == 0 && lane == 0)
+            reinterpret_cast<int *>(smem + PL::kRaw + rb * PL::kRawBytes + PL::kRawMeta)[kMetaStop] =
+                1;
+        __syncwarp();
+        if (lane == 0)
             mbar_arrive(bar_res_full + 8 * rb);
-        }
     }
 }
 

@@ -199,3 +199,25 @@ def test_cluster_rule_keeps_a_streaming_grid():
     # few CTAs, so the stream-K split over the SMs (and the separate merge) is kept.
     run_small_case([0, 0], 8, 1, 64, 1, [8192], 8192, seed=22, options={"tile_tokens": 128},
                    expect={"last_cluster_k": 0, "last_deferred_merge": 1})
+
+
+@pytest.mark.parametrize("d,tile", [(64, 64), (64, 128), (64, 256), (128, 64), (128, 128)])
+@pytest.mark.parametrize("pieces,deferred", [(5, 0), (7, 0), (9, 1)])
+def test_merge_of_five_to_nine_pieces(d, tile, pieces, deferred):
+    # One long segment a KV head over `pieces` CTAs: where a segment can meet at most 8 CTAs its
+    # records are merged by the last finisher, else by the merge launch (runs of 2 tiles: a segment
+    # of 2 k tiles meets k CTAs, and the bound for runs that start anywhere is k + 1).
+    nt = 2 * pieces
+    run_small_case([0], 6, 2, d, 1, [nt * tile - 5], nt * tile, seed=31, fused=True,
+                   options={"grid": 2 * pieces, "tile_tokens": tile, "cluster": 0},
+                   expect={"last_deferred_merge": deferred})
+
+
+@pytest.mark.parametrize("d,tile", [(64, 64), (64, 128), (64, 256), (128, 64), (128, 128)])
+@pytest.mark.parametrize("h,g", [(16, 1), (4, 4)])
+def test_many_pieces_a_cta(d, tile, h, g):
+    # Few CTAs, many short segments: every consumer warp hands its sums to the epilogue warp and
+    # goes on, a piece a tile or two, whole segments and cut ones, groups of 16 heads and of one.
+    lens = [1 + (i * 53) % (2 * tile) for i in range(37)]
+    run_small_case([0, 0], h, g, d, len(lens), lens, 2 * tile, seed=32, fused=True,
+                   options={"grid": 3, "tile_tokens": tile})
