@@ -453,6 +453,14 @@ __device__ __forceinline__ void st_async_v2(uint32_t a, float x, float y, uint32
         : "memory");
 }
 
+__device__ __forceinline__ void st_async_v4(uint32_t a, float4 v, uint32_t mbar)
+{
+    asm volatile(
+        "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::
+            "r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(mbar)
+        : "memory");
+}
+
 __device__ __forceinline__ void st_async_f32(uint32_t a, float x, uint32_t mbar)
 {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(a),

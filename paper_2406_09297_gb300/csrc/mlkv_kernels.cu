@@ -805,8 +805,9 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
                 mbar_arrive(bar_res_full + 8 * rb);
             ++nhand;
         } else {
-            // ---- the CTA's last piece: after one barrier each consumer warp finishes one row per
-            // pass from every warp's statistics of the row (as the epilogue warp does).
+            // ---- the CTA's last piece: after one barrier the consumer threads finish it together,
+            // four columns each a pass, from every warp's statistics of their row (as the epilogue
+            // warp does).
             if (p.cluster_k > 1)
                 cluster_wait();   // the partner CTAs' barriers exist
             consumer_bar_sync<NCW>();
@@ -814,8 +815,8 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
             const bool whole = (piece_first == seg_first && piece_end == seg_end && !part);
             __nv_bfloat16 *ob = p.out + static_cast<size_t>(layer) * p.ml_q_stride +
                                 (static_cast<size_t>(beta) * p.h + static_cast<size_t>(j) * G) * D;
-            constexpr int kPairs = NCW * 32;   // float2 outputs per pass
-            static_assert(D == 2 * 32 || D == 4 * 32, "a warp's pass covers 64 elements of one row");
+            constexpr int kPass = 4 * NCW * 32;   // outputs per pass
+            static_assert(D % 4 == 0, "a thread's four columns lie in one row");
             // mode: 0 whole, 1 cluster sender, 2 cluster leader, 3 partial record
             const int rank = p.cluster_k > 1 ? static_cast<int>(cluster_ctarank()) : 0;
             const int mode = whole ? 0 : (p.cluster_k > 1 ? (rank != 0 ? 1 : 2) : 3);
@@ -831,9 +832,9 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
             const size_t piece = ml ? static_cast<size_t>(rec) : static_cast<size_t>(seg + cta);
             float *po = p.part_o + piece * G * D;
 #pragma unroll 2
-            for (int i = 2 * ctid; i < G * D; i += 2 * kPairs) {
-                const int row = i / D, e = i - row * D;   // row is the same across the warp
-                // independent broadcast loads of the row's statistics of every warp
+            for (int i = 4 * ctid; i < G * D; i += kPass) {
+                const int row = i / D, e = i - row * D;
+                // independent loads of the row's statistics of every warp
                 float mw[NCW], lw[NCW];
 #pragma unroll
                 for (int w = 0; w < NCW; ++w) {
@@ -845,39 +846,66 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
                 for (int w = 1; w < NCW; ++w)
                     ms = fmaxf(ms, mw[w]);
                 float ls = 0.f;
-                float2 v = make_float2(0.f, 0.f);
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                 for (int w = 0; w < NCW; ++w) {
                     const float ew = fast_exp2(mw[w] - ms);
                     ls = fmaf(lw[w], ew, ls);
-                    const float2 x =
-                        *reinterpret_cast<const float2 *>(fbuf + (w * 16 + row) * FS + e);
+                    const float4 x =
+                        *reinterpret_cast<const float4 *>(fbuf + (w * 16 + row) * FS + e);
                     v.x = fmaf(ew, x.x, v.x);
                     v.y = fmaf(ew, x.y, v.y);
+                    v.z = fmaf(ew, x.z, v.z);
+                    v.w = fmaf(ew, x.w, v.w);
                 }
                 const float inv = fast_rcp(ls);
                 v.x *= inv;
                 v.y *= inv;
+                v.z *= inv;
+                v.w *= inv;
                 const float lse_row = ms + fast_log2(ls);
-                const bool row_head = (e == 0 && lane == 0);   // one lane per row
+                const bool row_head = e == 0;   // one thread per row
                 if (mode == 0) {
-                    *reinterpret_cast<uint32_t *>(ob + i) = pack_bf16x2(v.x, v.y);
+                    *reinterpret_cast<uint2 *>(ob + i) =
+                        make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
                 } else if (mode == 1) {
                     // the leader's barrier completes when all these bytes have landed
-                    st_async_v2(remote + i * 4, v.x, v.y, remote_bar);
+                    st_async_v4(remote + i * 4, v, remote_bar);
                     if (row_head)
                         st_async_f32(remote + PL::kResO + row * 4, lse_row, remote_bar);
                 } else if (mode == 2) {
                     // each element is read and rewritten by this thread alone
-                    *reinterpret_cast<float2 *>(fbuf + row * FS + e) = v;
+                    *reinterpret_cast<float4 *>(fbuf + row * FS + e) = v;
                     if (row_head)
                         flse[row] = lse_row;
                 } else {
-                    *reinterpret_cast<float2 *>(po + i) = v;
+                    *reinterpret_cast<float4 *>(po + i) = v;
                     if (row_head)
                         p.part_lse[piece * G + row] = lse_row;
                 }
             }
+            // Weighted mean of the four columns of up to K records.
+            auto merge4 = [&](const auto &l, const auto &x) {
+                constexpr int K = sizeof(l) / sizeof(l[0]);
+                float mx = NEG_INF;
+#pragma unroll
+                for (int k = 0; k < K; ++k)
+                    mx = fmaxf(mx, l[k]);
+                float tot = 0.f;
+                float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    const float w = fast_exp2(l[k] - mx);   // 0 past the records
+                    tot += w;
+                    a.x = fmaf(w, x[k].x, a.x);
+                    a.y = fmaf(w, x[k].y, a.y);
+                    a.z = fmaf(w, x[k].z, a.z);
+                    a.w = fmaf(w, x[k].w, a.w);
+                }
+                const float inv = fast_rcp(tot);
+                return make_uint2(pack_bf16x2(a.x * inv, a.y * inv),
+                                  pack_bf16x2(a.z * inv, a.w * inv));
+            };
             if (mode == 2) {
                 // Leader: its own result is in warp 0's rows; merge the other ranks' once landed.
                 if (!flags[0] && !mbar_wait_cluster(bar_cluster, 0)) {
@@ -886,40 +914,32 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
                 }
                 consumer_bar_sync<NCW>();   // flse is complete
                 const int k = p.cluster_k;   // 2 or 4
+                const bool stop = flags[0] != 0;
 #pragma unroll 2
-                for (int i = 2 * ctid; i < G * D; i += 2 * kPairs) {
+                for (int i = 4 * ctid; i < G * D; i += kPass) {
                     const int row = i / D, e = i - row * D;
                     float lr[4];
-                    float2 x[4];
+                    float4 x[4];
                     lr[0] = flse[row];
-                    x[0] = *reinterpret_cast<const float2 *>(fbuf + row * FS + e);
+                    x[0] = *reinterpret_cast<const float4 *>(fbuf + row * FS + e);
 #pragma unroll
                     for (int r = 1; r < 4; ++r) {
                         lr[r] = NEG_INF;
-                        x[r] = make_float2(0.f, 0.f);
+                        x[r] = make_float4(0.f, 0.f, 0.f, 0.f);
                         if (r < k) {
                             const uint8_t *sl = cs + (r - 1) * PL::kResBytes;
                             lr[r] = reinterpret_cast<const float *>(sl + PL::kResO)[row];
-                            x[r] = *reinterpret_cast<const float2 *>(sl + static_cast<size_t>(i) * 4);
+                            x[r] = *reinterpret_cast<const float4 *>(sl + static_cast<size_t>(i) * 4);
                         }
                     }
-                    const float mx = fmaxf(fmaxf(lr[0], lr[1]), fmaxf(lr[2], lr[3]));
-                    float tot = 0.f, ax = 0.f, ay = 0.f;
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const float w = fast_exp2(lr[r] - mx);   // 0 past k
-                        tot += w;
-                        ax = fmaf(w, x[r].x, ax);
-                        ay = fmaf(w, x[r].y, ay);
-                    }
-                    const float inv = fast_rcp(tot);
-                    if (!flags[0])
-                        *reinterpret_cast<uint32_t *>(ob + i) = pack_bf16x2(ax * inv, ay * inv);
+                    const uint2 o4 = merge4(lr, x);
+                    if (!stop)
+                        *reinterpret_cast<uint2 *>(ob + i) = o4;
                 }
             } else if (mode == 3 && !p.deferred_merge) {
                 const int c_first = cta_of_tile(seg_first, N, P);
                 const int c_last = cta_of_tile(seg_end - 1, N, P);
-                __threadfence();
+                // The barrier puts every thread's record before thread 0's release.
                 consumer_bar_sync<NCW>();
                 if (ctid == 0) {
                     const unsigned prev = atomic_add_acq_rel_gpu(&p.counters[seg], 1u);
@@ -927,36 +947,26 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
                 }
                 consumer_bar_sync<NCW>();
                 if (flags[1]) {
-                    // Last finisher of the segment: merge its <= 8 records (own included).
+                    // Last finisher of the segment: merge its <= 8 records (own included), every
+                    // record's loads of a pass in flight together.
                     const int np = c_last - c_first + 1;
                     const size_t rec0 = static_cast<size_t>(seg + c_first);
 #pragma unroll 1
-                    for (int i = 2 * ctid; i < G * D; i += 2 * kPairs) {
+                    for (int i = 4 * ctid; i < G * D; i += kPass) {
                         const int row = i / D;
                         float lv[kInlineMergeMaxPieces];
-                        float2 ov[kInlineMergeMaxPieces];
-                        float mx = NEG_INF;
+                        float4 ov[kInlineMergeMaxPieces];
 #pragma unroll
                         for (int k = 0; k < kInlineMergeMaxPieces; ++k) {
                             lv[k] = NEG_INF;
-                            ov[k] = make_float2(0.f, 0.f);
+                            ov[k] = make_float4(0.f, 0.f, 0.f, 0.f);
                             if (k < np) {
                                 lv[k] = __ldcg(&p.part_lse[(rec0 + k) * G + row]);
-                                ov[k] = __ldcg(reinterpret_cast<const float2 *>(
+                                ov[k] = __ldcg(reinterpret_cast<const float4 *>(
                                     p.part_o + (rec0 + k) * G * D + i));
                             }
-                            mx = fmaxf(mx, lv[k]);
                         }
-                        float tot = 0.f, ax = 0.f, ay = 0.f;
-#pragma unroll
-                        for (int k = 0; k < kInlineMergeMaxPieces; ++k) {
-                            const float w = fast_exp2(lv[k] - mx);   // 0 past np
-                            tot += w;
-                            ax += w * ov[k].x;
-                            ay += w * ov[k].y;
-                        }
-                        const float inv = fast_rcp(tot);
-                        *reinterpret_cast<uint32_t *>(ob + i) = pack_bf16x2(ax * inv, ay * inv);
+                        *reinterpret_cast<uint2 *>(ob + i) = merge4(lv, ov);
                     }
                     if (ctid == 0)
                         p.counters[seg] = 0u;
