@@ -69,6 +69,19 @@ def test_merge_matches_oracle(name, owner, h, g, row):
     _check(owner, h, g, W, _merge(owner, h, g, W))
 
 
+@pytest.mark.parametrize("l,h", [(1, 3), (1, 5), (1, 7), (3, 3), (1, 11), (2, 6), (1, 13), (4, 6),
+                                 (5, 5), (3, 12), (6, 12), (11, 9), (12, 12), (1, 2), (16, 16)])
+@pytest.mark.parametrize("scale", [0, 100, -110])
+def test_merge_member_counts(l, h, scale):
+    # The mean's quotient for member counts of every kind (odd, even, powers of two), weights near
+    # 1 and scaled to the ends of the exponent range (there the mean is at least 2^-124, so its
+    # quotient stays a normal float), columns of unlike magnitudes.
+    W = gen.bf16_bits_to_f64(_weights(64 + l * h, l, h, 512))
+    W = np.ldexp(W, scale + (np.arange(512) % 9 - 4)[None, None, :])
+    W = _bf16(W)
+    _check([0] * l, h, 1, W, _merge([0] * l, h, 1, W))
+
+
 def test_identity_map_copies_bits():
     W = _weights(62, 3, 6, 256)
     np.testing.assert_array_equal(_merge([0, 1, 2], 6, 6, W), W)
