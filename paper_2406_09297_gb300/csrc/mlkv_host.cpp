@@ -863,6 +863,7 @@ static int fused_issue(mlkv_cache_t c, const void *Q, void *out, int n_q_layers,
     p.s_max = c->max_seq;
     p.slot = slot0;
     p.sm_count = c->sm_count;
+    p.kv_direct = 0;
     p.head_pairs = 0;
     p.fused_L = L;
     p.fused_L1 = L1;
@@ -1747,6 +1748,36 @@ int mlkv_decode_step_host(mlkv_cache_t c, const void *Q, const void *K, const vo
     return record_or_replay(c, key, c->host_key, c->host_pending, c->host_exec, stream, issue);
 }
 
+// Stores positions [0, len) of an owner layer's keys and values in its slot: one kernel for 16-byte
+// aligned tensors, else two pitched copies.  under_prefill: see launch_prefix_copy.
+static int store_prefix(mlkv_cache_t c, int layer, const void *K, const void *V, int len,
+                        cudaStream_t s, bool under_prefill)
+{
+    const size_t row = static_cast<size_t>(len) * c->d * 2;
+    const size_t pitch = static_cast<size_t>(c->max_seq) * c->d * 2;
+    const size_t slot_bytes = c->cache_bytes / c->m;
+    char *base = static_cast<char *>(c->cache) + slot_bytes * c->slot[layer];
+    const size_t rows = static_cast<size_t>(c->b) * c->g;
+    if (aligned16(K) && aligned16(V)) {
+        mlkv::PrefixParams p;
+        p.K = static_cast<const uint4 *>(K);
+        p.V = static_cast<const uint4 *>(V);
+        p.k_dst = reinterpret_cast<uint4 *>(base);
+        p.v_dst = reinterpret_cast<uint4 *>(base + slot_bytes / 2);
+        p.rows = static_cast<long long>(rows);
+        p.row_vecs = static_cast<long long>(row / 16);
+        p.pitch_vecs = static_cast<long long>(pitch / 16);
+        p.under_prefill = under_prefill ? 1 : 0;
+        const cudaError_t e = mlkv::launch_prefix_copy(p, s);
+        return e == cudaSuccess ? MLKV_OK : fail_cuda(e, "prefix copy");
+    }
+    cudaError_t e = cudaMemcpy2DAsync(base, pitch, K, row, row, rows, cudaMemcpyDeviceToDevice, s);
+    if (e == cudaSuccess)
+        e = cudaMemcpy2DAsync(base + slot_bytes / 2, pitch, V, row, row, rows,
+                              cudaMemcpyDeviceToDevice, s);
+    return e == cudaSuccess ? MLKV_OK : fail_cuda(e, "prefix copy");
+}
+
 int mlkv_load_prefix(mlkv_cache_t c, int layer, const void *K, const void *V, int len,
                      void *cuda_stream)
 {
@@ -1763,19 +1794,7 @@ int mlkv_load_prefix(mlkv_cache_t c, int layer, const void *K, const void *V, in
     if (K == nullptr || V == nullptr)
         return fail(MLKV_ERR_INVALID_ARG, "K and V must be non-NULL");
     DeviceGuard guard(c->device);
-    const size_t row = static_cast<size_t>(len) * c->d * 2;
-    const size_t pitch = static_cast<size_t>(c->max_seq) * c->d * 2;
-    const size_t slot_bytes = c->cache_bytes / c->m;
-    char *base = static_cast<char *>(c->cache) + slot_bytes * c->slot[layer];
-    const size_t rows = static_cast<size_t>(c->b) * c->g;
-    cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    cudaError_t e = cudaMemcpy2DAsync(base, pitch, K, row, row, rows, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpy2DAsync(base + slot_bytes / 2, pitch, V, row, row, rows,
-                              cudaMemcpyDeviceToDevice, s);
-    if (e != cudaSuccess)
-        return fail_cuda(e, "prefix copy");
-    return MLKV_OK;
+    return store_prefix(c, layer, K, V, len, static_cast<cudaStream_t>(cuda_stream), false);
 }
 
 int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const void *V, void *out,
@@ -1811,12 +1830,6 @@ int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const 
         return fail(MLKV_ERR_INVALID_ARG, "K and V must be non-NULL and 16-byte aligned");
     DeviceGuard guard(c->device);
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    // Sec. 3: only an owner layer stores K/V -- the prompt's, at positions [0, s_max).
-    if (owner) {
-        int rc = mlkv_load_prefix(c, layer, K, V, s_max, cuda_stream);
-        if (rc != MLKV_OK)
-            return rc;
-    }
     cudaError_t e;
     if (!c->prefill_ready) {
         if ((e = mlkv::prepare_prefill(c->d)) != cudaSuccess)
@@ -1842,7 +1855,26 @@ int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const 
     if (r != CUDA_SUCCESS)
         return fail(MLKV_ERR_CUDA, "cuTensorMapEncodeTiled(Q) failed (CUresult %d)",
                     static_cast<int>(r));
-    // The cache, with boxes of 128 positions (the map of the 128-position decode variant).
+    // K and V in boxes of 128 positions: an owner layer's prompt where it is, [b][g][s_max][d]; for
+    // the other layers the cache (the map of the 128-position decode variant).
+    CUtensorMap tmap_in[2];
+    if (owner) {
+        const cuuint64_t kdims[3] = {static_cast<cuuint64_t>(c->d), static_cast<cuuint64_t>(s_max),
+                                     static_cast<cuuint64_t>(c->b) * c->g};
+        const cuuint64_t kstrides[2] = {static_cast<cuuint64_t>(c->d) * 2,
+                                        static_cast<cuuint64_t>(s_max) * c->d * 2};
+        const cuuint32_t kbox[3] = {64u, 128u, 1u};
+        const void *kv[2] = {K, V};
+        for (int i = 0; i < 2; ++i) {
+            r = encode(&tmap_in[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(kv[i]),
+                       kdims, kstrides, kbox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                       CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+            if (r != CUDA_SUCCESS)
+                return fail(MLKV_ERR_CUDA, "cuTensorMapEncodeTiled(prompt K/V) failed (CUresult %d)",
+                            static_cast<int>(r));
+        }
+    }
     const CUtensorMap *tmap_kv = nullptr;
     for (auto &v : c->variants)
         if (v.v->tile_tokens == 128)
@@ -1861,7 +1893,10 @@ int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const 
     p.s_max = s_max;
     p.slot = c->slot[layer];
     p.sm_count = c->sm_count;
+    p.kv_direct = owner ? 1 : 0;
     p.fused_L = p.fused_L1 = 0;
+    const CUtensorMap *tmap_k = owner ? &tmap_in[0] : tmap_kv;
+    const CUtensorMap *tmap_v = owner ? &tmap_in[1] : tmap_kv;
     for (int beta = 0; beta < c->b; ++beta)
         p.prompt_len[beta] = prompt_lens[beta];
     // Work units, those that see the most keys first.  head_dim 64: one query block of one head
@@ -1882,7 +1917,7 @@ int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const 
                              (static_cast<uint32_t>(sel) << 24);
                 if (++n == mlkv::kPrefillMaxUnits) {
                     p.n_units = n;
-                    if ((e = mlkv::launch_prefill(c->d, &tmap_q, tmap_kv, p, stream)) !=
+                    if ((e = mlkv::launch_prefill(c->d, &tmap_q, tmap_k, tmap_v, p, stream)) !=
                         cudaSuccess)
                         return fail_cuda(e, "prefill launch");
                     n = 0;
@@ -1892,10 +1927,11 @@ int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const 
     }
     if (n > 0) {
         p.n_units = n;
-        if ((e = mlkv::launch_prefill(c->d, &tmap_q, tmap_kv, p, stream)) != cudaSuccess)
+        if ((e = mlkv::launch_prefill(c->d, &tmap_q, tmap_k, tmap_v, p, stream)) != cudaSuccess)
             return fail_cuda(e, "prefill launch");
     }
-    return MLKV_OK;
+    // Sec. 3: only an owner layer stores K/V -- the prompt's, at positions [0, s_max).
+    return owner ? store_prefix(c, layer, K, V, s_max, stream, true) : MLKV_OK;
 }
 
 int mlkv_decode_block_fused(mlkv_cache_t c, int owner_layer, const void *Q, void *out,

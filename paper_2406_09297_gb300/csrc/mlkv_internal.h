@@ -104,6 +104,8 @@ struct PrefillParams {
     float scale_log2;         // log2(e) / sqrt(D)
     int b, h, g, G, s_max, slot, n_units, head_pairs;
     int sm_count;             // the launch's persistent CTAs: one or two per SM, at most n_units
+    int kv_direct;            // prefill: K and V are the prompt's own tensors (an owner layer), each
+                              // under a map of its own; 0: the cache slot's, under one map
     // Cross-layer fused decode (mlkv_decode_block_fused, and mlkv_decode_step's fused form): every
     // block has L layers, L1 of them in tile B (the rest in tile A); prompt_len holds the sequence
     // lengths.  Both 0 for prefill.  A unit's block blk (fused_nblk blocks in all) reads slot
@@ -132,8 +134,8 @@ struct PrefillParams {
 // programmatic dependent launch on `stream`.
 size_t prefill_smem_bytes(int head_dim);
 cudaError_t prepare_prefill(int head_dim);
-cudaError_t launch_prefill(int head_dim, const CUtensorMap *tmap_q, const CUtensorMap *tmap_kv,
-                           const PrefillParams &p, cudaStream_t stream);
+cudaError_t launch_prefill(int head_dim, const CUtensorMap *tmap_q, const CUtensorMap *tmap_k,
+                           const CUtensorMap *tmap_v, const PrefillParams &p, cudaStream_t stream);
 // Fused decode forms (head_dim 64 with L * G <= 128 may take either one-tile form; otherwise the
 // two-tile form is used whatever is asked): 0 two query tiles per CTA; 1 one tile, two CTAs per
 // SM; 2 one tile, one CTA per SM with a 12-tile ring and two S buffers.
@@ -255,5 +257,17 @@ cudaError_t max_active_clusters(const DecodeVariant &v, int k, int *out);
 // Every owner slot's new token in one launch (mlkv_stage.cu), for the fused step.
 cudaError_t launch_append_slots(const AppendParams &p, cudaStream_t stream);
 cudaError_t launch_append(const AppendParams &p, cudaStream_t stream);
+
+// The keys and values of positions [0, row_vecs / (D / 8)) into a slot (mlkv_stage.cu): `rows` rows
+// (sequence, KV head) of K and of V, row_vecs 16-byte vectors each, contiguous in the source and
+// pitch_vecs apart in the slot.  under_prefill: launched right behind the prefill kernel that reads
+// the same K and V (and does not read the slot): runs in its tail, waiting for it only at the end.
+struct PrefixParams {
+    const uint4 *K, *V;
+    uint4 *k_dst, *v_dst;
+    long long rows, row_vecs, pitch_vecs;
+    int under_prefill;
+};
+cudaError_t launch_prefix_copy(const PrefixParams &p, cudaStream_t stream);
 
 }  // namespace mlkv

@@ -2,8 +2,9 @@
 //
 // Prefill runs a whole prompt through one layer at once: prompt position t of query head i
 // attends to positions 0 .. t of KV head j(i) = i / G of the layer's owner slot (causal
-// attention, Eqs. 2-3 with the MLKV maps of Eqs. 13-18).  Owner layers first store the prompt's
-// K/V in their slot (mlkv_host.cpp); every layer of the block then attends over it.
+// attention, Eqs. 2-3 with the MLKV maps of Eqs. 13-18).  An owner layer attends over the prompt's
+// K/V where they are and stores them in its slot (prefix_copy_kernel, launched behind this kernel
+// and running in its tail); the block's other layers attend over the slot.
 //
 // Persistent CTAs: the grid is at most one wave, and CTA c takes units c, 2P - 1 - c, 2P + c, ... of
 // the longest-first list (P CTAs).  All roles run on over the units: while a unit's last tile is in
@@ -171,7 +172,7 @@ struct Unit {
     int n_a, n_b;         // key tiles of query tiles A (0: no tile A) and B, n_a <= n_b
     int qb_b;             // prefill: tile B's query block
     int head_a, head_b, j;
-    int zk, zv;           // rows of the cache's tensor map: K and V of (slot, sequence, KV head)
+    int zk, zv;           // rows of the K and V tensor maps: (slot, sequence, KV head)
     bool has_end;         // the unit holds the sequence's last key tile
 };
 
@@ -205,8 +206,12 @@ __device__ __forceinline__ Unit unit_of(const PrefillParams &p, int i)
         x.head_b = p.head_pairs ? 2 * sel + 1 : sel;
         x.j = x.head_b / p.G;   // Eq. 15
     }
-    x.zk = (((p.slot + x.blk) * 2 + 0) * p.b + x.beta) * p.g + x.j;
-    x.zv = x.zk + p.b * p.g;
+    if (!kFused && p.kv_direct) {   // the prompt's own tensors, [b][g][s_max][D] each
+        x.zk = x.zv = x.beta * p.g + x.j;
+    } else {
+        x.zk = (((p.slot + x.blk) * 2 + 0) * p.b + x.beta) * p.g + x.j;
+        x.zv = x.zk + p.b * p.g;
+    }
     return x;
 }
 
@@ -223,7 +228,8 @@ template <int D, bool kFused, int kForm>
 __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
                                   PrefillPlan<D, kForm>::kMinBlocks)
     prefill_kernel(const __grid_constant__ CUtensorMap tmap_q,
-                   const __grid_constant__ CUtensorMap tmap_kv,
+                   const __grid_constant__ CUtensorMap tmap_k,
+                   const __grid_constant__ CUtensorMap tmap_v,
                    const __grid_constant__ PrefillParams p)
 {
     using PL = PrefillPlan<D, kForm>;
@@ -280,7 +286,8 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
     }
     if (threadIdx.x == PL::kProducer * 32) {
         prefetch_tensormap(&tmap_q);
-        prefetch_tensormap(&tmap_kv);
+        prefetch_tensormap(&tmap_k);
+        prefetch_tensormap(&tmap_v);
     }
     if (warp == PL::kMma) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -355,8 +362,9 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
             __syncwarp();
             const int sub = lane - (idx & 7) * 2;   // the lanes take turns
             if (sub >= 0 && sub < PL::kSub)
-                tma_load_3d(sbase + PL::kRing + s * PL::kTileBytes + sub * 16384, &tmap_kv, fb,
-                            sub * 64, ((k >> 1) + x.kt0) * 128, (k & 1) ? x.zv : x.zk);
+                tma_load_3d(sbase + PL::kRing + s * PL::kTileBytes + sub * 16384,
+                            (k & 1) ? &tmap_v : &tmap_k, fb, sub * 64, ((k >> 1) + x.kt0) * 128,
+                            (k & 1) ? x.zv : x.zk);
             ++idx;
             return true;
         };
@@ -1163,7 +1171,8 @@ const void *kernel_fn(int head_dim, bool fused, int form)
 }
 
 cudaError_t launch(int head_dim, bool fused, int form, const CUtensorMap *tmap_q,
-                   const CUtensorMap *tmap_kv, const PrefillParams &p, cudaStream_t stream)
+                   const CUtensorMap *tmap_k, const CUtensorMap *tmap_v, const PrefillParams &p,
+                   cudaStream_t stream)
 {
     cudaLaunchConfig_t cfg = {};
     // persistent CTAs: at most one wave, each taking units in turn (unit_index)
@@ -1177,8 +1186,8 @@ cudaError_t launch(int head_dim, bool fused, int form, const CUtensorMap *tmap_q
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    void *args[] = {const_cast<CUtensorMap *>(tmap_q), const_cast<CUtensorMap *>(tmap_kv),
-                    const_cast<PrefillParams *>(&p)};
+    void *args[] = {const_cast<CUtensorMap *>(tmap_q), const_cast<CUtensorMap *>(tmap_k),
+                    const_cast<CUtensorMap *>(tmap_v), const_cast<PrefillParams *>(&p)};
     return cudaLaunchKernelExC(&cfg, kernel_fn(head_dim, fused, form), args);
 }
 
@@ -1216,16 +1225,16 @@ cudaError_t prepare_fused(int head_dim, int form)
     return prepare(head_dim, true, fused_form(head_dim, form));
 }
 
-cudaError_t launch_prefill(int head_dim, const CUtensorMap *tmap_q, const CUtensorMap *tmap_kv,
-                           const PrefillParams &p, cudaStream_t stream)
+cudaError_t launch_prefill(int head_dim, const CUtensorMap *tmap_q, const CUtensorMap *tmap_k,
+                           const CUtensorMap *tmap_v, const PrefillParams &p, cudaStream_t stream)
 {
-    return launch(head_dim, false, prefill_form(head_dim), tmap_q, tmap_kv, p, stream);
+    return launch(head_dim, false, prefill_form(head_dim), tmap_q, tmap_k, tmap_v, p, stream);
 }
 
 cudaError_t launch_fused(int head_dim, int form, const CUtensorMap *tmap_q,
                          const CUtensorMap *tmap_kv, const PrefillParams &p, cudaStream_t stream)
 {
-    return launch(head_dim, true, fused_form(head_dim, form), tmap_q, tmap_kv, p, stream);
+    return launch(head_dim, true, fused_form(head_dim, form), tmap_q, tmap_kv, tmap_kv, p, stream);
 }
 
 cudaError_t launch_fused_combine(int head_dim, const PrefillParams &p, cudaStream_t stream)

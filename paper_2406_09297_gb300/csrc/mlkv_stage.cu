@@ -64,7 +64,61 @@ __global__ void __launch_bounds__(256) append_slots_kernel(const __grid_constant
     *dst = *src;
 }
 
+constexpr int kPrefixChunk = 1024;   // 16-byte vectors of one CTA: 4 a thread, all in flight
+
+// One CTA per 16 KB of a row; HBM-bound.
+__global__ void __launch_bounds__(256) prefix_copy_kernel(const __grid_constant__ PrefixParams p)
+{
+    // Behind the prefill of the same prompt: that kernel let this one go only after its own
+    // dependency wait, so K and V are in place and nothing earlier reads the slot.
+    if (!p.under_prefill)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+    const long long per_row = (p.row_vecs + kPrefixChunk - 1) / kPrefixChunk;
+    const long long r2 = blockIdx.x / per_row;   // K's rows, then V's
+    const long long c0 = (blockIdx.x - r2 * per_row) * kPrefixChunk;
+    const bool is_v = r2 >= p.rows;
+    const long long row = is_v ? r2 - p.rows : r2;
+    const uint4 *src = (is_v ? p.V : p.K) + row * p.row_vecs;
+    uint4 *dst = (is_v ? p.v_dst : p.k_dst) + row * p.pitch_vecs;
+    uint4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const long long i = c0 + u * 256 + threadIdx.x;
+        if (i < p.row_vecs)
+            v[u] = src[i];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const long long i = c0 + u * 256 + threadIdx.x;
+        if (i < p.row_vecs)
+            dst[i] = v[u];
+    }
+    // This grid ends after the prefill's (one waiting CTA is enough; the others leave their place to
+    // the copies still to come), so what waits for it waits for both.
+    if (p.under_prefill && blockIdx.x == 0)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 }  // namespace
+
+cudaError_t launch_prefix_copy(const PrefixParams &p, cudaStream_t stream)
+{
+    const long long per_row = (p.row_vecs + kPrefixChunk - 1) / kPrefixChunk;
+    const long long blocks = 2 * p.rows * per_row;
+    if (blocks > 0x7FFFFFFFLL)
+        return cudaErrorInvalidConfiguration;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(blocks));
+    cfg.blockDim = dim3(256);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    void *args[] = {const_cast<PrefixParams *>(&p)};
+    return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(&prefix_copy_kernel), args);
+}
 
 cudaError_t launch_append_slots(const AppendParams &p, cudaStream_t stream)
 {

@@ -80,6 +80,42 @@ def test_append_and_prefix_placement_bit_exact():
         c.sync_status()
 
 
+@pytest.mark.parametrize("d,length,s", [
+    (64, 1, 1), (64, 1, 300), (64, 127, 128), (64, 128, 200), (64, 129, 200),   # 1024 vectors a CTA
+    (128, 64, 65), (128, 65, 70), (64, 2000, 2000),
+])
+@pytest.mark.parametrize("how", ["load", "unaligned", "prefill"])
+def test_prefix_store_bit_exact(d, length, s, how):
+    # Positions [0, length) of K and V in the slot and nothing else, whatever way they come: the
+    # copy kernel alone, pitched copies for tensors off the 16-byte grid, or the copy kernel behind
+    # the prefill that reads the same tensors.
+    import torch
+
+    import paper_2406_09297_gb300 as mlkv
+    owner, b, h, g = [0, 0, 2], 3, 4, 2
+    with mlkv.MLKVCache(len(owner), h, d, owner, g, b, s) as c:
+        m, slot = oracle.slots(owner)
+        expect = np.zeros((m, 2, b, g, s, d), dtype=np.int16)
+        kv = [gen.gen_kv(10, 2, i, b, g, length, d) for i in range(2)]
+        for i in range(2):
+            expect[slot[2], i, :, :, :length] = kv[i].view(np.int16)
+        if how == "unaligned":
+            dev = []
+            for x in kv:
+                t = torch.empty(x.size + 1, dtype=torch.bfloat16, device="cuda")
+                t[1:] = to_dev(x).reshape(-1)
+                dev.append(t[1:])
+            c.load_prefix(2, dev[0], dev[1], length)
+        elif how == "load":
+            c.load_prefix(2, to_dev(kv[0]), to_dev(kv[1]), length)
+        else:
+            q = torch.zeros((b, length, h, d), dtype=torch.bfloat16, device="cuda")
+            lens = [length, 1 + length // 2, 1]   # positions past a prompt are stored too
+            c.prefill(2, q, to_dev(kv[0]), to_dev(kv[1]), torch.empty_like(q), lens)
+        np.testing.assert_array_equal(_read_cache(c, b, g, s, d), expect)
+        c.sync_status()
+
+
 def test_device_generator_matches_host_bits():
     import torch
 
