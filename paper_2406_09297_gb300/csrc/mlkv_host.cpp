@@ -351,7 +351,7 @@ int mlkv_cache_create(mlkv_cache_t *out, int n_layers, int n_q_heads, int head_d
 
     for (int vi = 0; vi < 6; ++vi) {
         const int T = 64 << (vi % 3);
-        const mlkv::DecodeVariant *v = mlkv::find_decode_variant(c->d, T, vi / 3);
+        const mlkv::DecodeVariant *v = mlkv::find_decode_variant(c->d, T, vi / 3, c->G);
         if (v == nullptr)
             continue;
         e = mlkv::prepare_decode_variant(*v, c->max_smem);
@@ -556,7 +556,7 @@ static int decode_impl(mlkv_cache_t c, int layer, const void *K_new, const void 
     // be better for a small layer: whole segments per CTA (no merge at all), or each segment in k
     // equal pieces run as one k-CTA cluster and merged over DSMEM.  They are chosen with a cost
     // model in units of one tile's consumer work (~0.5 us on GB300 when the tile is in L2):
-    // a DSMEM cluster merge costs ~2 tiles, the last-CTA merge of up to 8 partial records ~6 (a
+    // a DSMEM cluster merge costs ~2 tiles, the last-CTA merge of partial records ~6 (a
     // global write, an atomic and the reads, after the previous layer has finished) and the
     // separate combine launch ~7.
     const long long wave = std::min<long long>(
@@ -599,7 +599,7 @@ static int decode_impl(mlkv_cache_t c, int layer, const void *K_new, const void 
             const long long S = static_cast<long long>(c->b) * c->g;
             const long long per = tiles / grid;
             const long long pieces = per > 0 ? (nt - 1 + per - 1) / per + 1 : grid;
-            long long best = per_wave + (pieces <= 1 ? 0 : pieces <= mlkv::kInlineMergeMaxPieces ? 6 : 7);
+            long long best = per_wave + (pieces <= 1 ? 0 : pieces <= mlkv::inline_merge_pieces(c->G, c->d) ? 6 : 7);
             if (S <= wave && nt < best) {
                 best = nt;   // whole segments: grid S, each CTA exactly one segment
                 grid = static_cast<int>(S);
@@ -670,7 +670,8 @@ static int decode_impl(mlkv_cache_t c, int layer, const void *K_new, const void 
     // Segments split over many CTAs are merged by a separate parallel kernel: one warp merging
     // dozens of partials would serialise on its loads.
     p.deferred_merge = (cluster_k <= 1 &&
-                        mlkv::max_pieces_per_segment(p, T, grid) > mlkv::kInlineMergeMaxPieces)
+                        mlkv::max_pieces_per_segment(p, T, grid) >
+                            mlkv::inline_merge_pieces(c->G, c->d))
                            ? 1
                            : 0;
 
@@ -2078,7 +2079,7 @@ int mlkv_set_option(mlkv_cache_t c, const char *key, int64_t value)
     if (c == nullptr || key == nullptr)
         return fail(MLKV_ERR_INVALID_ARG, "null argument");
     if (std::strcmp(key, "tile_tokens") == 0) {
-        if (value != 0 && mlkv::find_decode_variant(c->d, static_cast<int>(value)) == nullptr)
+        if (value != 0 && mlkv::find_decode_variant(c->d, static_cast<int>(value), 0, c->G) == nullptr)
             return fail(MLKV_ERR_INVALID_ARG, "tile_tokens %lld not built for d=%d",
                         static_cast<long long>(value), c->d);
         c->tile_tokens = static_cast<int>(value);

@@ -184,7 +184,7 @@ struct DecodeVariant {
     int stages;
     int threads;
     size_t smem_bytes;        // without the per-sequence tables (see table_bytes)
-    size_t res_bytes;         // one piece result slot (cluster mode adds k-1 of them)
+    size_t res_bytes;         // what cluster mode adds k-1 times (0: the slots lie within smem_bytes)
     const void *fn;
     int tc = 0;               // 1: decode_tc_kernel (tcgen05, TMEM), 0: decode_kernel (mma.sync)
 };
@@ -197,8 +197,8 @@ extern const int kNumTcVariants;
 inline size_t table_bytes(int batch) { return ((8 * static_cast<size_t>(batch) + 4) + 15) & ~15ull; }
 
 // Returns the compiled variant for (head_dim, tile_tokens) of the tcgen05 kernel (tc = 1) or of
-// the mma.sync kernel (tc = 0), or nullptr.
-const DecodeVariant *find_decode_variant(int head_dim, int tile_tokens, int tc = 0);
+// the mma.sync kernel (tc = 0; for query groups of `group` heads), or nullptr.
+const DecodeVariant *find_decode_variant(int head_dim, int tile_tokens, int tc, int group);
 
 // Raises the variant's dynamic shared-memory limit (capped at max_smem, the device's opt-in
 // per-block maximum); call once per device before the first launch.
@@ -243,11 +243,16 @@ int max_pieces_per_segment(const DecodeParams &p, int T, int grid);
 cudaError_t launch_combine(const DecodeParams &p, int head_dim, cudaStream_t stream,
                            bool pdl = true);
 
-// Pieces per segment above which the decode launch defers its merges to combine_kernel.  Up to 8
-// the last finisher's merge is one round trip to L2 (every record's loads in flight together); the
-// separate launch costs ~3 us a layer (8 sequences of up to 3000 positions, 8 KV heads of 128, 6
-// pieces at most: 529 -> 505 us for 32 layers when the bound went from 4 to 8).
+// Pieces per segment above which the decode launch defers its merges to combine_kernel, for records
+// of `group` rows of d floats.  A record of at most 512 floats is one pass of the consumer threads,
+// so up to 8 of them are one round trip to L2, against ~3 us a layer for the separate launch (8
+// sequences of up to 3000 positions, 8 KV heads of 128 with 4 heads each, 6 pieces at most: 529 ->
+// 505 us for 32 layers when the bound went from 4 to 8).  Larger records take several passes: 4.
 constexpr int kInlineMergeMaxPieces = 8;
+inline int inline_merge_pieces(int group, int d)
+{
+    return group * d <= 512 ? kInlineMergeMaxPieces : 4;
+}
 // combine_kernel keeps one weight per piece in shared memory.
 constexpr int kCombineMaxPiecesHost = 1024;
 

@@ -41,6 +41,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "mlkv_internal.h"
 
 #include "mlkv_device.cuh"
@@ -52,92 +54,85 @@ namespace {
 // shared-memory plan
 // ------------------------------------------------------------------------------------------------
 
-template <int D, int T, int STAGES, int NCW>
+// kRows: query rows the CTA keeps room for, 16 or (groups of at most 8 heads) 8.
+template <int D, int T, int STAGES, int NCW, bool kT>
 struct Plan {
+    static constexpr int kRows = kT ? 8 : 16;
     static constexpr int kThreads = (NCW + 2) * 32;   // consumers, one producer, one epilogue warp
     // Variants whose ring fits twice in an SM's shared memory are sized for two resident CTAs.
-    static constexpr int kMinBlocks = (STAGES * 2 * T * D * 2 <= 80 * 1024) ? 2 : 1;
+    static constexpr int kMinBlocks = (STAGES * 2 * T * D * 2 <= (kT ? 96 : 80) * 1024) ? 2 : 1;
     static constexpr int kProducer = NCW;             // warp indices
     static constexpr int kEpilogue = NCW + 1;
     static constexpr int kSub = D / 64;               // 128-byte-wide column blocks per row
     static constexpr int kTW = T / NCW;               // positions per warp per tile
     static constexpr int kTileBytes = T * D * 2;      // one K (or V) tile
     static constexpr int kStageBytes = 2 * kTileBytes;
-    static constexpr int kResO = 16 * D * 4;          // a cluster rank's result: o[16][D] f32
+    static constexpr int kResO = kRows * D * 4;       // a cluster rank's result: o[kRows][D] f32
     static constexpr int kResBytes = kResO + 16 * 4 + 32;   // + lse[16] (cluster slots)
-    // A finished piece: every warp's raw sums o[NCW][16][kRawRow] f32 (rows padded so that the
+    // A finished piece: every warp's raw sums o[NCW][kRows][kRawRow] f32 (rows padded so that the
     // fragment stores of a warp's 8 rows fall in distinct banks), its row maxima and sums
     // [2][16][NCW], 8 ints of metadata and, in a cluster's leader, lse[16].
     static constexpr int kRawRow = D + 8;
-    static constexpr int kRawO = NCW * 16 * kRawRow * 4;
+    static constexpr int kRawO = NCW * kRows * kRawRow * 4;
     static constexpr int kRawMeta = kRawO + 2 * 16 * NCW * 4;
     static constexpr int kRawLse = kRawMeta + 32;
     static constexpr int kRawBytes = kRawLse + 64;
-    // Two buffers where shared memory has room for them beside the ring.
-    static constexpr int kRawBufs = (D == 128 && T == 128) ? 2 : 1;
+    // Two buffers where shared memory has room for them beside the ring: the epilogue warp takes
+    // ~1.3 us to merge a piece's warps (64 uneven sequences of up to 2048 positions, 12 heads of 64:
+    // 165 us for 12 layers, 172 with one buffer; 145 once the buffer was freed before the counter).
+    static constexpr int kRawBufs = (!kT && T == 256) ? 1 : 2;
     static constexpr int kRaw = STAGES * kStageBytes;                  // [kRawBufs][kRawBytes]
-    static constexpr int kEpiCap = 512;   // weights of the inline merge, behind a merged piece
-    static constexpr int kFlags = kRaw + kRawBufs * kRawBytes;         // int [4]
+    static constexpr int kEpiW = kRaw + kRawBufs * kRawBytes;   // weights of an inline merge, f32
+    static constexpr int kFlags = kEpiW + kInlineMergeMaxPieces * 16 * 4;   // int [4]
     // u64 full[S], empty[S], res_full[2], res_empty[2], cluster
     static constexpr int kBars = kFlags + 16;
-    // Dynamic tail: per-sequence tables (lengths differ) or, in cluster mode, the leader's
-    // slots for the other ranks' results ([k-1][kResBytes]).
+    // Dynamic tail: per-sequence tables (lengths differ) or, in cluster mode with one raw buffer,
+    // the leader's slots for the other ranks' results ([k-1][kResBytes]).
     // Per-stage query slots: the G rows of the segment whose first tile the stage holds, each row
     // padded by 16 bytes so that the fragment loads (8 rows apart) fall in distinct banks.
     static constexpr int kQRow = D * 2 + 16;
-    static constexpr int kQSlot = 16 * kQRow;
+    static constexpr int kQSlot = kRows * kQRow;
     static constexpr int kQ = (kBars + (2 * STAGES + 5) * 8 + 8 + 127) / 128 * 128;
     static constexpr int kTables = kQ + STAGES * kQSlot;
     static constexpr int kBytes = kTables;
+    // A cluster's CTAs hold one piece each, so the leader's slots can lie in its second raw buffer.
+    static constexpr bool kClusterInRaw = kRawBufs == 2;
+    static constexpr int kCluster = kClusterInRaw ? kRaw + kRawBytes : kTables;
+    static_assert(!kClusterInRaw || 3 * kResBytes <= kRawBytes, "slots of three ranks");
     static constexpr int kAlloc = kBytes + 1024;      // base aligned up to 1024 in the kernel
     static_assert(kTW % 16 == 0, "each warp takes whole 16-position mma steps");
     static_assert(NCW == 4 || NCW == 8, "tree merge over 4 or 8 warps");
     static_assert(D == 64 || D == 128, "head_dim 64 or 128");
     static_assert(T <= 256, "TMA box height");
     static_assert(kResBytes % 16 == 0, "result slots stay 16-byte aligned");
-    static_assert((16 * D + kEpiCap) * 4 <= kRawO, "a merged piece and its weights");
+    static_assert(kMinBlocks * (kAlloc + 1024) <= 228 * 1024, "shared memory of the resident CTAs");
+    static_assert(kRawBufs <= 2, "two pairs of raw-buffer barriers");
     static_assert(kRawBytes % 16 == 0 && kRawMeta % 16 == 0, "raw buffers stay 16-byte aligned");
 };
 
 
-// Query fragments of one (sequence, KV head) group from global memory: the A operand of
-// S = Q K^T in the mma.m16n8k16 layout, rows >= G (the padding of the group to 16 rows) zero.
-template <int D>
-__device__ __forceinline__ void load_q_frag(uint32_t (&qa)[D / 16][4], const DecodeParams &p,
-                                            const __nv_bfloat16 *Q, int beta, int j, int lane)
+// Query fragments of one (sequence, KV head) group, rows of D bf16 `stride` elements apart (global
+// memory, or the group's shared-memory slot); rows >= G are zero.  As the A operand of S = Q K^T in
+// the mma.m16n8k16 layout (16 rows), or, kT, as the B operand of S^T = K Q^T (8 rows).
+template <int D, bool kT>
+__device__ __forceinline__ void load_q_frag(uint32_t (&qf)[D / 16][kT ? 2 : 4],
+                                            const __nv_bfloat16 *qb, int stride, int G, int lane)
 {
-    const int G = p.G;
     const int qr = lane >> 2, qc = (lane & 3) * 2;
-    const __nv_bfloat16 *qb =
-        Q + (static_cast<size_t>(beta) * p.h + static_cast<size_t>(j) * G) * D;
     const bool r0 = qr < G, r1 = qr + 8 < G;
 #pragma unroll
     for (int ks = 0; ks < D / 16; ++ks) {
         const int c = ks * 16 + qc;
-        qa[ks][0] = r0 ? *reinterpret_cast<const uint32_t *>(qb + qr * D + c) : 0u;
-        qa[ks][1] = r1 ? *reinterpret_cast<const uint32_t *>(qb + (qr + 8) * D + c) : 0u;
-        qa[ks][2] = r0 ? *reinterpret_cast<const uint32_t *>(qb + qr * D + c + 8) : 0u;
-        qa[ks][3] = r1 ? *reinterpret_cast<const uint32_t *>(qb + (qr + 8) * D + c + 8) : 0u;
-    }
-}
-
-// Query fragments of one (sequence, KV head) group from its shared-memory slot (16 rows of
-// D bf16, row stride RS elements, rows >= G unused): the A operand of S = Q K^T in the
-// mma.m16n8k16 layout, rows >= G zero.
-template <int D, int RS>
-__device__ __forceinline__ void load_q_frag_smem(uint32_t (&qa)[D / 16][4], const uint8_t *slot,
-                                                 int G, int lane)
-{
-    const int qr = lane >> 2, qc = (lane & 3) * 2;
-    const __nv_bfloat16 *qb = reinterpret_cast<const __nv_bfloat16 *>(slot);
-    const bool r0 = qr < G, r1 = qr + 8 < G;
-#pragma unroll
-    for (int ks = 0; ks < D / 16; ++ks) {
-        const int c = ks * 16 + qc;
-        qa[ks][0] = r0 ? *reinterpret_cast<const uint32_t *>(qb + qr * RS + c) : 0u;
-        qa[ks][1] = r1 ? *reinterpret_cast<const uint32_t *>(qb + (qr + 8) * RS + c) : 0u;
-        qa[ks][2] = r0 ? *reinterpret_cast<const uint32_t *>(qb + qr * RS + c + 8) : 0u;
-        qa[ks][3] = r1 ? *reinterpret_cast<const uint32_t *>(qb + (qr + 8) * RS + c + 8) : 0u;
+        const __nv_bfloat16 *row = qb + qr * stride + c;
+        if constexpr (kT) {
+            qf[ks][0] = r0 ? *reinterpret_cast<const uint32_t *>(row) : 0u;
+            qf[ks][1] = r0 ? *reinterpret_cast<const uint32_t *>(row + 8) : 0u;
+        } else {
+            qf[ks][0] = r0 ? *reinterpret_cast<const uint32_t *>(row) : 0u;
+            qf[ks][1] = r1 ? *reinterpret_cast<const uint32_t *>(row + 8 * stride) : 0u;
+            qf[ks][2] = r0 ? *reinterpret_cast<const uint32_t *>(row + 8) : 0u;
+            qf[ks][3] = r1 ? *reinterpret_cast<const uint32_t *>(row + 8 * stride + 8) : 0u;
+        }
     }
 }
 
@@ -151,18 +146,24 @@ constexpr uint32_t kOnesBf16x2 = 0x3f803f80u;
 // decode kernel
 // ------------------------------------------------------------------------------------------------
 
-template <int D, int T, int STAGES, int NCW>
-__global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
-                                  Plan<D, T, STAGES, NCW>::kMinBlocks)
+// kT: query groups of at most 8 heads.  mma.m16n8k16 pads the group to 16 rows as the A operand, to
+// 8 columns as the B operand: with S^T = K Q^T and O^T += V^T P^T (A = positions, then channels;
+// movmatrix turns P^T's fragments) a tile takes half the MMAs, exponentials and accumulators.
+// Measured on GB300 (layer calls, 16-row form -> this one): 32 layers of 8 uneven sequences, 8 KV
+// heads of 128 with 4 heads each 413 -> 404 us; 12 layers of 128 uneven sequences, 4 KV heads of 64
+// with 3 heads each 602 -> 579 us.
+template <int D, int T, int STAGES, int NCW, bool kT>
+__global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
+                                  Plan<D, T, STAGES, NCW, kT>::kMinBlocks)
     decode_kernel(const __grid_constant__ CUtensorMap tmap,
                   const __grid_constant__ CUtensorMap tmap_rows,
                   const __grid_constant__ DecodeParams p)
 {
-    using PL = Plan<D, T, STAGES, NCW>;
+    using PL = Plan<D, T, STAGES, NCW, kT>;
     constexpr int TW = PL::kTW;
-    constexpr int NT = TW / 8;     // 8-position score tiles per warp
-    constexpr int KS = D / 16;     // 16-wide reduction steps over the head dimension
-    constexpr int NO = D / 8;      // 8-wide output column tiles
+    constexpr int NT = kT ? TW / 16 : TW / 8;   // score tiles per warp (16 or 8 positions)
+    constexpr int KS = D / 16;                  // 16-wide reduction steps over the head dimension
+    constexpr int NO = kT ? D / 16 : D / 8;     // output tiles (16 channels x 8 heads, or 8 x 16)
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>(
@@ -339,9 +340,12 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
     // so this grid finishes only after the previous one, as the next layer's wait expects.
     // The first piece's query fragments come straight from global memory, before the wait when
     // the queries cannot be the previous kernel's output; later pieces find theirs in a slot.
-    uint32_t qa[KS][4];
+    uint32_t qa[KS][kT ? 2 : 4];
+    auto q_rows = [&](int layer, int beta, int j) {
+        return q_of(layer) + (static_cast<size_t>(beta) * p.h + static_cast<size_t>(j) * p.G) * D;
+    };
     if (early && warp < NCW && tile_lo < tile_hi)
-        load_q_frag<D>(qa, p, q_of(wk.layer), wk.beta, wk.j, lane);
+        load_q_frag<D, kT>(qa, q_rows(wk.layer, wk.beta, wk.j), D, p.G, lane);
     if (warp != PL::kProducer && !early)
         grid_dependency_wait();
     if (warp == PL::kEpilogue && lane == 0)
@@ -430,68 +434,157 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
                 break;
             if (early && k == 0)
                 grid_dependency_wait();   // records and merges use the shared scratch
-            if (!flags[0]) {
-                float *raw = reinterpret_cast<float *>(slot);
-                float *st_m = reinterpret_cast<float *>(slot + PL::kRawO);   // [16][NCW]
-                float *st_l = st_m + 16 * NCW;
-                float *rlse = reinterpret_cast<float *>(slot + PL::kRawLse);
-                if (lane < p.G) {
-                    // lane r: row r's factors 2^(m_w - m*) / l* in place of m_w
-                    float mw[NCW], lw[NCW];
+            const int G = p.G;
+            const int seg = meta[kMetaSeg], whole = meta[kMetaWhole];
+            const int c_first = meta[kMetaFirst], c_last = meta[kMetaLast];
+            __nv_bfloat16 *ob =
+                p.out + static_cast<size_t>(meta[kMetaLayer]) * p.ml_q_stride +
+                (static_cast<size_t>(meta[kMetaBeta]) * p.h + static_cast<size_t>(meta[kMetaJ]) * G) * D;
+            // partial record seg + cta; a multi-layer launch's travels in kMetaFirst (its merge is
+            // deferred)
+            const size_t piece = ml ? static_cast<size_t>(c_first) : static_cast<size_t>(seg + cta);
+            const bool stop = flags[0] != 0;
+            const float *raw = reinterpret_cast<const float *>(slot);
+            float *st_m = reinterpret_cast<float *>(slot + PL::kRawO);   // [16][NCW]
+            const float *st_l = st_m + 16 * NCW;
+            if (lane < G) {
+                // lane r: row r's factors 2^(m_w - m*) / l* in place of m_w
+                float mw[NCW], lw[NCW];
 #pragma unroll
-                    for (int w = 0; w < NCW; ++w) {
-                        mw[w] = st_m[lane * NCW + w];
-                        lw[w] = st_l[lane * NCW + w];
-                    }
-                    float ms = mw[0];
-#pragma unroll
-                    for (int w = 1; w < NCW; ++w)
-                        ms = fmaxf(ms, mw[w]);   // finite: the piece holds a visible position
-                    float ls = 0.f;
-#pragma unroll
-                    for (int w = 0; w < NCW; ++w) {
-                        mw[w] = fast_exp2(mw[w] - ms);
-                        ls = fmaf(lw[w], mw[w], ls);
-                    }
-                    const float inv = fast_rcp(ls);
-#pragma unroll
-                    for (int w = 0; w < NCW; ++w)
-                        st_m[lane * NCW + w] = mw[w] * inv;
-                    rlse[lane] = ms + fast_log2(ls);
+                for (int w = 0; w < NCW; ++w) {
+                    mw[w] = st_m[lane * NCW + w];
+                    lw[w] = st_l[lane * NCW + w];
                 }
-                __syncwarp();
-                // Compact result [G][D] over warp 0's rows: row r ends before raw row r + 1 starts.
-                constexpr int E = D / 32;   // columns per lane
-                for (int r = 0; r < p.G; ++r) {
-                    float f[NCW], v[E];
+                float ms = mw[0];
 #pragma unroll
-                    for (int w = 0; w < NCW; ++w)
-                        f[w] = st_m[r * NCW + w];
+                for (int w = 1; w < NCW; ++w)
+                    ms = fmaxf(ms, mw[w]);   // finite: the piece holds a visible position
+                float ls = 0.f;
+#pragma unroll
+                for (int w = 0; w < NCW; ++w) {
+                    mw[w] = fast_exp2(mw[w] - ms);
+                    ls = fmaf(lw[w], mw[w], ls);
+                }
+                const float inv = fast_rcp(ls);
+#pragma unroll
+                for (int w = 0; w < NCW; ++w)
+                    st_m[lane * NCW + w] = mw[w] * inv;
+                if (!whole && !stop)
+                    p.part_lse[piece * G + lane] = ms + fast_log2(ls);
+            }
+            __syncwarp();
+            constexpr int E = D / 32;   // a lane's columns lane E .. lane E + E - 1 of every row
+            using Vec = typename std::conditional<E == 2, float2, float4>::type;
+            auto store_out = [&](int r, const float (&x)[E]) {
+                if constexpr (E == 2)
+                    *reinterpret_cast<uint32_t *>(ob + r * D + lane * E) = pack_bf16x2(x[0], x[1]);
+                else
+                    *reinterpret_cast<uint2 *>(ob + r * D + lane * E) =
+                        make_uint2(pack_bf16x2(x[0], x[1]), pack_bf16x2(x[2], x[3]));
+            };
+#pragma unroll 4
+            for (int r = 0; r < G; ++r) {
+                alignas(16) float v[E] = {};
+#pragma unroll
+                for (int w = 0; w < NCW; ++w) {
+                    const float f = st_m[r * NCW + w];
+                    const Vec x = *reinterpret_cast<const Vec *>(raw + (w * PL::kRows + r) * FS +
+                                                                 lane * E);
+                    const float *xe = reinterpret_cast<const float *>(&x);
 #pragma unroll
                     for (int e = 0; e < E; ++e)
-                        v[e] = 0.f;
-#pragma unroll
-                    for (int w = 0; w < NCW; ++w) {
-                        const float *src = raw + (w * 16 + r) * FS + lane * E;
-#pragma unroll
-                        for (int e = 0; e < E; e += 2) {
-                            const float2 x = *reinterpret_cast<const float2 *>(src + e);
-                            v[e] = fmaf(f[w], x.x, v[e]);
-                            v[e + 1] = fmaf(f[w], x.y, v[e + 1]);
-                        }
-                    }
-                    __syncwarp();
-#pragma unroll
-                    for (int e = 0; e < E; e += 2)
-                        *reinterpret_cast<float2 *>(raw + r * D + lane * E + e) =
-                            make_float2(v[e], v[e + 1]);
+                        v[e] = fmaf(f, xe[e], v[e]);
                 }
-                __syncwarp();
-                epilogue_piece<D>(p, raw, rlse, meta, raw + 16 * D, PL::kEpiCap, lane, cta);
+                if (whole && !stop) {
+                    store_out(r, v);
+                } else if (!stop) {
+                    *reinterpret_cast<Vec *>(p.part_o + (piece * G + r) * D + lane * E) =
+                        *reinterpret_cast<const Vec *>(v);
+                }
             }
+            // The buffer is free before the counter's round trip and a merge of records.
             __syncwarp();
             if (lane == 0)
                 mbar_arrive(bar_res_empty + 8 * rb);
+            if (whole || stop || p.deferred_merge)
+                continue;
+            unsigned prev = 0;
+            if (lane == 0)
+                prev = atomic_add_acq_rel_gpu(&p.counters[seg], 1u);
+            prev = __shfl_sync(0xffffffffu, prev, 0);
+            __syncwarp();
+            if (prev != static_cast<unsigned>(c_last - c_first))
+                continue;
+            // This CTA finished the segment last: it merges records seg + c_first .. seg + c_last (at
+            // most kInlineMergeMaxPieces), o = sum_c 2^(lse_c - M) o_c / sum_c 2^(lse_c - M), M the
+            // largest lse.
+            float *s_w = reinterpret_cast<float *>(smem + PL::kEpiW);
+            const int np = c_last - c_first + 1;
+            const size_t rec0 = static_cast<size_t>(seg + c_first);
+            for (int i = lane; i < np * G; i += 32)
+                s_w[i] = __ldcg(&p.part_lse[rec0 * G + i]);
+            __syncwarp();
+            if (lane < G) {
+                float mx = s_w[lane];
+                for (int c = 1; c < np; ++c)
+                    mx = fmaxf(mx, s_w[c * G + lane]);
+                float tot = 0.f;
+                for (int c = 0; c < np; ++c) {
+                    const float w = fast_exp2(s_w[c * G + lane] - mx);
+                    s_w[c * G + lane] = w;
+                    tot += w;
+                }
+                const float inv = 1.f / tot;
+                for (int c = 0; c < np; ++c)
+                    s_w[c * G + lane] *= inv;
+            }
+            __syncwarp();
+            // 4 x 4 columns a lane of 4 records in flight at a time (8 records at once: longer code,
+            // fetched cold, 4% slower).
+            const float *base = p.part_o + rec0 * G * D;
+            constexpr int CH = 4;
+            for (int c0 = 4 * lane; c0 < G * D; c0 += 128 * CH) {
+                float4 acc[CH];
+#pragma unroll
+                for (int u = 0; u < CH; ++u)
+                    acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int c = 0; c < np; c += 4) {
+                    float4 x[4][CH];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+#pragma unroll
+                        for (int u = 0; u < CH; ++u) {
+                            const int i = c0 + u * 128;
+                            x[q][u] = (i < G * D && c + q < np)
+                                          ? __ldcg(reinterpret_cast<const float4 *>(
+                                                base + static_cast<size_t>(c + q) * G * D + i))
+                                          : make_float4(0.f, 0.f, 0.f, 0.f);
+                        }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+#pragma unroll
+                        for (int u = 0; u < CH; ++u) {
+                            const int i = c0 + u * 128;
+                            const float w =
+                                (i < G * D && c + q < np) ? s_w[(c + q) * G + i / D] : 0.f;
+                            acc[u].x = fmaf(w, x[q][u].x, acc[u].x);
+                            acc[u].y = fmaf(w, x[q][u].y, acc[u].y);
+                            acc[u].z = fmaf(w, x[q][u].z, acc[u].z);
+                            acc[u].w = fmaf(w, x[q][u].w, acc[u].w);
+                        }
+                }
+#pragma unroll
+                for (int u = 0; u < CH; ++u) {
+                    const int i = c0 + u * 128;
+                    if (i < G * D)
+                        *reinterpret_cast<uint2 *>(ob + i) =
+                            make_uint2(pack_bf16x2(acc[u].x, acc[u].y),
+                                       pack_bf16x2(acc[u].z, acc[u].w));
+                }
+            }
+            __syncwarp();   // s_w may be rewritten
+            if (lane == 0)
+                p.counters[seg] = 0u;
         }
         __syncwarp();
         if (p.cluster_k > 1)
@@ -533,7 +626,7 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
 
         if (tile == tile_lo) {
             if (!early)
-                load_q_frag<D>(qa, p, q_of(layer), beta, j, lane);
+                load_q_frag<D, kT>(qa, q_rows(layer, beta, j), D, G, lane);
         } else {
             // A later piece: its query rows arrive with its first tile (the loop's wait for that
             // tile then returns at once).
@@ -542,7 +635,9 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
                 flags[0] = 1;
                 atomicOr(p.err, kErrWaitFull);
             }
-            load_q_frag_smem<D, PL::kQRow / 2>(qa, smem + PL::kQ + s0 * PL::kQSlot, G, lane);
+            load_q_frag<D, kT>(
+                qa, reinterpret_cast<const __nv_bfloat16 *>(smem + PL::kQ + s0 * PL::kQSlot),
+                PL::kQRow / 2, G, lane);
         }
 
         float o[NO][4];
@@ -551,7 +646,9 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
             o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
         float m_run[2] = {NEG_INF, NEG_INF};
         // Row sums of P, accumulated on the tensor core: P times a block of ones (every column
-        // of la holds its row's sum), in fp32 from the same bf16 weights P V uses.
+        // of la holds its row's sum; kT: every row its column's), in fp32 from the same bf16
+        // weights P V uses.  A thread's two statistics (m_run, la) are those of rows qr and qr + 8,
+        // or (kT) of heads qc and qc + 1.
         float la[4] = {0.f, 0.f, 0.f, 0.f};
 
         for (; tile < piece_end; ++tile, ++it) {
@@ -615,16 +712,17 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
                 const int mr = lane & 7;    // which row of it
                 // The K fragments of a group of up to 8 shared-memory loads go out together and
                 // the MMAs follow, so the loads' latency (~47 cycles each) is paid once per group.
-                constexpr int KG = (KS * (NT / 2) <= 8) ? KS : (8 / (NT / 2) > 0 ? 8 / (NT / 2) : 1);
+                constexpr int KL = kT ? NT : NT / 2;   // loads per reduction step
+                constexpr int KG = (KS * KL <= 8) ? KS : (8 / KL > 0 ? 8 / KL : 1);
 #pragma unroll
                 for (int k0 = 0; k0 < KS; k0 += KG) {
-                    uint32_t kf[KG][NT / 2][4];
+                    uint32_t kf[KG][KL][4];
 #pragma unroll
                     for (int kg = 0; kg < KG; ++kg) {
 #pragma unroll
-                        for (int n2 = 0; n2 < NT / 2; ++n2) {
-                            const int row = row0 + 8 * (2 * n2 + (mi >> 1)) + mr;
-                            const int chunk = 2 * (k0 + kg) + (mi & 1);
+                        for (int n2 = 0; n2 < KL; ++n2) {
+                            const int row = row0 + 16 * n2 + 8 * (kT ? (mi & 1) : (mi >> 1)) + mr;
+                            const int chunk = 2 * (k0 + kg) + (kT ? (mi >> 1) : (mi & 1));
                             ldsm_x4(kt + swz<T>(row, chunk), kf[kg][n2][0], kf[kg][n2][1],
                                     kf[kg][n2][2], kf[kg][n2][3]);
                         }
@@ -632,28 +730,34 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
 #pragma unroll
                     for (int kg = 0; kg < KG; ++kg) {
 #pragma unroll
-                        for (int n2 = 0; n2 < NT / 2; ++n2) {
-                            mma_bf16_16816(sc[2 * n2], qa[k0 + kg], kf[kg][n2][0], kf[kg][n2][1]);
-                            mma_bf16_16816(sc[2 * n2 + 1], qa[k0 + kg], kf[kg][n2][2],
-                                           kf[kg][n2][3]);
+                        for (int n2 = 0; n2 < KL; ++n2) {
+                            if constexpr (kT) {
+                                mma_bf16_16816(sc[n2], kf[kg][n2], qa[k0 + kg][0], qa[k0 + kg][1]);
+                            } else {
+                                mma_bf16_16816(sc[2 * n2], qa[k0 + kg], kf[kg][n2][0],
+                                               kf[kg][n2][1]);
+                                mma_bf16_16816(sc[2 * n2 + 1], qa[k0 + kg], kf[kg][n2][2],
+                                               kf[kg][n2][3]);
+                            }
                         }
                     }
                 }
                 // The V fragments of the first group of P V (up to 8 loads) go out now: their
                 // latency overlaps the softmax below.
-                constexpr int VQ = NO / 2;                         // loads per 16 positions
-                constexpr int VG = (VQ * (NT / 2) <= 8) ? NT / 2 : (8 / VQ > 0 ? 8 / VQ : 1);
+                constexpr int NG = kT ? NT : NT / 2;               // groups of 16 positions
+                constexpr int VQ = kT ? NO : NO / 2;               // loads per 16 positions
+                constexpr int VG = (VQ * NG <= 8) ? NG : (8 / VQ > 0 ? 8 / VQ : 1);
+                auto load_v = [&](int grp, int q, uint32_t (&f)[4]) {
+                    const int row = row0 + 16 * grp + 8 * (kT ? (mi >> 1) : (mi & 1)) + mr;
+                    const int chunk = 2 * q + (kT ? (mi & 1) : (mi >> 1));
+                    ldsm_x4_trans(vt + swz<T>(row, chunk), f[0], f[1], f[2], f[3]);
+                };
                 uint32_t vf[VG][VQ][4];
 #pragma unroll
-                for (int kg = 0; kg < VG; ++kg) {
+                for (int kg = 0; kg < VG; ++kg)
 #pragma unroll
-                    for (int q = 0; q < VQ; ++q) {
-                        const int row = row0 + 16 * kg + 8 * (mi & 1) + mr;
-                        const int chunk = 2 * q + (mi >> 1);
-                        ldsm_x4_trans(vt + swz<T>(row, chunk), vf[kg][q][0], vf[kg][q][1],
-                                      vf[kg][q][2], vf[kg][q][3]);
-                    }
-                }
+                    for (int q = 0; q < VQ; ++q)
+                        load_v(kg, q, vf[kg][q]);
 
                 // ---- online softmax (base 2, scale folded into the exponent) ----
                 float mx[2] = {NEG_INF, NEG_INF};
@@ -662,7 +766,8 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
                     for (int n = 0; n < NT; ++n) {
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
-                            const int pos_in_slice = 8 * n + qc + (c & 1);
+                            const int pos_in_slice =
+                                kT ? 16 * n + qr + 8 * (c >> 1) : 8 * n + qc + (c & 1);
                             if (pos_in_slice >= valid)
                                 sc[n][c] = NEG_INF;
                         }
@@ -670,8 +775,8 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
                 }
 #pragma unroll
                 for (int n = 0; n < NT; ++n) {
-                    mx[0] = fmaxf(mx[0], fmaxf(sc[n][0], sc[n][1]));
-                    mx[1] = fmaxf(mx[1], fmaxf(sc[n][2], sc[n][3]));
+                    mx[0] = fmaxf(mx[0], fmaxf(sc[n][0], sc[n][kT ? 2 : 1]));
+                    mx[1] = fmaxf(mx[1], fmaxf(sc[n][kT ? 1 : 2], sc[n][3]));
                 }
                 // The reference maximum moves only when a score exceeds it by more than 2^8 (in
                 // the exponent): weights then stay in [0, 256], exactly as accurate in bf16, and
@@ -683,8 +788,14 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
                     float alpha[2];
 #pragma unroll
                     for (int hr = 0; hr < 2; ++hr) {
-                        mx[hr] = fmaxf(mx[hr], __shfl_xor_sync(0xffffffffu, mx[hr], 1));
-                        mx[hr] = fmaxf(mx[hr], __shfl_xor_sync(0xffffffffu, mx[hr], 2));
+                        if constexpr (kT) {
+                            mx[hr] = fmaxf(mx[hr], __shfl_xor_sync(0xffffffffu, mx[hr], 4));
+                            mx[hr] = fmaxf(mx[hr], __shfl_xor_sync(0xffffffffu, mx[hr], 8));
+                            mx[hr] = fmaxf(mx[hr], __shfl_xor_sync(0xffffffffu, mx[hr], 16));
+                        } else {
+                            mx[hr] = fmaxf(mx[hr], __shfl_xor_sync(0xffffffffu, mx[hr], 1));
+                            mx[hr] = fmaxf(mx[hr], __shfl_xor_sync(0xffffffffu, mx[hr], 2));
+                        }
                         const float m_new = fmaxf(m_run[hr], mx[hr] * scale);
                         alpha[hr] = (m_new == NEG_INF) ? 1.f : fast_exp2(m_run[hr] - m_new);
                         m_run[hr] = m_new;
@@ -692,63 +803,67 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
 #pragma unroll
                     for (int n = 0; n < NO; ++n) {
                         o[n][0] *= alpha[0];
-                        o[n][1] *= alpha[0];
-                        o[n][2] *= alpha[1];
+                        o[n][1] *= alpha[kT ? 1 : 0];
+                        o[n][2] *= alpha[kT ? 0 : 1];
                         o[n][3] *= alpha[1];
                     }
                     la[0] *= alpha[0];
-                    la[1] *= alpha[0];
-                    la[2] *= alpha[1];
+                    la[1] *= alpha[kT ? 1 : 0];
+                    la[2] *= alpha[kT ? 0 : 1];
                     la[3] *= alpha[1];
                 }
                 const float m_use[2] = {m_run[0] == NEG_INF ? 0.f : m_run[0],
                                         m_run[1] == NEG_INF ? 0.f : m_run[1]};
-                // P in bf16 (the mma A operand).
-                uint32_t pa[NT / 2][4];
+                // P in bf16: the mma A operand, or (kT) P^T as the B operand, its 8 x 8 blocks
+                // turned from [position][head] pairs to position pairs of one head.
+                uint32_t pa[NG][kT ? 2 : 4];
 #pragma unroll
                 for (int n = 0; n < NT; ++n) {
                     const float p0 = fast_exp2(fmaf(sc[n][0], scale, -m_use[0]));
-                    const float p1 = fast_exp2(fmaf(sc[n][1], scale, -m_use[0]));
-                    const float p2 = fast_exp2(fmaf(sc[n][2], scale, -m_use[1]));
+                    const float p1 = fast_exp2(fmaf(sc[n][1], scale, -m_use[kT ? 1 : 0]));
+                    const float p2 = fast_exp2(fmaf(sc[n][2], scale, -m_use[kT ? 0 : 1]));
                     const float p3 = fast_exp2(fmaf(sc[n][3], scale, -m_use[1]));
-                    pa[n >> 1][(n & 1) * 2 + 0] = pack_bf16x2(p0, p1);
-                    pa[n >> 1][(n & 1) * 2 + 1] = pack_bf16x2(p2, p3);
+                    if constexpr (kT) {
+                        pa[n][0] = movmatrix_trans(pack_bf16x2(p0, p1));
+                        pa[n][1] = movmatrix_trans(pack_bf16x2(p2, p3));
+                    } else {
+                        pa[n >> 1][(n & 1) * 2 + 0] = pack_bf16x2(p0, p1);
+                        pa[n >> 1][(n & 1) * 2 + 1] = pack_bf16x2(p2, p3);
+                    }
                 }
 
                 // ---- O += P V ----
-#pragma unroll
-                for (int kg = 0; kg < VG; ++kg) {
+                const uint32_t ones[4] = {kOnesBf16x2, kOnesBf16x2, kOnesBf16x2, kOnesBf16x2};
+                auto add_pv = [&](int grp, const uint32_t (&f)[VQ][4]) {
 #pragma unroll
                     for (int q = 0; q < VQ; ++q) {
-                        mma_bf16_16816(o[2 * q], pa[kg], vf[kg][q][0], vf[kg][q][1]);
-                        mma_bf16_16816(o[2 * q + 1], pa[kg], vf[kg][q][2], vf[kg][q][3]);
+                        if constexpr (kT) {
+                            mma_bf16_16816(o[q], f[q], pa[grp][0], pa[grp][1]);
+                        } else {
+                            mma_bf16_16816(o[2 * q], pa[grp], f[q][0], f[q][1]);
+                            mma_bf16_16816(o[2 * q + 1], pa[grp], f[q][2], f[q][3]);
+                        }
                     }
-                    mma_bf16_16816(la, pa[kg], kOnesBf16x2, kOnesBf16x2);
-                }
+                    if constexpr (kT)
+                        mma_bf16_16816(la, ones, pa[grp][0], pa[grp][1]);
+                    else
+                        mma_bf16_16816(la, pa[grp], kOnesBf16x2, kOnesBf16x2);
+                };
+#pragma unroll
+                for (int kg = 0; kg < VG; ++kg)
+                    add_pv(kg, vf[kg]);
                 // the remaining 16-position groups (longer tiles), a group's loads first
 #pragma unroll
-                for (int k0 = VG; k0 < NT / 2; k0 += VG) {
+                for (int k0 = VG; k0 < NG; k0 += VG) {
                     uint32_t vg[VG][VQ][4];
 #pragma unroll
-                    for (int kg = 0; kg < VG; ++kg) {
+                    for (int kg = 0; kg < VG; ++kg)
 #pragma unroll
-                        for (int q = 0; q < VQ; ++q) {
-                            const int row = row0 + 16 * (k0 + kg) + 8 * (mi & 1) + mr;
-                            const int chunk = 2 * q + (mi >> 1);
-                            ldsm_x4_trans(vt + swz<T>(row, chunk), vg[kg][q][0], vg[kg][q][1],
-                                          vg[kg][q][2], vg[kg][q][3]);
-                        }
-                    }
+                        for (int q = 0; q < VQ; ++q)
+                            load_v(k0 + kg, q, vg[kg][q]);
 #pragma unroll
-                    for (int kg = 0; kg < VG; ++kg) {
-#pragma unroll
-                        for (int q = 0; q < VQ; ++q) {
-                            mma_bf16_16816(o[2 * q], pa[k0 + kg], vg[kg][q][0], vg[kg][q][1]);
-                            mma_bf16_16816(o[2 * q + 1], pa[k0 + kg], vg[kg][q][2],
-                                           vg[kg][q][3]);
-                        }
-                        mma_bf16_16816(la, pa[k0 + kg], kOnesBf16x2, kOnesBf16x2);
-                    }
+                    for (int kg = 0; kg < VG; ++kg)
+                        add_pv(k0 + kg, vg[kg]);
                 }
             }
             __syncwarp();
@@ -769,21 +884,28 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
             flags[0] = 1;
             atomicOr(p.err, kErrWaitEmpty);
         }
-        float *fbuf = reinterpret_cast<float *>(slot_raw);                       // [NCW][16][FS]
+        float *fbuf = reinterpret_cast<float *>(slot_raw);                       // [NCW][kRows][FS]
         float *red_m = reinterpret_cast<float *>(slot_raw + PL::kRawO);          // [16][NCW]
         float *red_l = red_m + 16 * NCW;
         float *flse = reinterpret_cast<float *>(slot_raw + PL::kRawLse);         // [16]
 #pragma unroll
         for (int hr = 0; hr < 2; ++hr) {
-            const int row = qr + 8 * hr;
+            const int row = kT ? qc + hr : qr + 8 * hr;
             if (row < G) {
+                float *dst = fbuf + (warp * PL::kRows + row) * FS;
 #pragma unroll
-                for (int n = 0; n < NO; ++n)
-                    *reinterpret_cast<float2 *>(fbuf + (warp * 16 + row) * FS + n * 8 + qc) =
-                        make_float2(o[n][2 * hr], o[n][2 * hr + 1]);
-                if (qc == 0) {
+                for (int n = 0; n < NO; ++n) {
+                    if constexpr (kT) {
+                        dst[n * 16 + qr] = o[n][hr];
+                        dst[n * 16 + 8 + qr] = o[n][2 + hr];
+                    } else {
+                        *reinterpret_cast<float2 *>(dst + n * 8 + qc) =
+                            make_float2(o[n][2 * hr], o[n][2 * hr + 1]);
+                    }
+                }
+                if (kT ? qr == 0 : qc == 0) {
                     red_m[row * NCW + warp] = m_run[hr];
-                    red_l[row * NCW + warp] = la[2 * hr];
+                    red_l[row * NCW + warp] = la[kT ? hr : 2 * hr];
                 }
             }
         }
@@ -816,14 +938,17 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
             __nv_bfloat16 *ob = p.out + static_cast<size_t>(layer) * p.ml_q_stride +
                                 (static_cast<size_t>(beta) * p.h + static_cast<size_t>(j) * G) * D;
             constexpr int kPass = 4 * NCW * 32;   // outputs per pass
+            // One or two passes (groups of at most 8 heads, or head_dim 64) take the shorter code,
+            // which is fetched cold once a launch; up to four overlap in pairs.
+            constexpr int kPassUnroll = (!kT && D == 128) ? 2 : 1;
             static_assert(D % 4 == 0, "a thread's four columns lie in one row");
             // mode: 0 whole, 1 cluster sender, 2 cluster leader, 3 partial record
             const int rank = p.cluster_k > 1 ? static_cast<int>(cluster_ctarank()) : 0;
             const int mode = whole ? 0 : (p.cluster_k > 1 ? (rank != 0 ? 1 : 2) : 3);
             if (early && mode == 3)
                 grid_dependency_wait();   // partial records and counters are shared scratch
-            const uint32_t cslots = sbase + PL::kTables;
-            const uint8_t *cs = smem + PL::kTables;
+            const uint32_t cslots = sbase + PL::kCluster;
+            const uint8_t *cs = smem + PL::kCluster;
             uint32_t remote = 0, remote_bar = 0;
             if (mode == 1) {
                 remote = map_to_rank(cslots + (rank - 1) * PL::kResBytes, 0);
@@ -831,7 +956,7 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
             }
             const size_t piece = ml ? static_cast<size_t>(rec) : static_cast<size_t>(seg + cta);
             float *po = p.part_o + piece * G * D;
-#pragma unroll 2
+#pragma unroll kPassUnroll
             for (int i = 4 * ctid; i < G * D; i += kPass) {
                 const int row = i / D, e = i - row * D;
                 // independent loads of the row's statistics of every warp
@@ -852,7 +977,7 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
                     const float ew = fast_exp2(mw[w] - ms);
                     ls = fmaf(lw[w], ew, ls);
                     const float4 x =
-                        *reinterpret_cast<const float4 *>(fbuf + (w * 16 + row) * FS + e);
+                        *reinterpret_cast<const float4 *>(fbuf + (w * PL::kRows + row) * FS + e);
                     v.x = fmaf(ew, x.x, v.x);
                     v.y = fmaf(ew, x.y, v.y);
                     v.z = fmaf(ew, x.z, v.z);
@@ -915,7 +1040,7 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW>::kThreads,
                 consumer_bar_sync<NCW>();   // flse is complete
                 const int k = p.cluster_k;   // 2 or 4
                 const bool stop = flags[0] != 0;
-#pragma unroll 2
+#pragma unroll kPassUnroll
                 for (int i = 4 * ctid; i < G * D; i += kPass) {
                     const int row = i / D, e = i - row * D;
                     float lr[4];
@@ -1155,28 +1280,30 @@ __global__ void append_kernel(const __grid_constant__ AppendParams p)
     *dst = *src;
 }
 
-template <int D, int T, int STAGES, int NCW>
+template <int D, int T, int STAGES, int NCW, bool kT>
 constexpr DecodeVariant make_variant()
 {
-    using PL = Plan<D, T, STAGES, NCW>;
+    using PL = Plan<D, T, STAGES, NCW, kT>;
     return DecodeVariant{D, T, STAGES, PL::kThreads, static_cast<size_t>(PL::kAlloc),
-                         static_cast<size_t>(PL::kResBytes),
-                         reinterpret_cast<const void *>(&decode_kernel<D, T, STAGES, NCW>)};
+                         PL::kClusterInRaw ? 0 : static_cast<size_t>(PL::kResBytes),
+                         reinterpret_cast<const void *>(&decode_kernel<D, T, STAGES, NCW, kT>)};
 }
 
-// (head_dim, positions per tile, ring stages, consumer warps); the first match of a
-// (head_dim, tile) pair is used.  <64, 128, 2, 4> fits twice on an SM (90 KB, 167 registers).
-const DecodeVariant kVariants[] = {
-    make_variant<64, 128, 2, 4>(),
-    make_variant<64, 256, 3, 4>(),
-    make_variant<64, 64, 4, 4>(),
-    make_variant<128, 64, 5, 4>(),
-    make_variant<128, 128, 2, 4>(),
+// (head_dim, positions per tile, ring stages, consumer warps) for groups of more than 8 heads, and
+// for those of at most 8; the first match of a (head_dim, tile) pair is used.  <64, 128, 2, 4> fits
+// twice on an SM (90 KB, 163 registers).
+const DecodeVariant kVariants[2][5] = {
+    {make_variant<64, 128, 2, 4, false>(), make_variant<64, 256, 3, 4, false>(),
+     make_variant<64, 64, 4, 4, false>(), make_variant<128, 64, 4, 4, false>(),
+     make_variant<128, 128, 2, 4, false>()},
+    {make_variant<64, 128, 2, 4, true>(), make_variant<64, 256, 3, 4, true>(),
+     make_variant<64, 64, 4, 4, true>(), make_variant<128, 64, 5, 4, true>(),
+     make_variant<128, 128, 2, 4, true>()},
 };
 
 }  // namespace
 
-const DecodeVariant *find_decode_variant(int head_dim, int tile_tokens, int tc)
+const DecodeVariant *find_decode_variant(int head_dim, int tile_tokens, int tc, int group)
 {
     if (tc) {
         for (int i = 0; i < kNumTcVariants; ++i)
@@ -1184,7 +1311,7 @@ const DecodeVariant *find_decode_variant(int head_dim, int tile_tokens, int tc)
                 return &kTcVariants[i];
         return nullptr;
     }
-    for (const DecodeVariant &v : kVariants)
+    for (const DecodeVariant &v : kVariants[group <= 8 ? 1 : 0])
         if (v.head_dim == head_dim && v.tile_tokens == tile_tokens)
             return &v;
     return nullptr;

@@ -92,14 +92,16 @@ void setup_device(int dev, DeviceSetup &st)
         return;
     }
     for (int d : {64, 128})
-        for (int T : {64, 128, 256}) {
-            const mlkv::DecodeVariant *v = mlkv::find_decode_variant(d, T);
-            if (v != nullptr && (e = mlkv::prepare_decode_variant(*v, st.max_smem)) != cudaSuccess) {
-                st.status = MLKV_ERR_CUDA;
-                st.error = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e);
-                return;
+        for (int T : {64, 128, 256})
+            for (int group : {1, MLKV_MAX_GROUP}) {   // either kernel of a (head_dim, tile) pair
+                const mlkv::DecodeVariant *v = mlkv::find_decode_variant(d, T, 0, group);
+                if (v != nullptr &&
+                    (e = mlkv::prepare_decode_variant(*v, st.max_smem)) != cudaSuccess) {
+                    st.status = MLKV_ERR_CUDA;
+                    st.error = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e);
+                    return;
+                }
             }
-        }
 }
 
 }  // namespace
@@ -155,12 +157,12 @@ extern "C" int mlkv_decode_attention_static(const void *kv_slot, int batch, int 
     // batch * kv_heads segments); 64 when the per-sequence tables do not fit beside the ring.
     const double mean_len = static_cast<double>(len_sum) / batch;
     int T = mlkv::default_tile_tokens(head_dim, mean_len, batch * kv_heads);
-    const mlkv::DecodeVariant *v = mlkv::find_decode_variant(head_dim, T);
+    const mlkv::DecodeVariant *v = mlkv::find_decode_variant(head_dim, T, 0, G);
     if (v == nullptr)
         return fail(MLKV_ERR_UNSUPPORTED, "no decode variant");
     if (!uniform && v->smem_bytes + mlkv::table_bytes(batch) > st.max_smem) {
         T = 64;
-        v = mlkv::find_decode_variant(head_dim, T);
+        v = mlkv::find_decode_variant(head_dim, T, 0, G);
         if (v == nullptr || v->smem_bytes + mlkv::table_bytes(batch) > st.max_smem)
             return fail(MLKV_ERR_UNSUPPORTED, "batch too large for varied lengths");
     }
@@ -265,7 +267,7 @@ extern "C" int mlkv_decode_attention_static(const void *kv_slot, int batch, int 
     p.ml_kv_stride = 0;
     p.Q_next = nullptr;
     p.deferred_merge =
-        mlkv::max_pieces_per_segment(p, T, grid) > mlkv::kInlineMergeMaxPieces ? 1 : 0;
+        mlkv::max_pieces_per_segment(p, T, grid) > mlkv::inline_merge_pieces(G, head_dim) ? 1 : 0;
     const size_t smem = v->smem_bytes + (uniform ? 0 : mlkv::table_bytes(batch));
     e = mlkv::launch_decode(*v, grid, smem, stream, &tmap, &tmap_rows, p, nullptr);
     if (e != cudaSuccess)

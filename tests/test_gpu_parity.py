@@ -221,3 +221,15 @@ def test_many_pieces_a_cta(d, tile, h, g):
     lens = [1 + (i * 53) % (2 * tile) for i in range(37)]
     run_small_case([0, 0], h, g, d, len(lens), lens, 2 * tile, seed=32, fused=True,
                    options={"grid": 3, "tile_tokens": tile})
+
+
+@pytest.mark.parametrize("d,tile", [(64, 64), (64, 128), (64, 256), (128, 64), (128, 128)])
+@pytest.mark.parametrize("G", [1, 2, 7, 8, 9])
+def test_group_sizes_around_eight(d, tile, G):
+    # Groups of at most 8 heads take the kernel that holds them as the MMAs' 8 columns, larger ones
+    # the 16-row kernel; whole, cut and ragged segments, new tokens in the tiles.
+    lens = [1, 17, tile - 1, tile, tile + 1, 3 * tile - 7]
+    run_small_case([0, 0], 2 * G, 2, d, len(lens), lens, 3 * tile, seed=33, fused=True,
+                   options={"grid": 7, "tile_tokens": tile})
+    run_small_case([0], 2 * G, 2, d, 2, [2 * tile, 2 * tile], 2 * tile, seed=34,
+                   options={"tile_tokens": tile})
