@@ -337,31 +337,24 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
         bool waited = !early;
         int idx = 0;   // ring tiles sent so far: K_0, V_0, K_1, V_1, ... over all units
         int uc = 0;    // units whose queries were sent
-        auto agreed = [&](int ok) { return __shfl_sync(0xffffffffu, ok, 0) != 0; };
         // Ring tile k of unit x (K of key tile k / 2 if k is even, else V).
         auto send_kv = [&](const Unit &x, int k) {
             const int s = idx % R;
-            int ok = 1;
-            if (lane == 0) {
-                if (idx >= R && !flags[0] &&
-                    !mbar_wait(bar_empty + 8 * s, ((idx / R) & 1) ^ 1)) {
-                    flags[0] = 1;
-                    atomicOr(p.err, kErrWaitEmpty);
-                }
-                ok = !flags[0];
+            if (idx >= R && !flags[0] &&
+                !mbar_wait(bar_empty + 8 * s, ((idx / R) & 1) ^ 1)) {
+                flags[0] = 1;
+                atomicOr(p.err, kErrWaitEmpty);
             }
-            if (!agreed(ok))
+            if (flags[0])
                 return false;
             if (!waited && x.has_end && (k >> 1) == x.n_b - 1) {
                 grid_dependency_wait();   // the tile that holds the new row
                 waited = true;
             }
             const uint32_t fb = bar_full + 8 * s;
-            if (lane == 0)
-                mbar_arrive_expect_tx(fb, PL::kTileBytes);
-            __syncwarp();
-            const int sub = lane - (idx & 7) * 2;   // the lanes take turns
-            if (sub >= 0 && sub < PL::kSub)
+            mbar_arrive_expect_tx(fb, PL::kTileBytes);
+#pragma unroll
+            for (int sub = 0; sub < PL::kSub; ++sub)
                 tma_load_3d(sbase + PL::kRing + s * PL::kTileBytes + sub * 16384,
                             (k & 1) ? &tmap_v : &tmap_k, fb, sub * 64, ((k >> 1) + x.kt0) * 128,
                             (k & 1) ? x.zv : x.zk);
@@ -374,16 +367,12 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
                 ++uc;   // the last warp reads the queries from host memory
                 return true;
             }
-            int ok = 1;
-            if (lane == 0) {
-                if (uc >= NQ && !flags[0] &&
-                    !mbar_wait(bar_q_free + 8 * qb, ((uc / NQ) & 1) ^ 1)) {
-                    flags[0] = 1;
-                    atomicOr(p.err, kErrWaitEmpty);
-                }
-                ok = !flags[0];
+            if (uc >= NQ && !flags[0] &&
+                !mbar_wait(bar_q_free + 8 * qb, ((uc / NQ) & 1) ^ 1)) {
+                flags[0] = 1;
+                atomicOr(p.err, kErrWaitEmpty);
             }
-            if (!agreed(ok))
+            if (flags[0])
                 return false;
             const uint32_t qbar = bar_q + 8 * qb;
             const uint32_t dst = sbase + PL::kQ + qb * PL::kTiles * PL::kTileBytes;
@@ -393,49 +382,48 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
             // from the block's first layer (tile B) and its layer L1 (tile A)
             const int box_rows =
                 kFused ? (p.fused_L < p.fused_L1 ? p.fused_L : p.fused_L1) * p.G : 128;
-            if (lane == 0)
-                mbar_arrive_expect_tx(qbar, n_tiles * PL::kSub * box_rows * 128);
-            __syncwarp();
-            const int sub = lane & 1, g = 1 - ((lane >> 1) & 1);
-            if (lane < 2 * n_tiles && sub < PL::kSub) {
-                const uint32_t d = dst + slot_of(g) * PL::kTileBytes + sub * 16384;
-                if (kFused)
-                    tma_load_5d(d, &tmap_q, qbar, sub * 64, 0, x.j, x.beta,
-                                x.blk * p.fused_L + (g ? 0 : p.fused_L1));
-                else
-                    tma_load_4d(d, &tmap_q, qbar, sub * 64, g ? x.head_b : x.head_a,
-                                (g ? x.qb_b : x.n_a - 1) * 128, x.beta);
-            }
+            mbar_arrive_expect_tx(qbar, n_tiles * PL::kSub * box_rows * 128);
+            for (int g = 1; g >= 2 - n_tiles; --g)
+#pragma unroll
+                for (int sub = 0; sub < PL::kSub; ++sub) {
+                    const uint32_t d = dst + slot_of(g) * PL::kTileBytes + sub * 16384;
+                    if (kFused)
+                        tma_load_5d(d, &tmap_q, qbar, sub * 64, 0, x.j, x.beta,
+                                    x.blk * p.fused_L + (g ? 0 : p.fused_L1));
+                    else
+                        tma_load_4d(d, &tmap_q, qbar, sub * 64, g ? x.head_b : x.head_a,
+                                    (g ? x.qb_b : x.n_a - 1) * 128, x.beta);
+                }
             ++uc;
             return true;
         };
-        bool ok = true;
-        for (int n = 0; ok; ++n) {
-            const int i = unit_index(p, n);
-            if (i < 0)
-                break;
-            const Unit x = unit_of<kFused, PL::kTiles>(p, i);
-            const int n_idx = 2 * x.n_b;
-            int k = 0;
-            if (n == 0 && early && !q_early) {
-                // mode 2: the cache tiles that hold no new row first, as far as the ring goes
-                const int n_pre = n_idx < R ? n_idx : R;
-                while (ok && k < n_pre && !(x.has_end && (k >> 1) == x.n_b - 1))
-                    ok = send_kv(x, k++);
-                grid_dependency_wait();   // the step's inputs are in place
-                waited = true;
-            }
-            // a later unit's first key tile can go before its queries' slot is free
-            if (n > 0 && NQ == 1)
-                ok = ok && send_kv(x, k++);
-            ok = ok && send_q(x);
-            while (ok && k < n_idx)
-                ok = send_kv(x, k++);
-            if (kSplit)
-                break;   // one unit per CTA
-        }
-        // No copy may still be in flight when the CTA exits.
         if (lane == 0) {
+            bool ok = true;
+            for (int n = 0; ok; ++n) {
+                const int i = unit_index(p, n);
+                if (i < 0)
+                    break;
+                const Unit x = unit_of<kFused, PL::kTiles>(p, i);
+                const int n_idx = 2 * x.n_b;
+                int k = 0;
+                if (n == 0 && early && !q_early) {
+                    // mode 2: the cache tiles that hold no new row first, as far as the ring goes
+                    const int n_pre = n_idx < R ? n_idx : R;
+                    while (ok && k < n_pre && !(x.has_end && (k >> 1) == x.n_b - 1))
+                        ok = send_kv(x, k++);
+                    grid_dependency_wait();   // the step's inputs are in place
+                    waited = true;
+                }
+                // a later unit's first key tile can go before its queries' slot is free
+                if (n > 0 && NQ == 1)
+                    ok = ok && send_kv(x, k++);
+                ok = ok && send_q(x);
+                while (ok && k < n_idx)
+                    ok = send_kv(x, k++);
+                if (kSplit)
+                    break;   // one unit per CTA
+            }
+            // No copy may still be in flight when the CTA exits.
             if (!(kFused && p.q_host != nullptr))
                 for (int k = uc > NQ ? uc - NQ : 0; k < uc; ++k)
                     if (!mbar_wait(bar_q + 8 * (k % NQ), (k / NQ) & 1))
