@@ -915,6 +915,10 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
                 tmem_fence_before();
             }
             if (PL::kStageInQ) {
+                // A warpgroup without a tile in this unit has waited for nothing in it: it must not
+                // run ahead into the barrier's next phase.
+                if (PL::kTiles == 2 && n_g == 0)
+                    wait(bar_q + 8 * qb, n / NQ);
                 // the next queries may be written over the stage
                 fence_proxy_async_smem();
                 __syncwarp();
