@@ -804,7 +804,7 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
                 asm volatile("bar.sync 1, %0;" ::"n"(8 * 32) : "memory");
                 if (wg == 0) {
                     const float2 o1 = ml[r];
-                    if (o1.y > 0.f) {
+                    if (o1.y != 0.f) {   // a NaN sum goes on into the row's output
                         const float mxx = fmaxf(m_run, o1.x);
                         a0 = fast_exp2(m_run - mxx);
                         a1 = fast_exp2(o1.x - mxx);
@@ -816,13 +816,17 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
             // O of this row, 32 columns at c: this warpgroup's buffer, merged with the second's
             auto load_o = [&](int c, float (&ov)[32]) {
                 tmem_ld32_nowait(col_o + c * 32, ov);
-                if (kSplit && a1 > 0.f) {
+                // The load is the whole warp's: its condition must not differ from row to row (a
+                // row's a1 may be 0 or NaN).
+                if (kSplit && n_g > 1) {
                     float o1[32];
                     tmem_ld32_nowait(col_o + D + c * 32, o1);
                     tmem_wait_ld();
+                    if (a1 > 0.f) {
 #pragma unroll
-                    for (int k = 0; k < 32; ++k)
-                        ov[k] = ov[k] * a0 + o1[k] * a1;
+                        for (int k = 0; k < 32; ++k)
+                            ov[k] = ov[k] * a0 + o1[k] * a1;
+                    }
                 } else {
                     tmem_wait_ld();
                 }

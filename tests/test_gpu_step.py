@@ -456,6 +456,42 @@ def test_fused_step(owner, h, g, d, b, L, kc, units, tiles, deep):
         cache.sync_status()
 
 
+@pytest.mark.parametrize("b,L", [(16, 400), (1, 20000)])
+def test_fused_step_uneven_rows(b, L):
+    # The deep form merges two partial results a row, row by row: a query so long that one of the
+    # two weighs 0 (its scores lie further apart than fp32's exponent range), and one holding a NaN,
+    # between ordinary rows.  The NaN stays in its own row, every other output is the clean run's.
+    import torch
+
+    import paper_2406_09297_gb300 as mlkv
+    owner, h, g, d = [0] * 6 + [6] * 6, 12, 1, 64
+    lens = np.full(b, L, dtype=np.int32)
+    with mlkv.MLKVCache(12, h, d, owner, g, b, L) as cache:
+        ref = oracle.OracleCache(owner, h, g, d, b, L)
+        qb, kn, vn = _inputs(owner, h, g, d, b, lens, L, 87, cache, ref)
+        big = (0, 0, [1, 4, 9])
+        qb[big] = gen.f32_to_bf16_bits(gen.bf16_bits_to_f32(qb[big]) * np.float32(1024))
+        Q, K, V = to_dev(qb), to_dev(kn), to_dev(vn)
+        cache.set_option("step_fused", 2)
+        outs = []
+        for nan in (False, True):
+            if nan:
+                Q[1, 0, 5, 7] = float("nan")
+            out = torch.zeros((12, b, h, d), dtype=torch.bfloat16, device="cuda")
+            cache.decode_step(Q, K, V, out, lens)
+            torch.cuda.synchronize()
+            assert cache.get_option("last_step_fused") == 1
+            outs.append(out)
+        ref.append(0, gen.bf16_bits_to_f64(kn[0]), gen.bf16_bits_to_f64(vn[0]), lens)
+        expect = ref.decode(0, gen.bf16_bits_to_f64(qb[0]), lens, nthreads=8)
+        mx, mean = errors(from_dev(outs[0][0]), expect)
+        assert mx <= MAX_ABS and mean <= MEAN_ABS, (mx, mean)
+        assert torch.isnan(outs[1][1, 0, 5]).all()
+        outs[1][1, 0, 5] = outs[0][1, 0, 5]
+        assert torch.equal(outs[1].view(torch.int16), outs[0].view(torch.int16))
+        cache.sync_status()
+
+
 @pytest.mark.parametrize("chunked", [False, True])
 def test_fused_step_host_buffers(chunked):
     # mlkv_decode_step_host in the fused form: the store launch lets the fused launch go at once,
