@@ -521,29 +521,22 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
             float *s_w = reinterpret_cast<float *>(smem + PL::kEpiW);
             const int np = c_last - c_first + 1;
             const size_t rec0 = static_cast<size_t>(seg + c_first);
-            for (int i = lane; i < np * G; i += 32)
-                s_w[i] = __ldcg(&p.part_lse[rec0 * G + i]);
-            __syncwarp();
-            if (lane < G) {
-                float mx = s_w[lane];
-                for (int c = 1; c < np; ++c)
-                    mx = fmaxf(mx, s_w[c * G + lane]);
-                float tot = 0.f;
-                for (int c = 0; c < np; ++c) {
-                    const float w = fast_exp2(s_w[c * G + lane] - mx);
-                    s_w[c * G + lane] = w;
-                    tot += w;
-                }
-                const float inv = 1.f / tot;
-                for (int c = 0; c < np; ++c)
-                    s_w[c * G + lane] *= inv;
-            }
-            __syncwarp();
+            // Lane r: row r's log-sum-exps, in flight with the first records.  (One round trip to L2
+            // after the other, with the weights' chain through shared memory between them, was the
+            // launch's last microsecond: 64 uneven segments over 138 CTAs, 32 heads of 128, 12.7 us a
+            // layer, now 12.1.)
+            float lv[kInlineMergeMaxPieces];
+#pragma unroll
+            for (int c = 0; c < kInlineMergeMaxPieces; ++c)
+                lv[c] = (lane < G && c < np) ? __ldcg(&p.part_lse[(rec0 + c) * G + lane])
+                                             : -__int_as_float(0x7f800000);
+            bool weighed = false;
             // 4 x 4 columns a lane of 4 records in flight at a time (8 records at once: longer code,
             // fetched cold, 4% slower).
             const float *base = p.part_o + rec0 * G * D;
             constexpr int CH = 4;
-            for (int c0 = 4 * lane; c0 < G * D; c0 += 128 * CH) {
+            for (int cb = 0; cb < G * D; cb += 128 * CH) {
+                const int c0 = cb + 4 * lane;
                 float4 acc[CH];
 #pragma unroll
                 for (int u = 0; u < CH; ++u)
@@ -560,6 +553,26 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
                                                 base + static_cast<size_t>(c + q) * G * D + i))
                                           : make_float4(0.f, 0.f, 0.f, 0.f);
                         }
+                    if (!weighed) {
+                        weighed = true;
+                        if (lane < G) {
+                            float mx = lv[0];
+#pragma unroll
+                            for (int k = 1; k < kInlineMergeMaxPieces; ++k)
+                                mx = fmaxf(mx, lv[k]);
+                            float tot = 0.f;
+#pragma unroll
+                            for (int k = 0; k < kInlineMergeMaxPieces; ++k) {
+                                lv[k] = fast_exp2(lv[k] - mx);   // 0 past the records
+                                tot += lv[k];
+                            }
+                            const float inv = 1.f / tot;
+#pragma unroll
+                            for (int k = 0; k < kInlineMergeMaxPieces; ++k)
+                                s_w[k * G + lane] = lv[k] * inv;
+                        }
+                        __syncwarp();
+                    }
 #pragma unroll
                     for (int q = 0; q < 4; ++q)
 #pragma unroll
