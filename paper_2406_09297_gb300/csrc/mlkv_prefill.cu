@@ -1019,14 +1019,16 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
 // Merges the context chunks of the fused decode: per output row (block, sequence, KV head, block
 // layer, group head) o = sum_c 2^(lse_c - M) o_c / sum_c 2^(lse_c - M), M = max_c lse_c.  W warps
 // per row (fused_combine_w: 1, 2, 4 or 8, more for more chunks): warp w takes chunks w, w + W, ...,
-// 4 of them in flight, and each lane keeps a running maximum, sum of weights and weighted sum for
+// 8 of them in flight, and each lane keeps a running maximum, sum of weights and weighted sum for
 // its D / 32 columns; the W warps' states are then merged through shared memory.
+// Bound by latency: a few round trips to L2 behind the end of the decode grid.  The row's divisions
+// run before the wait for it, and up to 64 chunks take one round trip (4 in flight and the
+// divisions behind the wait: a step over 4 sequences of 8,192 tokens 15.2 us, now 12.1; one of
+// 131,072 tokens 27.1, now 24.3; 12 in flight 12.8 and 24.2).
 template <int D>
-__global__ void __launch_bounds__(256, D == 64 ? 6 : 4) combine_fused_kernel(const __grid_constant__ PrefillParams p)
+__global__ void __launch_bounds__(256, D == 64 ? 4 : 3) combine_fused_kernel(const __grid_constant__ PrefillParams p)
 {
-    // Launched while the decode grid still runs: the partials are read after it has finished.
-    grid_dependency_wait();
-    grid_dependents_launch();
+    constexpr int U = 8;        // chunks in flight a warp
     constexpr int E = D / 32;   // columns per lane
     using Vec = typename std::conditional<E == 2, float2, float4>::type;
     __shared__ float s_m[8], s_l[8];
@@ -1047,17 +1049,22 @@ __global__ void __launch_bounds__(256, D == 64 ? 6 : 4) combine_fused_kernel(con
         const long long bb = bj / p.g;
         beta = static_cast<int>(bb % p.b);
         blk = static_cast<int>(bb / p.b);
+        base = static_cast<size_t>(bj) * p.fused_cmax * rows_per_head + rr;
+    }
+    // Launched while the decode grid still runs: the partials are read after it has finished.
+    grid_dependency_wait();
+    grid_dependents_launch();
+    if (live) {
         const int n_kt = (p.prompt_len[beta] + 127) / 128;
         chunks = (n_kt + p.fused_kc - 1) / p.fused_kc;
-        base = static_cast<size_t>(bj) * p.fused_cmax * rows_per_head + rr;
     }
     float m = NEG_INF, l = 0.f;
     float acc[E] = {};
-    for (int c0 = w; c0 < chunks; c0 += 4 * W) {
-        float lse[4];
-        Vec v[4];
+    for (int c0 = w; c0 < chunks; c0 += U * W) {
+        float lse[U];
+        Vec v[U];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < U; ++u) {
             const int c = c0 + u * W;
             const size_t r = base + static_cast<size_t>(c) * rows_per_head;
             if (c < chunks) {
@@ -1068,14 +1075,17 @@ __global__ void __launch_bounds__(256, D == 64 ? 6 : 4) combine_fused_kernel(con
                 v[u] = Vec{};
             }
         }
-        const float mx = fmaxf(fmaxf(m, fmaxf(lse[0], lse[1])), fmaxf(lse[2], lse[3]));
+        float mx = m;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            mx = fmaxf(mx, lse[u]);
         const float scale = m == NEG_INF ? 0.f : exp2f(m - mx);
         l *= scale;
 #pragma unroll
         for (int e = 0; e < E; ++e)
             acc[e] *= scale;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < U; ++u) {
             const float wt = lse[u] == NEG_INF ? 0.f : exp2f(lse[u] - mx);
             l += wt;
             const float *x = reinterpret_cast<const float *>(&v[u]);
