@@ -1831,6 +1831,26 @@ int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const 
         return fail(MLKV_ERR_INVALID_ARG, "K and V must be non-NULL and 16-byte aligned");
     DeviceGuard guard(c->device);
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+    // An owner layer reads the prompt's K/V in place and stores them afterwards, unless the outputs
+    // would overwrite them or the store's target is one of the inputs: then it stores them first.
+    bool direct = owner;
+    if (owner) {
+        const size_t kvbytes = static_cast<size_t>(c->b) * c->g * s_max * c->d * 2;
+        auto overlap = [](const void *a, size_t na, const void *b, size_t nb) {
+            const char *x = static_cast<const char *>(a), *y = static_cast<const char *>(b);
+            return x < y + nb && y < x + na;
+        };
+        for (const void *kv : {K, V})
+            if (overlap(kv, kvbytes, out, qbytes) || overlap(kv, kvbytes, c->cache, c->cache_bytes))
+                direct = false;
+        if (overlap(Q, qbytes, c->cache, c->cache_bytes))
+            direct = false;
+        if (!direct) {
+            const int rc = store_prefix(c, layer, K, V, s_max, stream, false);
+            if (rc != MLKV_OK)
+                return rc;
+        }
+    }
     cudaError_t e;
     if (!c->prefill_ready) {
         if ((e = mlkv::prepare_prefill(c->d)) != cudaSuccess)
@@ -1856,10 +1876,10 @@ int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const 
     if (r != CUDA_SUCCESS)
         return fail(MLKV_ERR_CUDA, "cuTensorMapEncodeTiled(Q) failed (CUresult %d)",
                     static_cast<int>(r));
-    // K and V in boxes of 128 positions: an owner layer's prompt where it is, [b][g][s_max][d]; for
-    // the other layers the cache (the map of the 128-position decode variant).
+    // K and V in boxes of 128 positions: an owner layer's prompt where it is, [b][g][s_max][d]; else
+    // the cache (the map of the 128-position decode variant).
     CUtensorMap tmap_in[2];
-    if (owner) {
+    if (direct) {
         const cuuint64_t kdims[3] = {static_cast<cuuint64_t>(c->d), static_cast<cuuint64_t>(s_max),
                                      static_cast<cuuint64_t>(c->b) * c->g};
         const cuuint64_t kstrides[2] = {static_cast<cuuint64_t>(c->d) * 2,
@@ -1894,10 +1914,10 @@ int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const 
     p.s_max = s_max;
     p.slot = c->slot[layer];
     p.sm_count = c->sm_count;
-    p.kv_direct = owner ? 1 : 0;
+    p.kv_direct = direct ? 1 : 0;
     p.fused_L = p.fused_L1 = 0;
-    const CUtensorMap *tmap_k = owner ? &tmap_in[0] : tmap_kv;
-    const CUtensorMap *tmap_v = owner ? &tmap_in[1] : tmap_kv;
+    const CUtensorMap *tmap_k = direct ? &tmap_in[0] : tmap_kv;
+    const CUtensorMap *tmap_v = direct ? &tmap_in[1] : tmap_kv;
     for (int beta = 0; beta < c->b; ++beta)
         p.prompt_len[beta] = prompt_lens[beta];
     // Work units, those that see the most keys first.  head_dim 64: one query block of one head
@@ -1932,7 +1952,7 @@ int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const 
             return fail_cuda(e, "prefill launch");
     }
     // Sec. 3: only an owner layer stores K/V -- the prompt's, at positions [0, s_max).
-    return owner ? store_prefix(c, layer, K, V, s_max, stream, true) : MLKV_OK;
+    return direct ? store_prefix(c, layer, K, V, s_max, stream, true) : MLKV_OK;
 }
 
 int mlkv_decode_block_fused(mlkv_cache_t c, int owner_layer, const void *Q, void *out,

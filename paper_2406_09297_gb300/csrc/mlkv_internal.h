@@ -87,8 +87,9 @@ struct DecodeParams {
                                          // a multi-layer launch: the sequences, longest first
 };
 
-// Causal prefill of one layer (mlkv_prefill.cu): one CTA per work unit, a unit being two query
-// tiles of 128 prompt positions over one KV head.  Passed by value.
+// Causal prefill of one layer (mlkv_prefill.cu): persistent CTAs over a longest-first list of work
+// units, a unit being one (head_dim 64) or two query tiles of 128 prompt positions over one KV head.
+// Passed by value.
 //   units[u] = beta | qb_b << 10 | sel << 24, qb_b the block (of 128 positions) of tile B.
 //   head_pairs = 1 (G even): tiles A and B are heads 2 sel and 2 sel + 1 at block qb_b.
 //   head_pairs = 0 (G odd):  both are head sel; A is block qb_b - 1 when qb_b is odd, else absent.

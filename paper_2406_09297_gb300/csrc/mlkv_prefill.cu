@@ -4,7 +4,8 @@
 // attends to positions 0 .. t of KV head j(i) = i / G of the layer's owner slot (causal
 // attention, Eqs. 2-3 with the MLKV maps of Eqs. 13-18).  An owner layer attends over the prompt's
 // K/V where they are and stores them in its slot (prefix_copy_kernel, launched behind this kernel
-// and running in its tail); the block's other layers attend over the slot.
+// and running in its tail), or, when its outputs would overwrite them, stores them first and attends
+// over the slot, as the block's other layers do.
 //
 // Persistent CTAs: the grid is at most one wave, and CTA c takes units c, 2P - 1 - c, 2P + c, ... of
 // the longest-first list (P CTAs).  All roles run on over the units: while a unit's last tile is in
@@ -51,9 +52,12 @@
 // What bounds it, per key tile and query tile of an SM: the tensor core (head_dim 64: 4 x 66 cycles
 // of S and 8 x 34 of P V; head_dim 128: 16 x 66) and the softmax warps' issue slots (~690 cycles:
 // 128 exponentials, and paired multiply-adds, sums and conversions that take two slots each).
-// Measured on GB300 (two layers, before -> after the persistent form with early S columns and
-// elected issuing threads): 8 x 2048 positions x 12 heads, head_dim 64, 168.6 -> 132.1 us; 4 x 2048
-// x 32 heads, head_dim 128, 313.8 -> 240.6 us; 32 prompts of 1 to 777 positions 103.7 -> 83.0 us.
+// Measured on GB300, an owner layer and a later one of its block.  First the former form (a CTA per
+// unit), then persistent CTAs with early S columns and elected issuing threads, then also with the
+// owner's K/V read in place and the producer one thread:
+//   8 x 2048 positions x 12 heads, head_dim 64    168.6   132.1   122.7 us
+//   4 x 2048 x 32 heads, head_dim 128             313.8   240.6   215 us
+//   32 prompts of 1 to 777 positions, head_dim 64 103.7    83.0    54.2 us
 //
 // The diagonal tile masks keys after the query; keys past the prompt's end only meet such masked
 // scores, and their V rows are zeroed in shared memory so that 0 * V stays 0.

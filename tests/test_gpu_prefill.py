@@ -153,3 +153,34 @@ def test_prefill_rejects_bad_arguments():
         assert e.value.code == mlkv.MLKV_ERR_INVALID_ARG
         cache.prefill(1, q, None, None, out, [5, 5])       # a non-owner layer needs no K/V
         cache.sync_status()
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("shared", ["K", "V"])
+def test_prefill_out_over_prompt_kv(d, shared):
+    # The outputs may be written over the prompt's own keys or values: an owner layer then stores
+    # them before it attends.  Outputs and cache equal those with separate buffers, bit for bit.
+    import torch
+
+    import paper_2406_09297_gb300 as mlkv
+    from tests.test_gpu_cache import _read_cache
+    h = g = 4
+    b, s_max, max_seq = 3, 700, 704
+    prompts = np.array([700, 1, 333], dtype=np.int32)
+    Q = to_dev(gen.gen_q(61, 0, b * s_max, h, d).reshape(b, s_max, h, d))
+    kv = [to_dev(gen.gen_kv(61, 0, i, b, g, s_max, d)) for i in range(2)]
+    results = []
+    for overlap in (False, True):
+        with mlkv.MLKVCache(1, h, d, [0], g, b, max_seq) as cache:
+            K, V = (t.clone() for t in kv)
+            out = torch.zeros((b, s_max, h, d), dtype=torch.bfloat16, device="cuda")
+            if overlap:
+                out = (K if shared == "K" else V).view(b, s_max, h, d)
+            cache.prefill(0, Q, K, V, out, prompts)
+            torch.cuda.synchronize()
+            cache.sync_status()
+            results.append(([out[i, :n].clone() for i, n in enumerate(prompts)],
+                            _read_cache(cache, b, g, max_seq, d)[:, :, :, :, :s_max]))
+    for x, y in zip(results[0][0], results[1][0]):
+        assert torch.equal(x.view(torch.int16), y.view(torch.int16))
+    assert (results[0][1] == results[1][1]).all()
