@@ -266,10 +266,11 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
     }
     if (threadIdx.x == 0) {
         for (int q = 0; q < NQ; ++q) {
-            // the query tiles' barrier: the producer's tensor-map copy, or the last warp's loads
-            // from host memory; freed by the unit's last S and, where the outputs are staged in
+            // the query tiles' barrier: the producer's tensor-map copy, or the loads from host
+            // memory by the last warp (deep form: by every softmax warp); freed by the unit's last S and, where the outputs are staged in
             // the query tiles, by the softmax warps
-            mbar_init(bar_q + 8 * q, 1);
+            mbar_init(bar_q + 8 * q,
+                      kSplit && kFused && p.q_host != nullptr ? PL::kSoftWarps : 1);
             mbar_init(bar_q_free + 8 * q, 1 + (PL::kStageInQ ? PL::kSoftWarps : 0));
         }
         for (int s = 0; s < R; ++s) {
@@ -333,10 +334,46 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
     if (!early)
         grid_dependency_wait();
     grid_dependents_launch();
+    // A unit's query rows from page-locked host memory through its device-mapped address (16 bytes a
+    // load, FLY of them in flight per thread of N), written into the query tiles the way the tensor
+    // map would have (128-byte swizzle); rows past them stay zero.
+    auto load_q_host = [&](const Unit &x, int qb, int t, auto n_, auto fly_) {
+        constexpr int N = decltype(n_)::value, FLY = decltype(fly_)::value;
+        constexpr int kC = D / 8;   // 16-byte chunks of a row
+        const int rows_b = (p.fused_L < p.fused_L1 ? p.fused_L : p.fused_L1) * p.G;
+        uint8_t *dst = smem + PL::kQ + qb * PL::kTiles * PL::kTileBytes;
+        const int total = (rows_b + (x.n_a > 0 ? (p.fused_L - p.fused_L1) * p.G : 0)) * kC;
+        for (int k0 = t; k0 < total; k0 += N * FLY) {
+            uint4 v[FLY];
+#pragma unroll
+            for (int u = 0; u < FLY; ++u) {
+                const int k = k0 + u * N;
+                if (k < total) {
+                    const int rr = k / kC, c = k - rr * kC;
+                    const int rw = rr < rows_b ? rr : rr - rows_b;
+                    const int lay =
+                        x.blk * p.fused_L + (rr < rows_b ? 0 : p.fused_L1) + rw / p.G;
+                    v[u] = *reinterpret_cast<const uint4 *>(
+                        p.q_host + ((static_cast<size_t>(lay) * p.b + x.beta) * p.h + x.j * p.G +
+                                    rw % p.G) * D + c * 8);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < FLY; ++u) {
+                const int k = k0 + u * N;
+                if (k < total) {
+                    const int rr = k / kC, c = k - rr * kC;
+                    const int rw = rr < rows_b ? rr : rr - rows_b;
+                    *reinterpret_cast<uint4 *>(dst + slot_of(rr < rows_b ? 1 : 0) * PL::kTileBytes +
+                                               (c >> 3) * 16384 + rw * 128 +
+                                               (((c & 7) ^ (rw & 7)) << 4)) = v[u];
+                }
+            }
+        }
+    };
     if (warp == PL::kProducer) {
         // ------------------------------------ producer ------------------------------------------
-        // Lane 0 waits and announces the bytes; the copies of a tile go out from different lanes
-        // (one thread completes about one bulk copy per 0.4 us, different lanes side by side).
+        // One thread waits, announces the bytes and sends the copies.
         setmaxnreg_dec<PL::kRegsLow>();
         bool waited = !early;
         int idx = 0;   // ring tiles sent so far: K_0, V_0, K_1, V_1, ... over all units
@@ -635,6 +672,18 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
                 atomicOr(p.err, kErrWaitFull);
             }
         };
+        if (kFused && kSplit && p.q_host != nullptr) {
+            // The CTA's only unit: nothing to compute before its queries, so every softmax warp
+            // loads, one round trip over the link (by the last warp alone, two: 64 sequences of
+            // 2,048 tokens end to end 34.5 us a step, now 32.9).
+            load_q_host(unit_of<kFused, PL::kTiles>(p, unit_index(p, 0)), 0, threadIdx.x,
+                        std::integral_constant<int, 32 * PL::kSoftWarps>{},
+                        std::integral_constant<int, 4>{});
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0)
+                mbar_arrive(bar_q);
+        }
         int kb = 0;     // key tiles of the units before
         int used = 0;   // score tiles this warpgroup has taken
         int outs = 0;   // units it has finished (P over S: phases of pv_done)
@@ -947,14 +996,8 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
         }
     } else {
         setmaxnreg_dec<PL::kRegsLow>();
-        if (kFused && p.q_host != nullptr && warp == PL::kSoftWarps + 3) {
-            // The last warp: each unit's query rows from page-locked host memory through its
-            // device-mapped address (16 bytes a load, several in flight per lane), written into the
-            // query tiles the way the tensor map would have (128-byte swizzle); rows past them stay
-            // zero.
-            constexpr int kFly = PL::kRegsLow >= 72 ? 10 : 4;
-            constexpr int kC = D / 8;   // 16-byte chunks of a row
-            const int rows_b = (p.fused_L < p.fused_L1 ? p.fused_L : p.fused_L1) * p.G;
+        if (kFused && !kSplit && p.q_host != nullptr && warp == PL::kSoftWarps + 3) {
+            // The last warp loads each unit's query rows from host memory, ahead of the unit.
             for (int n = 0;; ++n) {
                 const int i = unit_index(p, n);
                 if (i < 0)
@@ -971,41 +1014,12 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
                     ok = !flags[0];
                 if (!__shfl_sync(0xffffffffu, ok, 0))
                     break;
-                uint8_t *dst = smem + PL::kQ + qb * PL::kTiles * PL::kTileBytes;
-                const int total = (rows_b + (x.n_a > 0 ? (p.fused_L - p.fused_L1) * p.G : 0)) * kC;
-                for (int k0 = lane; k0 < total; k0 += 32 * kFly) {
-                    uint4 v[kFly];
-#pragma unroll
-                    for (int u = 0; u < kFly; ++u) {
-                        const int k = k0 + u * 32;
-                        if (k < total) {
-                            const int rr = k / kC, c = k - rr * kC;
-                            const int rw = rr < rows_b ? rr : rr - rows_b;
-                            const int lay = x.blk * p.fused_L + (rr < rows_b ? 0 : p.fused_L1) +
-                                            rw / p.G;
-                            v[u] = *reinterpret_cast<const uint4 *>(
-                                p.q_host + ((static_cast<size_t>(lay) * p.b + x.beta) * p.h +
-                                            x.j * p.G + rw % p.G) * D + c * 8);
-                        }
-                    }
-#pragma unroll
-                    for (int u = 0; u < kFly; ++u) {
-                        const int k = k0 + u * 32;
-                        if (k < total) {
-                            const int rr = k / kC, c = k - rr * kC;
-                            const int rw = rr < rows_b ? rr : rr - rows_b;
-                            *reinterpret_cast<uint4 *>(
-                                dst + slot_of(rr < rows_b ? 1 : 0) * PL::kTileBytes +
-                                (c >> 3) * 16384 + rw * 128 + (((c & 7) ^ (rw & 7)) << 4)) = v[u];
-                        }
-                    }
-                }
+                load_q_host(x, qb, lane, std::integral_constant<int, 32>{},
+                            std::integral_constant<int, PL::kRegsLow >= 72 ? 10 : 4>{});
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0)
                     mbar_arrive(bar_q + 8 * qb);
-                if (kSplit)
-                    break;   // one unit per CTA
             }
         }
     }
