@@ -127,8 +127,11 @@ struct mlkv_cache {
     int prefill_ready = 0;      // the prefill kernel's shared-memory limit is set
     int fused_ready = 0;        // the same for the fused-decode forms (bit 1 << form)
     int fused_deep = 1;         // fused decode: the deep one-tile form where one unit per SM
-    float *fused_part = nullptr;   // context-chunk partials of the fused decode
+    // Context-chunk partials of the fused decode.  A buffer that was outgrown lives until the cache
+    // is destroyed: recorded graphs, the caller's captures among them, hold its address.
+    float *fused_part = nullptr;
     size_t fused_part_floats = 0;
+    std::vector<float *> fused_outgrown;
     int step_fused = 1;         // mlkv_decode_step: the cross-layer fused form where it pays (1),
                                 // wherever the map allows it (2), never (0)
     int last_step_fused = 0;    // 1 if the most recent step ran in that form
@@ -448,6 +451,8 @@ int mlkv_cache_destroy(mlkv_cache_t c)
         cudaFree(c->stage);
     if (c->fused_part)
         cudaFree(c->fused_part);
+    for (float *part : c->fused_outgrown)
+        cudaFree(part);
     if (c->record_stream)
         cudaStreamDestroy(c->record_stream);
     free_all(c);
@@ -889,16 +894,22 @@ static int fused_issue(mlkv_cache_t c, const void *Q, void *out, int n_q_layers,
         const size_t rows = static_cast<size_t>(nblk) * c->b * c->g * cmax * L * c->G;
         const size_t floats = rows * (c->d + 1);
         if (floats > c->fused_part_floats) {
-            if (c->fused_part)
-                cudaFree(c->fused_part);
-            c->fused_part = nullptr;
-            c->fused_part_floats = 0;
-            if ((e = cudaMalloc(&c->fused_part, floats * sizeof(float))) != cudaSuccess) {
-                c->fused_part = nullptr;
+            // At least twice the former size, so that all the outgrown buffers together are smaller
+            // than the one in use; as much as is needed where that does not fit.
+            float *part = nullptr;
+            size_t want = std::max(floats, 2 * c->fused_part_floats);
+            if ((e = cudaMalloc(&part, want * sizeof(float))) != cudaSuccess && want > floats) {
+                cudaGetLastError();
+                want = floats;
+                e = cudaMalloc(&part, want * sizeof(float));
+            }
+            if (e != cudaSuccess)
                 return fail(MLKV_ERR_OOM, "fused-decode partials (%zu bytes): %s",
                             floats * sizeof(float), cudaGetErrorString(e));
-            }
-            c->fused_part_floats = floats;
+            if (c->fused_part != nullptr)
+                c->fused_outgrown.push_back(c->fused_part);
+            c->fused_part = part;
+            c->fused_part_floats = want;
         }
         p.part = c->fused_part;
         p.part_lse = c->fused_part + rows * c->d;

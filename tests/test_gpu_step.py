@@ -573,3 +573,59 @@ def test_fused_step_host_buffers_beyond_one_wave(owner, h, g, d, b):
             mx, mean = errors(from_dev(out[n]), ref.decode(n, gen.bf16_bits_to_f64(qb[n]), lens))
             assert mx <= MAX_ABS and mean <= MEAN_ABS, (n, mx, mean)
         cache.sync_status()
+
+
+@pytest.mark.parametrize("how", ["step", "host", "capture"])
+def test_recorded_step_after_scratch_grew(how):
+    # A recorded step (the cache's own graph of a step on device or host buffers, or a capture of the
+    # caller's) is replayed after a step over a longer context made the fused form's scratch grow:
+    # the graph still writes and merges the partials it was recorded with.  Bit for bit the outputs
+    # of the same step before.
+    import torch
+
+    import paper_2406_09297_gb300 as mlkv
+    owner, h, g, d, b, short, long = [0] * 6 + [6] * 6, 12, 1, 64, 1, 1500, 40000
+    with mlkv.MLKVCache(12, h, d, owner, g, b, long) as cache:
+        qb, kn, vn = _inputs(owner, h, g, d, b, [short], long, 95, cache, None)
+        cache.set_option("step_fused", 2)
+        cache.set_option("step_graph", 1)
+        tensors = [to_dev(x) for x in (qb, kn, vn)]
+        tensors.append(torch.empty((12, b, h, d), dtype=torch.bfloat16, device="cuda"))
+        if how == "host":
+            # off the 16-byte grid: copied to the device, the step recorded in a graph
+            dev, tensors = tensors, []
+            for x in dev:
+                t = torch.empty(x.numel() + 1, dtype=torch.bfloat16).pin_memory()[1:].view(x.shape)
+                t.copy_(x)
+                tensors.append(t)
+        Q, K, V, out = tensors
+        call = cache.decode_step_host if how == "host" else cache.decode_step
+
+        def step(n):
+            call(Q, K, V, out, np.full(b, n, dtype=np.int32))
+            torch.cuda.synchronize()
+            assert cache.get_option("last_deferred_merge") == 1
+            return out.clone()
+
+        first = step(short)
+        if how == "capture":
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                cache.decode_step(Q, K, V, out, np.full(b, short, dtype=np.int32),
+                                  stream=torch.cuda.current_stream())
+        else:
+            step(short)
+        replays = cache.get_option("step_graph_replays")
+        assert replays == (0 if how == "capture" else 1)
+        step(long)
+        filler = torch.full((64 << 20,), float("nan"), device="cuda")   # over whatever was given back
+        out.fill_(float("nan"))
+        if how == "capture":
+            graph.replay()
+        else:
+            call(Q, K, V, out, np.full(b, short, dtype=np.int32))
+            assert cache.get_option("step_graph_replays") == replays + 1
+        torch.cuda.synchronize()
+        del filler
+        assert torch.equal(out.view(torch.int16), first.view(torch.int16))
+        cache.sync_status()
