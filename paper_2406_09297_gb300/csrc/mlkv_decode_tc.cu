@@ -192,10 +192,14 @@ __global__ void __launch_bounds__(TcPlan<D, T, STAGES>::kThreads, 1)
 
     // Dependency discipline as in decode_kernel: with p.early_fetch (inside mlkv_decode_step) the
     // previous kernel wrote nothing this one reads but the newest row of a segment (its last tile)
-    // and the merge scratch; otherwise nothing global is touched before the wait.
+    // and the merge scratch; otherwise nothing global is touched before the wait.  The next kernel
+    // goes as soon as any warp lets it; with p.trigger_late (a step's first layer) each does so only
+    // after the wait.
     if (warp == PL::kProducer) {
         // ------------------------------------ producer ------------------------------------------
         if (lane != 0) {
+            if (p.trigger_late)
+                grid_dependency_wait();
             grid_dependents_launch();   // only lane 0 touches global memory
         } else {
             int issued = 0;
@@ -271,6 +275,8 @@ __global__ void __launch_bounds__(TcPlan<D, T, STAGES>::kThreads, 1)
         // soon as its K/V has landed and an S^T buffer is free (up to two tiles ahead of the
         // softmax), and O^T += V^T P^T of a tile as soon as its P^T is written -- which also frees
         // the tile's stage for the producer.  Lane 0 polls and decides; the warp follows.
+        if (p.trigger_late)
+            grid_dependency_wait();
         grid_dependents_launch();
         constexpr uint32_t kIdS = umma_idesc(128, 16, 0, 0);
         constexpr uint32_t kIdPV = umma_idesc(D, 16, 1, 1);

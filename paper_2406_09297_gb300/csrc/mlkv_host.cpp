@@ -669,6 +669,7 @@ static int decode_impl(mlkv_cache_t c, int layer, const void *K_new, const void 
     p.tile_tokens = T;
     p.decode_grid = grid;
     p.early_fetch = early_fetch;
+    p.trigger_late = (in_step && early_fetch == 0 && c->pdl && c->early_fetch != 0) ? 1 : 0;
     p.newest_ready = newest_ready;
     p.store_new = K_new != nullptr ? store_new : 0;
     p.Q_next = static_cast<const __nv_bfloat16 *>(Q_next);
@@ -1298,6 +1299,7 @@ static int issue_step_ml(mlkv_cache_t c, const char *Q, const char *K, const cha
     p.Q_next = nullptr;
     // After this library's input copy the first tile of each CTA goes out before the wait.
     p.early_fetch = (stage != nullptr && c->pdl) ? 2 : 0;
+    p.trigger_late = 0;
     p.newest_ready = 1;
     p.store_new = 0;
     // L2 prefetch of every slot's visible rows when they all fit with room to spare.

@@ -49,6 +49,10 @@ struct DecodeParams {
                               // dependency wait.  2: the previous kernel is this library's copy of
                               // the step's inputs (Q, K_new, V_new), which writes no cache row:
                               // only the CTA's first tile is fetched before the wait
+    int trigger_late;         // 1: the next kernel goes only after this one's dependency wait (a
+                              // step's first layer: the layers behind it read cache rows, queries
+                              // and new tokens before their own wait, so every kernel that came
+                              // before the step must have ended); 0: at once
     int newest_ready;         // 1: the segments' newest rows are replaced from K_new/V_new by this
                               // grid: no wait before a segment's last tile
     int store_new;            // with K_new: 1 = also store the new token in the cache (the owner

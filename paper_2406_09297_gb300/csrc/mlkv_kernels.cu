@@ -276,8 +276,10 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
     bool pre_issued = false;
     // The trigger comes first: the next launch (inside a decode step, the next layer's decode)
     // may start as soon as every CTA of this grid is resident.  What it reads before its own
-    // dependency wait is fixed by p.early_fetch, and it finishes only after this grid.
-    if (threadIdx.x == 0)
+    // dependency wait is fixed by p.early_fetch, and it finishes only after this grid.  The first
+    // layer of a step triggers after its own wait instead: the kernels before the step may still be
+    // writing what the next layers read early.
+    if (threadIdx.x == 0 && !p.trigger_late)
         grid_dependents_launch();
     if (warp == PL::kProducer) {
         if (lane == 0) {
@@ -348,8 +350,11 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
         load_q_frag<D, kT>(qa, q_rows(wk.layer, wk.beta, wk.j), D, p.G, lane);
     if (warp != PL::kProducer && !early)
         grid_dependency_wait();
-    if (warp == PL::kEpilogue && lane == 0)
+    if (warp == PL::kEpilogue && lane == 0) {
         grid_dependency_wait();
+        if (p.trigger_late)
+            grid_dependents_launch();
+    }
 
     // -------------------------------- producer warp --------------------------------------------
     // Every lane walks the same tiles; lane 0 waits (dependency, free stages) and announces each

@@ -255,6 +255,7 @@ extern "C" int mlkv_decode_attention_static(const void *kv_slot, int batch, int 
     p.tile_tokens = T;
     p.decode_grid = grid;
     p.early_fetch = 0;
+    p.trigger_late = 0;
     p.newest_ready = 0;
     p.store_new = 0;
     p.pf_own = 0;

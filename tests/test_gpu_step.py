@@ -629,3 +629,55 @@ def test_recorded_step_after_scratch_grew(how):
         del filler
         assert torch.equal(out.view(torch.int16), first.view(torch.int16))
         cache.sync_status()
+
+
+@pytest.mark.parametrize("before", ["load", "prefill", "append"])
+@pytest.mark.parametrize("options", [{"early_fetch": 1}, {"early_fetch": 2},
+                                     {"early_fetch": 1, "tc": 1, "tile_tokens": 128}])
+def test_step_right_behind_cache_writes(before, options):
+    # A step of per-layer launches queued right behind calls that write cache rows other than its
+    # newest ones: the layers after the first read cache tiles before their own dependency wait, so
+    # the first lets them go only once those calls have ended.  Bit for bit the outputs of the same
+    # calls with a host wait before the step.
+    import torch
+
+    import paper_2406_09297_gb300 as mlkv
+    owner, h, g, d, b, L = [0, 0, 0, 3, 3, 3], 12, 2, 64, 8, 1025
+    lens = np.full(b, L, dtype=np.int32)   # the newest row alone in its tile
+    with mlkv.MLKVCache(6, h, d, owner, g, b, L) as cache:
+        for key, value in {"step_kernel": 0, "step_graph": 0, **options}.items():
+            cache.set_option(key, value)
+        qb, kn, vn = _inputs(owner, h, g, d, b, lens, L, 97, cache, None)
+        Q, K, V = to_dev(qb), to_dev(kn), to_dev(vn)
+        out = torch.empty((6, b, h, d), dtype=torch.bfloat16, device="cuda")
+        pq = torch.zeros((b, L - 1, h, d), dtype=torch.bfloat16, device="cuda")
+        po = torch.empty_like(pq)
+
+        def run(rep, wait):
+            # other rows every time: a row read too early is the time before's
+            gen_ = torch.Generator(device="cuda").manual_seed(rep)
+            out.fill_(float("nan"))
+            for n in (0, 3):
+                k, v = (torch.randn((b, g, L - 1, d), device="cuda", generator=gen_).bfloat16()
+                        for _ in range(2))
+                if before == "load":
+                    cache.load_prefix(n, k, v, L - 1)
+                elif before == "prefill":
+                    cache.prefill(n, pq, k, v, po, [L - 1] * b)
+                else:
+                    rows = [(pos, k[:, :, pos - 1].contiguous(), v[:, :, pos - 1].contiguous())
+                            for pos in range(L - 9, L)]
+                    for pos, kr, vr in rows:
+                        cache.append(n, kr, vr, [pos] * b)
+            if wait:
+                torch.cuda.synchronize()
+            cache.decode_step(Q, K, V, out, lens)
+            torch.cuda.synchronize()
+            assert cache.get_option("last_step_kernel") == 0
+            return out.clone()
+
+        expect = [run(rep, True) for rep in range(4)]
+        for rep in range(16):
+            assert torch.equal(run(rep % 4, False).view(torch.int16),
+                               expect[rep % 4].view(torch.int16)), rep
+        cache.sync_status()
