@@ -71,7 +71,8 @@ struct TcPlan {
     static constexpr int kPBytes = T * 32;            // P^T [2][T][8] bf16
     static constexpr int kResO = 16 * D * 4;          // a piece's result: o[16][D] f32
     static constexpr int kResBytes = kResO + 16 * 4 + 32;   // + lse[16] + 8 ints of metadata
-    static constexpr int kEpiCap = 64;                // epilogue merge weights (more: recomputed)
+    // weights of an inline merge, pieces x heads (8 x 8 or 4 x 16 at most), and a reciprocal a head
+    static constexpr int kEpiCap = 64 + 16;
     static constexpr int kQ = STAGES * kStageBytes;   // [2][kQBytes]
     static constexpr int kP = kQ + 2 * kQBytes;       // [2][kPBytes]
     static constexpr int kRes = kP + 2 * kPBytes;     // [2][kResBytes]
@@ -436,7 +437,7 @@ __global__ void __launch_bounds__(TcPlan<D, T, STAGES>::kThreads, 1)
             if (!flags[0])
                 epilogue_piece<D>(p, reinterpret_cast<const float *>(slot),
                                   reinterpret_cast<const float *>(slot + PL::kResO), meta, s_w,
-                                  PL::kEpiCap, lane, cta);
+                                  lane, cta);
             __syncwarp();
             if (lane == 0)
                 mbar_arrive(bar_res_empty + 8 * rb);
@@ -803,7 +804,8 @@ __global__ void __launch_bounds__(TcPlan<D, T, STAGES>::kThreads, 1)
                     }
                     soft_bar_sync();
                     if (flags[1]) {
-                        // Last finisher of the segment: merge its <= 4 records (own included).
+                        // Last finisher of the segment: merge its records (own included; at most
+                        // inline_merge_pieces of them).
                         const int np = c_last - c_first + 1;
                         const size_t rec0 = static_cast<size_t>(seg + c_first);
                         for (int i = 2 * tid; i < G * D; i += 256) {
@@ -827,8 +829,8 @@ __global__ void __launch_bounds__(TcPlan<D, T, STAGES>::kThreads, 1)
                             for (int k = 0; k < kInlineMergeMaxPieces; ++k) {
                                 const float w = fast_exp2(lv[k] - mx);   // 0 past np
                                 tot += w;
-                                ax += w * ovv[k].x;
-                                ay += w * ovv[k].y;
+                                ax = fmaf(w, ovv[k].x, ax);
+                                ay = fmaf(w, ovv[k].y, ay);
                             }
                             const float inv = fast_rcp(tot);
                             *reinterpret_cast<uint32_t *>(ob + i) = pack_bf16x2(ax * inv, ay * inv);

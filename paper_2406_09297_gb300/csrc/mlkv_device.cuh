@@ -523,11 +523,14 @@ enum : int { kMetaBeta = 0, kMetaJ, kMetaSeg, kMetaWhole, kMetaFirst, kMetaLast,
 // One piece's result (normalised o, lse, metadata) sits in a shared-memory slot.  A whole segment
 // goes straight to `out`.  Otherwise the slot becomes partial record seg + cta; the counter of the
 // segment (acquire-release) tells the CTA that finished it last, which merges all its records:
-//   o = sum_c 2^(lse_c - M) o_c / sum_c 2^(lse_c - M),  M = max_c lse_c.
+//   o = sum_c 2^(lse_c - M) o_c / sum_c 2^(lse_c - M),  M = max_c lse_c,
+// summed in the records' order and multiplied by the reciprocal at the end, as the softmax warps do
+// when their piece is the last: the outputs do not depend on which CTA that is.  s_w: room for
+// (kInlineMergeMaxPieces records or 4, see inline_merge_pieces) x G weights and G reciprocals.
 template <int D>
 __device__ __forceinline__ void epilogue_piece(const DecodeParams &p, const float *ro,
                                                const float *rlse, const int *meta, float *s_w,
-                                               int cap, int lane, int cta)
+                                               int lane, int cta)
 {
     const int G = p.G;
     const int beta = meta[kMetaBeta], j = meta[kMetaJ], seg = meta[kMetaSeg];
@@ -566,90 +569,72 @@ __device__ __forceinline__ void epilogue_piece(const DecodeParams &p, const floa
     const int np = c_last - c_first + 1;
     const size_t rec0 = static_cast<size_t>(seg + c_first);
     const float NEG_INF = -__int_as_float(0x7f800000);
-    if (np * G <= cap) {
-        for (int i = lane; i < np * G; i += 32)
-            s_w[i] = __ldcg(&p.part_lse[rec0 * G + i]);
-        __syncwarp();
-        for (int r = lane; r < G; r += 32) {
-            float mx = NEG_INF;
-            for (int k = 0; k < np; ++k)
-                mx = fmaxf(mx, s_w[k * G + r]);
-            float tot = 0.f;
-            for (int k = 0; k < np; ++k) {
-                const float w = fast_exp2(s_w[k * G + r] - mx);
-                s_w[k * G + r] = w;
-                tot += w;
-            }
-            const float inv = 1.f / tot;
-            for (int k = 0; k < np; ++k)
-                s_w[k * G + r] *= inv;
+    float *s_inv = s_w + np * G;
+    for (int i = lane; i < np * G; i += 32)
+        s_w[i] = __ldcg(&p.part_lse[rec0 * G + i]);
+    __syncwarp();
+    if (lane < G) {
+        float mx = NEG_INF;
+        for (int k = 0; k < np; ++k)
+            mx = fmaxf(mx, s_w[k * G + lane]);
+        float tot = 0.f;
+        for (int k = 0; k < np; ++k) {
+            const float w = fast_exp2(s_w[k * G + lane] - mx);
+            s_w[k * G + lane] = w;
+            tot += w;
         }
-        __syncwarp();
-        // Each lane owns CH float4 columns of a 128*CH-element chunk; the loads of all its
-        // columns for two pieces are in flight together.
-        constexpr int CH = 8;
-        const float *base = p.part_o + rec0 * G * D;
-        for (int c0 = 0; c0 < G * D; c0 += 128 * CH) {
-            float4 acc[CH];
+        s_inv[lane] = fast_rcp(tot);
+    }
+    __syncwarp();
+    // Each lane owns CH float4 columns of a 128*CH-element chunk; the loads of all its columns for
+    // two pieces are in flight together.
+    constexpr int CH = 8;
+    const float *base = p.part_o + rec0 * G * D;
+    for (int c0 = 0; c0 < G * D; c0 += 128 * CH) {
+        float4 acc[CH];
 #pragma unroll
-            for (int u = 0; u < CH; ++u)
-                acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int k = 0; k < np; k += 2) {
-                float4 v0[CH], v1[CH];
+        for (int u = 0; u < CH; ++u)
+            acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k = 0; k < np; k += 2) {
+            float4 v0[CH], v1[CH];
 #pragma unroll
-                for (int u = 0; u < CH; ++u) {
-                    const int i = c0 + u * 128 + lane * 4;
-                    const bool in = i < G * D;
-                    v0[u] = in ? __ldcg(reinterpret_cast<const float4 *>(
-                                     base + static_cast<size_t>(k) * G * D + i))
-                               : make_float4(0.f, 0.f, 0.f, 0.f);
-                    v1[u] = (in && k + 1 < np)
-                                ? __ldcg(reinterpret_cast<const float4 *>(
-                                      base + static_cast<size_t>(k + 1) * G * D + i))
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-#pragma unroll
-                for (int u = 0; u < CH; ++u) {
-                    const int i = c0 + u * 128 + lane * 4;
-                    if (i < G * D) {
-                        const int row = i / D;
-                        const float w0 = s_w[k * G + row];
-                        const float w1 = (k + 1 < np) ? s_w[(k + 1) * G + row] : 0.f;
-                        acc[u].x += w0 * v0[u].x + w1 * v1[u].x;
-                        acc[u].y += w0 * v0[u].y + w1 * v1[u].y;
-                        acc[u].z += w0 * v0[u].z + w1 * v1[u].z;
-                        acc[u].w += w0 * v0[u].w + w1 * v1[u].w;
-                    }
-                }
+            for (int u = 0; u < CH; ++u) {
+                const int i = c0 + u * 128 + lane * 4;
+                const bool in = i < G * D;
+                v0[u] = in ? __ldcg(reinterpret_cast<const float4 *>(
+                                 base + static_cast<size_t>(k) * G * D + i))
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+                v1[u] = (in && k + 1 < np) ? __ldcg(reinterpret_cast<const float4 *>(
+                                                 base + static_cast<size_t>(k + 1) * G * D + i))
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
             for (int u = 0; u < CH; ++u) {
                 const int i = c0 + u * 128 + lane * 4;
                 if (i < G * D) {
-                    uint2 w2;
-                    w2.x = pack_bf16x2(acc[u].x, acc[u].y);
-                    w2.y = pack_bf16x2(acc[u].z, acc[u].w);
-                    *reinterpret_cast<uint2 *>(ob + i) = w2;
+                    const int row = i / D;
+                    const float w0 = s_w[k * G + row];
+                    const float w1 = (k + 1 < np) ? s_w[(k + 1) * G + row] : 0.f;
+                    acc[u].x = fmaf(w1, v1[u].x, fmaf(w0, v0[u].x, acc[u].x));
+                    acc[u].y = fmaf(w1, v1[u].y, fmaf(w0, v0[u].y, acc[u].y));
+                    acc[u].z = fmaf(w1, v1[u].z, fmaf(w0, v0[u].z, acc[u].z));
+                    acc[u].w = fmaf(w1, v1[u].w, fmaf(w0, v0[u].w, acc[u].w));
                 }
             }
         }
-        __syncwarp();
-    } else {
-        // Very many pieces: the same merge, weights recomputed per element.
-        for (int i = lane; i < G * D; i += 32) {
-            const int row = i / D;
-            float mx = NEG_INF;
-            for (int k = 0; k < np; ++k)
-                mx = fmaxf(mx, __ldcg(&p.part_lse[(rec0 + k) * G + row]));
-            float acc = 0.f, wsum = 0.f;
-            for (int k = 0; k < np; ++k) {
-                const float w = fast_exp2(__ldcg(&p.part_lse[(rec0 + k) * G + row]) - mx);
-                wsum += w;
-                acc += w * __ldcg(&p.part_o[(rec0 + k) * G * D + i]);
+#pragma unroll
+        for (int u = 0; u < CH; ++u) {
+            const int i = c0 + u * 128 + lane * 4;
+            if (i < G * D) {
+                const float inv = s_inv[i / D];
+                uint2 w2;
+                w2.x = pack_bf16x2(acc[u].x * inv, acc[u].y * inv);
+                w2.y = pack_bf16x2(acc[u].z * inv, acc[u].w * inv);
+                *reinterpret_cast<uint2 *>(ob + i) = w2;
             }
-            ob[i] = __float2bfloat16_rn(acc / wsum);
         }
     }
+    __syncwarp();   // s_w may be rewritten
     if (lane == 0)
         p.counters[seg] = 0u;
 }

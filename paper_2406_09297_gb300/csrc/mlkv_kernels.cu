@@ -82,8 +82,9 @@ struct Plan {
     // 165 us for 12 layers, 172 with one buffer; 145 once the buffer was freed before the counter).
     static constexpr int kRawBufs = (!kT && T == 256) ? 1 : 2;
     static constexpr int kRaw = STAGES * kStageBytes;                  // [kRawBufs][kRawBytes]
-    static constexpr int kEpiW = kRaw + kRawBufs * kRawBytes;   // weights of an inline merge, f32
-    static constexpr int kFlags = kEpiW + kInlineMergeMaxPieces * 16 * 4;   // int [4]
+    // an inline merge's weights [kInlineMergeMaxPieces][16] and reciprocals [16], f32
+    static constexpr int kEpiW = kRaw + kRawBufs * kRawBytes;
+    static constexpr int kFlags = kEpiW + (kInlineMergeMaxPieces + 1) * 16 * 4;   // int [4]
     // u64 full[S], empty[S], res_full[2], res_empty[2], cluster
     static constexpr int kBars = kFlags + 16;
     // Dynamic tail: per-sequence tables (lengths differ) or, in cluster mode with one raw buffer,
@@ -522,7 +523,8 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
                 continue;
             // This CTA finished the segment last: it merges records seg + c_first .. seg + c_last (at
             // most kInlineMergeMaxPieces), o = sum_c 2^(lse_c - M) o_c / sum_c 2^(lse_c - M), M the
-            // largest lse.
+            // largest lse, summed in the records' order and multiplied by the reciprocal at the end as
+            // the consumer warps do (merge4): the outputs do not depend on which CTA is last.
             float *s_w = reinterpret_cast<float *>(smem + PL::kEpiW);
             const int np = c_last - c_first + 1;
             const size_t rec0 = static_cast<size_t>(seg + c_first);
@@ -571,10 +573,10 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
                                 lv[k] = fast_exp2(lv[k] - mx);   // 0 past the records
                                 tot += lv[k];
                             }
-                            const float inv = 1.f / tot;
 #pragma unroll
                             for (int k = 0; k < kInlineMergeMaxPieces; ++k)
-                                s_w[k * G + lane] = lv[k] * inv;
+                                s_w[k * G + lane] = lv[k];
+                            s_w[kInlineMergeMaxPieces * G + lane] = fast_rcp(tot);
                         }
                         __syncwarp();
                     }
@@ -594,10 +596,12 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
 #pragma unroll
                 for (int u = 0; u < CH; ++u) {
                     const int i = c0 + u * 128;
-                    if (i < G * D)
+                    if (i < G * D) {
+                        const float inv = s_w[kInlineMergeMaxPieces * G + i / D];
                         *reinterpret_cast<uint2 *>(ob + i) =
-                            make_uint2(pack_bf16x2(acc[u].x, acc[u].y),
-                                       pack_bf16x2(acc[u].z, acc[u].w));
+                            make_uint2(pack_bf16x2(acc[u].x * inv, acc[u].y * inv),
+                                       pack_bf16x2(acc[u].z * inv, acc[u].w * inv));
+                    }
                 }
             }
             __syncwarp();   // s_w may be rewritten

@@ -233,3 +233,35 @@ def test_group_sizes_around_eight(d, tile, G):
                    options={"grid": 7, "tile_tokens": tile})
     run_small_case([0], 2 * G, 2, d, 2, [2 * tile, 2 * tile], 2 * tile, seed=34,
                    options={"tile_tokens": tile})
+
+
+@pytest.mark.parametrize("h,g,d,b,s,options", [
+    (32, 8, 128, 8, 3000, {}),                        # 6 pieces a segment at most, groups of 4
+    (12, 4, 64, 64, 3000, {}),                        # groups of 3, 3 pieces
+    (32, 2, 64, 12, 6000, {"tile_tokens": 128, "grid": 32}),   # the 16-row kernel
+    (32, 8, 128, 8, 3000, {"tc": 1, "tile_tokens": 128}),
+    (32, 2, 64, 12, 6000, {"tc": 1, "tile_tokens": 128, "grid": 32}),
+])
+def test_split_merges_are_reproducible(h, g, d, b, s, options):
+    # A cut segment is merged by whichever CTA finishes it last, in its epilogue warp or, if the
+    # piece is the CTA's last, by all its warps: the same bits every time.
+    import torch
+
+    import paper_2406_09297_gb300 as mlkv
+    lens = np.array([1 + (i * 977) % s for i in range(b - 1)] + [s], dtype=np.int32)
+    gen_ = torch.Generator(device="cuda").manual_seed(35)
+    k, v = (torch.randn((b, g, s, d), device="cuda", generator=gen_).bfloat16() for _ in range(2))
+    q = torch.randn((b, h, d), device="cuda", generator=gen_).bfloat16()
+    with mlkv.MLKVCache(1, h, d, [0], g, b, s) as cache:
+        for key, value in options.items():
+            cache.set_option(key, value)
+        cache.load_prefix(0, k, v, s)
+        outs = [torch.empty_like(q) for _ in range(64)]
+        for out in outs:
+            cache.decode_attention(0, q, out, lens)
+        torch.cuda.synchronize()
+        assert cache.get_option("last_deferred_merge") == 0
+        assert cache.get_option("last_tc") == options.get("tc", 0)
+        for out in outs[1:]:
+            assert torch.equal(out.view(torch.int16), outs[0].view(torch.int16))
+        cache.sync_status()
