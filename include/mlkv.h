@@ -218,10 +218,10 @@ int mlkv_decode_step_host(mlkv_cache_t c, const void *Q, const void *K, const vo
  *   out          device bf16 [batch][s_max][h][d]; rows past a prompt's length are not written
  *   prompt_lens  host int32[batch], 1 <= prompt_lens[beta] <= s_max
  *   s_max        1 <= s_max <= max_seq
- * An owner layer reads K and V in place and stores them behind the attention; out may overlap them
- * (they are then stored first).  The caller keeps the buffers valid until the stream has finished
- * the call's work.  Errors: MLKV_ERR_INVALID_ARG (null or unaligned pointer, out overlapping Q),
- * MLKV_ERR_RANGE (lengths), MLKV_ERR_CUDA.
+ * An owner layer reads K and V in place and stores them behind the attention; if out overlaps them,
+ * or they lie in another GPU's memory or the host's, they are stored first.  The caller keeps the
+ * buffers valid until the stream has finished the call's work.  Errors: MLKV_ERR_INVALID_ARG (null
+ * or unaligned pointer, out overlapping Q), MLKV_ERR_RANGE (lengths), MLKV_ERR_CUDA.
  */
 int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const void *V, void *out,
                  const int *prompt_lens, int s_max, void *cuda_stream);
@@ -229,6 +229,8 @@ int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const 
 /*
  * mlkv_load_prefix - bulk-stores positions [0, len) of an owner layer's keys and values
  * (prefill).  K, V: device bf16 [batch][g][len][d].  No-op (MLKV_OK) for a non-owner layer.
+ * A kernel copies them; if K or V lies in another GPU's memory or the host's, or off the 16-byte
+ * grid, two cudaMemcpy2DAsync do.
  * Paper: Sec. 4.5 starts decoding from a pre-filled ("dummy") cache.
  */
 int mlkv_load_prefix(mlkv_cache_t c, int layer, const void *K, const void *V, int len,

@@ -1762,17 +1762,30 @@ int mlkv_decode_step_host(mlkv_cache_t c, const void *Q, const void *K, const vo
     return record_or_replay(c, key, c->host_key, c->host_pending, c->host_exec, stream, issue);
 }
 
-// Stores positions [0, len) of an owner layer's keys and values in its slot: one kernel for 16-byte
-// aligned tensors, else two pitched copies.  under_prefill: see launch_prefix_copy.
+// Whether the cache's GPU holds p in its own memory.  Only that is read by kernels as a prompt's K/V:
+// another GPU's memory may not be mapped here, and the host's may not be readable by kernels.
+static bool on_device(const mlkv_cache *c, const void *p)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == c->device;
+}
+
+// Stores positions [0, len) of an owner layer's keys and values in its slot: one kernel, or (K or V
+// off the 16-byte grid or not in this device's memory) two pitched copies.  under_prefill: see
+// launch_prefix_copy.
 static int store_prefix(mlkv_cache_t c, int layer, const void *K, const void *V, int len,
-                        cudaStream_t s, bool under_prefill)
+                        cudaStream_t s, bool by_kernel, bool under_prefill)
 {
     const size_t row = static_cast<size_t>(len) * c->d * 2;
     const size_t pitch = static_cast<size_t>(c->max_seq) * c->d * 2;
     const size_t slot_bytes = c->cache_bytes / c->m;
     char *base = static_cast<char *>(c->cache) + slot_bytes * c->slot[layer];
     const size_t rows = static_cast<size_t>(c->b) * c->g;
-    if (aligned16(K) && aligned16(V)) {
+    if (by_kernel) {
         mlkv::PrefixParams p;
         p.K = static_cast<const uint4 *>(K);
         p.V = static_cast<const uint4 *>(V);
@@ -1808,7 +1821,9 @@ int mlkv_load_prefix(mlkv_cache_t c, int layer, const void *K, const void *V, in
     if (K == nullptr || V == nullptr)
         return fail(MLKV_ERR_INVALID_ARG, "K and V must be non-NULL");
     DeviceGuard guard(c->device);
-    return store_prefix(c, layer, K, V, len, static_cast<cudaStream_t>(cuda_stream), false);
+    const bool by_kernel = aligned16(K) && aligned16(V) && on_device(c, K) && on_device(c, V);
+    return store_prefix(c, layer, K, V, len, static_cast<cudaStream_t>(cuda_stream), by_kernel,
+                        false);
 }
 
 int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const void *V, void *out,
@@ -1844,10 +1859,13 @@ int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const 
         return fail(MLKV_ERR_INVALID_ARG, "K and V must be non-NULL and 16-byte aligned");
     DeviceGuard guard(c->device);
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    // An owner layer reads the prompt's K/V in place and stores them afterwards, unless the outputs
-    // would overwrite them or the store's target is one of the inputs: then it stores them first.
+    // An owner layer reads the prompt's K/V in place and stores them afterwards, unless they lie in
+    // memory kernels may not read, the outputs would overwrite them or the store's target is one of
+    // the inputs: then it stores them first.
     bool direct = owner;
     if (owner) {
+        const bool local = on_device(c, K) && on_device(c, V);
+        direct = local;
         const size_t kvbytes = static_cast<size_t>(c->b) * c->g * s_max * c->d * 2;
         auto overlap = [](const void *a, size_t na, const void *b, size_t nb) {
             const char *x = static_cast<const char *>(a), *y = static_cast<const char *>(b);
@@ -1859,7 +1877,7 @@ int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const 
         if (overlap(Q, qbytes, c->cache, c->cache_bytes))
             direct = false;
         if (!direct) {
-            const int rc = store_prefix(c, layer, K, V, s_max, stream, false);
+            const int rc = store_prefix(c, layer, K, V, s_max, stream, local, false);
             if (rc != MLKV_OK)
                 return rc;
         }
@@ -1965,7 +1983,7 @@ int mlkv_prefill(mlkv_cache_t c, int layer, const void *Q, const void *K, const 
             return fail_cuda(e, "prefill launch");
     }
     // Sec. 3: only an owner layer stores K/V -- the prompt's, at positions [0, s_max).
-    return direct ? store_prefix(c, layer, K, V, s_max, stream, true) : MLKV_OK;
+    return direct ? store_prefix(c, layer, K, V, s_max, stream, true, true) : MLKV_OK;
 }
 
 int mlkv_decode_block_fused(mlkv_cache_t c, int owner_layer, const void *Q, void *out,

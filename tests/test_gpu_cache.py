@@ -116,6 +116,72 @@ def test_prefix_store_bit_exact(d, length, s, how):
         c.sync_status()
 
 
+def _captured_nodes(stream, call):
+    """The kinds of the nodes `call` records in a capture of `stream` (nothing runs)."""
+    import ctypes
+    cuda = ctypes.CDLL("libcuda.so.1")
+    handle, graph = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p()
+    assert cuda.cuStreamBeginCapture_v2(handle, 1) == 0   # thread-local
+    try:
+        call()
+    finally:
+        assert cuda.cuStreamEndCapture(handle, ctypes.byref(graph)) == 0
+    n = ctypes.c_size_t()
+    assert cuda.cuGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert cuda.cuGraphGetNodes(graph, nodes, ctypes.byref(n)) == 0
+    kinds = []
+    for node in nodes:
+        kind = ctypes.c_int()
+        assert cuda.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        kinds.append({0: "kernel", 1: "copy"}.get(kind.value, kind.value))
+    assert cuda.cuGraphDestroy(graph) == 0
+    return sorted(kinds)
+
+
+def test_prefix_outside_device_memory():
+    # K and V elsewhere than in the cache's device memory are left to the copy engine, which reaches
+    # them all; no kernel reads them, neither the store's nor an owner's prefill.
+    import torch
+
+    import paper_2406_09297_gb300 as mlkv
+    b, h, g, d, s = 3, 4, 2, 64, 200
+    K, V = (to_dev(gen.gen_kv(12, 0, i, b, g, s, d)) for i in range(2))
+    Q = to_dev(gen.gen_q(12, 0, b * s, h, d).reshape(b, s, h, d))
+    lens = [s, 70, 1]
+    stream = torch.cuda.Stream()
+    pinned = [x.cpu().pin_memory() for x in (K, V)]
+    with mlkv.MLKVCache(1, h, d, [0], g, b, s) as c:
+        out = torch.zeros_like(Q)
+        c.prefill(0, Q, K, V, out, lens)
+        torch.cuda.synchronize()
+        want, want_kv = out.clone(), _read_cache(c, b, g, s, d)
+
+        def kinds(k, v, prefill):
+            if prefill:
+                return _captured_nodes(stream, lambda: c.prefill(0, Q, k, v, out, lens, stream=stream))
+            return _captured_nodes(stream, lambda: c.load_prefix(0, k, v, s, stream=stream))
+
+        assert kinds(K, V, False) == ["kernel"]
+        assert kinds(K, V, True) == ["kernel", "kernel"]      # attention, store
+        for k, v in (pinned, (K, pinned[1]), (pinned[0], V)):
+            assert kinds(k, v, False) == ["copy", "copy"]
+            assert kinds(k, v, True) == ["copy", "copy", "kernel"]
+    for k, v in (pinned, [x.cpu() for x in (K, V)]):
+        for prefill in (False, True):
+            with mlkv.MLKVCache(1, h, d, [0], g, b, s) as c:
+                out = torch.zeros_like(Q)
+                if prefill:
+                    c.prefill(0, Q, k, v, out, lens)
+                else:
+                    c.load_prefix(0, k, v, s)
+                torch.cuda.synchronize()
+                np.testing.assert_array_equal(_read_cache(c, b, g, s, d), want_kv)
+                if prefill:
+                    assert torch.equal(out.view(torch.int16), want.view(torch.int16))
+                c.sync_status()
+
+
 def test_device_generator_matches_host_bits():
     import torch
 
