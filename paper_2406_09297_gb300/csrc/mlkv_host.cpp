@@ -148,13 +148,13 @@ struct mlkv_cache {
         std::vector<int> lens;
         int tile = -1, grid = -1, cluster = -1, pdl = -1, l2 = -1, tc = -1, pf = -1, sk = -1;
         int sg = -1;   // step_graph: a graph recorded under one mode is not replayed under another
-        int ef = -1, sf = -1;
+        int ef = -1, sf = -1, fd = -1, fk = -1;
         bool operator==(const StepKey &o) const
         {
             return Q == o.Q && K == o.K && V == o.V && out == o.out && lens == o.lens &&
                    tile == o.tile && grid == o.grid && cluster == o.cluster && pdl == o.pdl &&
                    l2 == o.l2 && tc == o.tc && pf == o.pf && sk == o.sk && sg == o.sg &&
-                   ef == o.ef && sf == o.sf;
+                   ef == o.ef && sf == o.sf && fd == o.fd && fk == o.fk;
         }
     } step_key, pending_key;   // recorded arguments; arguments seen once, not yet recorded
     int step_graph_replays = 0;
@@ -1436,6 +1436,8 @@ mlkv_cache::StepKey step_key_of(const mlkv_cache *c, const void *Q, const void *
     key.sg = c->step_graph;
     key.ef = c->early_fetch;
     key.sf = c->step_fused;
+    key.fd = c->fused_deep;
+    key.fk = c->fused_kc;
     return key;
 }
 

@@ -681,3 +681,42 @@ def test_step_right_behind_cache_writes(before, options):
             assert torch.equal(run(rep % 4, False).view(torch.int16),
                                expect[rep % 4].view(torch.int16)), rep
         cache.sync_status()
+
+
+@pytest.mark.parametrize("host", [False, True])
+@pytest.mark.parametrize("key,value", [
+    ("fused_deep", 0), ("fused_kc", 2), ("step_fused", 0), ("step_kernel", 0), ("tile_tokens", 64),
+    ("grid", 20), ("cluster", 0), ("pdl", 0), ("early_fetch", 0), ("l2_prefetch", 1), ("tc", 1),
+])
+def test_option_change_is_not_replayed(key, value, host):
+    # A recorded step is replayed only under the options it was recorded with.
+    import torch
+
+    import paper_2406_09297_gb300 as mlkv
+    owner, h, g, d, b, L = [0] * 6 + [6] * 6, 12, 1, 64, 4, 1000
+    lens = np.full(b, L, dtype=np.int32)
+    with mlkv.MLKVCache(12, h, d, owner, g, b, L) as cache:
+        qb, kn, vn = _inputs(owner, h, g, d, b, lens, L, 98, cache, None)
+        tensors = [to_dev(x) for x in (qb, kn, vn)]
+        tensors.append(torch.empty((12, b, h, d), dtype=torch.bfloat16, device="cuda"))
+        if host:
+            tensors = [x.cpu().pin_memory() for x in tensors]
+        call = cache.decode_step_host if host else cache.decode_step
+        cache.set_option("step_graph", 1)
+        cache.set_option("step_fused", 2)
+
+        def replayed():
+            before = cache.get_option("step_graph_replays")
+            call(*tensors, lens)
+            torch.cuda.synchronize()
+            return cache.get_option("step_graph_replays") - before
+
+        assert [replayed() for _ in range(3)] == [0, 1, 1]
+        old = cache.get_option(key)
+        assert old != value
+        cache.set_option(key, value)
+        assert replayed() == 0
+        if key == "fused_kc":
+            assert cache.get_option("last_fused_kc") == value
+        cache.set_option(key, old)
+        cache.sync_status()
