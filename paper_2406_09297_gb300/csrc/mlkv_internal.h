@@ -254,7 +254,7 @@ cudaError_t launch_combine(const DecodeParams &p, int head_dim, cudaStream_t str
 // sequences of up to 3000 positions, 8 KV heads of 128 with 4 heads each, 6 pieces at most: 529 ->
 // 505 us for 32 layers when the bound went from 4 to 8).  Larger records take several passes: 4.
 constexpr int kInlineMergeMaxPieces = 8;
-inline int inline_merge_pieces(int group, int d)
+constexpr int inline_merge_pieces(int group, int d)
 {
     return group * d <= 512 ? kInlineMergeMaxPieces : 4;
 }

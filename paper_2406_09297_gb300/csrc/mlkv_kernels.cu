@@ -82,9 +82,10 @@ struct Plan {
     // 165 us for 12 layers, 172 with one buffer; 145 once the buffer was freed before the counter).
     static constexpr int kRawBufs = (!kT && T == 256) ? 1 : 2;
     static constexpr int kRaw = STAGES * kStageBytes;                  // [kRawBufs][kRawBytes]
-    // an inline merge's weights [kInlineMergeMaxPieces][16] and reciprocals [16], f32
-    static constexpr int kEpiW = kRaw + kRawBufs * kRawBytes;
-    static constexpr int kFlags = kEpiW + (kInlineMergeMaxPieces + 1) * 16 * 4;   // int [4]
+    // records an inline merge may take (inline_merge_pieces of the largest group they are 8 for)
+    static constexpr int kMaxPieces = kT ? kInlineMergeMaxPieces : inline_merge_pieces(9, D);
+    static constexpr int kEpiW = kRaw + kRawBufs * kRawBytes;   // its weights, f32 [pieces][G]
+    static constexpr int kFlags = kEpiW + kMaxPieces * kRows * 4;   // int [4]
     // u64 full[S], empty[S], res_full[2], res_empty[2], cluster
     static constexpr int kBars = kFlags + 16;
     // Dynamic tail: per-sequence tables (lengths differ) or, in cluster mode with one raw buffer,
@@ -522,9 +523,9 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
             if (prev != static_cast<unsigned>(c_last - c_first))
                 continue;
             // This CTA finished the segment last: it merges records seg + c_first .. seg + c_last (at
-            // most kInlineMergeMaxPieces), o = sum_c 2^(lse_c - M) o_c / sum_c 2^(lse_c - M), M the
-            // largest lse, summed in the records' order and multiplied by the reciprocal at the end as
-            // the consumer warps do (merge4): the outputs do not depend on which CTA is last.
+            // most PL::kMaxPieces), o = sum_c 2^(lse_c - M) o_c / sum_c 2^(lse_c - M), M the
+            // largest lse; the weights first, then the sums in the records' order, as the consumer
+            // warps do (merge4): the outputs do not depend on which CTA is last.
             float *s_w = reinterpret_cast<float *>(smem + PL::kEpiW);
             const int np = c_last - c_first + 1;
             const size_t rec0 = static_cast<size_t>(seg + c_first);
@@ -532,9 +533,9 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
             // after the other, with the weights' chain through shared memory between them, was the
             // launch's last microsecond: 64 uneven segments over 138 CTAs, 32 heads of 128, 12.7 us a
             // layer, now 12.1.)
-            float lv[kInlineMergeMaxPieces];
+            float lv[PL::kMaxPieces];
 #pragma unroll
-            for (int c = 0; c < kInlineMergeMaxPieces; ++c)
+            for (int c = 0; c < PL::kMaxPieces; ++c)
                 lv[c] = (lane < G && c < np) ? __ldcg(&p.part_lse[(rec0 + c) * G + lane])
                                              : -__int_as_float(0x7f800000);
             bool weighed = false;
@@ -565,18 +566,18 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
                         if (lane < G) {
                             float mx = lv[0];
 #pragma unroll
-                            for (int k = 1; k < kInlineMergeMaxPieces; ++k)
+                            for (int k = 1; k < PL::kMaxPieces; ++k)
                                 mx = fmaxf(mx, lv[k]);
                             float tot = 0.f;
 #pragma unroll
-                            for (int k = 0; k < kInlineMergeMaxPieces; ++k) {
+                            for (int k = 0; k < PL::kMaxPieces; ++k) {
                                 lv[k] = fast_exp2(lv[k] - mx);   // 0 past the records
                                 tot += lv[k];
                             }
+                            const float inv = fast_rcp(tot);
 #pragma unroll
-                            for (int k = 0; k < kInlineMergeMaxPieces; ++k)
-                                s_w[k * G + lane] = lv[k];
-                            s_w[kInlineMergeMaxPieces * G + lane] = fast_rcp(tot);
+                            for (int k = 0; k < PL::kMaxPieces; ++k)
+                                s_w[k * G + lane] = lv[k] * inv;
                         }
                         __syncwarp();
                     }
@@ -596,12 +597,10 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
 #pragma unroll
                 for (int u = 0; u < CH; ++u) {
                     const int i = c0 + u * 128;
-                    if (i < G * D) {
-                        const float inv = s_w[kInlineMergeMaxPieces * G + i / D];
+                    if (i < G * D)
                         *reinterpret_cast<uint2 *>(ob + i) =
-                            make_uint2(pack_bf16x2(acc[u].x * inv, acc[u].y * inv),
-                                       pack_bf16x2(acc[u].z * inv, acc[u].w * inv));
-                    }
+                            make_uint2(pack_bf16x2(acc[u].x, acc[u].y),
+                                       pack_bf16x2(acc[u].z, acc[u].w));
                 }
             }
             __syncwarp();   // s_w may be rewritten
@@ -1038,20 +1037,23 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
 #pragma unroll
                 for (int k = 0; k < K; ++k)
                     mx = fmaxf(mx, l[k]);
-                float tot = 0.f;
+                float tot = 0.f, w[K];
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    w[k] = fast_exp2(l[k] - mx);   // 0 past the records
+                    tot += w[k];
+                }
+                const float inv = fast_rcp(tot);
                 float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                 for (int k = 0; k < K; ++k) {
-                    const float w = fast_exp2(l[k] - mx);   // 0 past the records
-                    tot += w;
-                    a.x = fmaf(w, x[k].x, a.x);
-                    a.y = fmaf(w, x[k].y, a.y);
-                    a.z = fmaf(w, x[k].z, a.z);
-                    a.w = fmaf(w, x[k].w, a.w);
+                    const float f = w[k] * inv;
+                    a.x = fmaf(f, x[k].x, a.x);
+                    a.y = fmaf(f, x[k].y, a.y);
+                    a.z = fmaf(f, x[k].z, a.z);
+                    a.w = fmaf(f, x[k].w, a.w);
                 }
-                const float inv = fast_rcp(tot);
-                return make_uint2(pack_bf16x2(a.x * inv, a.y * inv),
-                                  pack_bf16x2(a.z * inv, a.w * inv));
+                return make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
             };
             if (mode == 2) {
                 // Leader: its own result is in warp 0's rows; merge the other ranks' once landed.
@@ -1101,10 +1103,10 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
 #pragma unroll 1
                     for (int i = 4 * ctid; i < G * D; i += kPass) {
                         const int row = i / D;
-                        float lv[kInlineMergeMaxPieces];
-                        float4 ov[kInlineMergeMaxPieces];
+                        float lv[PL::kMaxPieces];
+                        float4 ov[PL::kMaxPieces];
 #pragma unroll
-                        for (int k = 0; k < kInlineMergeMaxPieces; ++k) {
+                        for (int k = 0; k < PL::kMaxPieces; ++k) {
                             lv[k] = NEG_INF;
                             ov[k] = make_float4(0.f, 0.f, 0.f, 0.f);
                             if (k < np) {
