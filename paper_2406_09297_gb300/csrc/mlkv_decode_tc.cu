@@ -71,8 +71,7 @@ struct TcPlan {
     static constexpr int kPBytes = T * 32;            // P^T [2][T][8] bf16
     static constexpr int kResO = 16 * D * 4;          // a piece's result: o[16][D] f32
     static constexpr int kResBytes = kResO + 16 * 4 + 32;   // + lse[16] + 8 ints of metadata
-    // weights of an inline merge, pieces x heads (8 x 8 or 4 x 16 at most), and a reciprocal a head
-    static constexpr int kEpiCap = 64 + 16;
+    static constexpr int kEpiCap = 64;                // weights of an inline merge (below)
     static constexpr int kQ = STAGES * kStageBytes;   // [2][kQBytes]
     static constexpr int kP = kQ + 2 * kQBytes;       // [2][kPBytes]
     static constexpr int kRes = kP + 2 * kPBytes;     // [2][kResBytes]
@@ -93,6 +92,10 @@ struct TcPlan {
     static_assert(D == 64 || D == 128, "head_dim 64 or 128");
     static_assert(kQ % 1024 == 0 && kQBytes % 1024 == 0, "swizzled query blocks stay aligned");
     static_assert(kResBytes % 16 == 0, "result slots stay 16-byte aligned");
+    // 8 records up to the group size they are allowed for (8 heads of 64, 4 of 128), else 4
+    static_assert(inline_merge_pieces(512 / D, D) * (512 / D) <= kEpiCap &&
+                      inline_merge_pieces(512 / D + 1, D) * 16 <= kEpiCap,
+                  "an inline merge's weights");
 };
 
 // ------------------------------------------------------------------------------------------------
@@ -827,13 +830,17 @@ __global__ void __launch_bounds__(TcPlan<D, T, STAGES>::kThreads, 1)
                             float tot = 0.f, ax = 0.f, ay = 0.f;
 #pragma unroll
                             for (int k = 0; k < kInlineMergeMaxPieces; ++k) {
-                                const float w = fast_exp2(lv[k] - mx);   // 0 past np
-                                tot += w;
+                                lv[k] = fast_exp2(lv[k] - mx);   // 0 past np
+                                tot += lv[k];
+                            }
+                            const float inv = fast_rcp(tot);
+#pragma unroll
+                            for (int k = 0; k < kInlineMergeMaxPieces; ++k) {
+                                const float w = lv[k] * inv;
                                 ax = fmaf(w, ovv[k].x, ax);
                                 ay = fmaf(w, ovv[k].y, ay);
                             }
-                            const float inv = fast_rcp(tot);
-                            *reinterpret_cast<uint32_t *>(ob + i) = pack_bf16x2(ax * inv, ay * inv);
+                            *reinterpret_cast<uint32_t *>(ob + i) = pack_bf16x2(ax, ay);
                         }
                         if (tid == 0)
                             p.counters[seg] = 0u;

@@ -524,9 +524,9 @@ enum : int { kMetaBeta = 0, kMetaJ, kMetaSeg, kMetaWhole, kMetaFirst, kMetaLast,
 // goes straight to `out`.  Otherwise the slot becomes partial record seg + cta; the counter of the
 // segment (acquire-release) tells the CTA that finished it last, which merges all its records:
 //   o = sum_c 2^(lse_c - M) o_c / sum_c 2^(lse_c - M),  M = max_c lse_c,
-// summed in the records' order and multiplied by the reciprocal at the end, as the softmax warps do
-// when their piece is the last: the outputs do not depend on which CTA that is.  s_w: room for
-// (kInlineMergeMaxPieces records or 4, see inline_merge_pieces) x G weights and G reciprocals.
+// the weights first, then the sums in the records' order, as the softmax warps do when their piece
+// is the last: the outputs do not depend on which CTA that is.  s_w: room for the weights of
+// inline_merge_pieces records of G rows.
 template <int D>
 __device__ __forceinline__ void epilogue_piece(const DecodeParams &p, const float *ro,
                                                const float *rlse, const int *meta, float *s_w,
@@ -569,7 +569,6 @@ __device__ __forceinline__ void epilogue_piece(const DecodeParams &p, const floa
     const int np = c_last - c_first + 1;
     const size_t rec0 = static_cast<size_t>(seg + c_first);
     const float NEG_INF = -__int_as_float(0x7f800000);
-    float *s_inv = s_w + np * G;
     for (int i = lane; i < np * G; i += 32)
         s_w[i] = __ldcg(&p.part_lse[rec0 * G + i]);
     __syncwarp();
@@ -583,7 +582,9 @@ __device__ __forceinline__ void epilogue_piece(const DecodeParams &p, const floa
             s_w[k * G + lane] = w;
             tot += w;
         }
-        s_inv[lane] = fast_rcp(tot);
+        const float inv = fast_rcp(tot);
+        for (int k = 0; k < np; ++k)
+            s_w[k * G + lane] *= inv;
     }
     __syncwarp();
     // Each lane owns CH float4 columns of a 128*CH-element chunk; the loads of all its columns for
@@ -626,10 +627,9 @@ __device__ __forceinline__ void epilogue_piece(const DecodeParams &p, const floa
         for (int u = 0; u < CH; ++u) {
             const int i = c0 + u * 128 + lane * 4;
             if (i < G * D) {
-                const float inv = s_inv[i / D];
                 uint2 w2;
-                w2.x = pack_bf16x2(acc[u].x * inv, acc[u].y * inv);
-                w2.y = pack_bf16x2(acc[u].z * inv, acc[u].w * inv);
+                w2.x = pack_bf16x2(acc[u].x, acc[u].y);
+                w2.y = pack_bf16x2(acc[u].z, acc[u].w);
                 *reinterpret_cast<uint2 *>(ob + i) = w2;
             }
         }
