@@ -531,20 +531,22 @@ static int decode_impl(mlkv_cache_t c, int layer, const void *K_new, const void 
     bool uniform = true;
     for (int beta = 1; beta < c->b; ++beta)
         uniform = uniform && seq_lens[beta] == seq_lens[0];
-    if (!uniform && var->v->smem_bytes + mlkv::table_bytes(c->b) > c->max_smem) {
-        // The per-sequence tables do not fit beside this variant's ring: take the 64-position
-        // tile variant, whose ring is small.
+    static thread_local mlkv::DecodeParams p;
+    size_t smem = mlkv::decode_smem(*var->v, uniform, c->b, &p.raw_bufs);
+    if (smem > c->max_smem) {
+        // The per-sequence tables do not fit beside this variant's ring (the tcgen05 kernel's long
+        // tiles): take the 64-position tile variant, whose ring is small.
         var = nullptr;
         for (auto &v : c->variants)
-            if (v.v->tile_tokens == 64 && v.v->smem_bytes + mlkv::table_bytes(c->b) <= c->max_smem)
+            if (v.v->tile_tokens == 64)
                 var = &v;
-        if (var == nullptr)
+        if (var == nullptr ||
+            (smem = mlkv::decode_smem(*var->v, uniform, c->b, &p.raw_bufs)) > c->max_smem)
             return fail(MLKV_ERR_UNSUPPORTED, "batch %d too large for varied lengths", c->b);
     }
     const int T = var->v->tile_tokens;
 
     // Stream-K style split: tiles of all (beta, j) segments end to end, equal runs per CTA.
-    static thread_local mlkv::DecodeParams p;
     long long tiles = 0;
     for (int beta = 0; beta < c->b; ++beta) {
         p.tile_start[beta] = static_cast<int>(tiles);
@@ -711,9 +713,8 @@ static int decode_impl(mlkv_cache_t c, int layer, const void *K_new, const void 
         winp = &win;
     }
     DeviceGuard guard(c->device);
-    const size_t smem = var->v->smem_bytes +
-                        (cluster_k > 1 ? (cluster_k - 1) * var->v->res_bytes
-                                       : (uniform ? 0 : mlkv::table_bytes(c->b)));
+    if (cluster_k > 1)   // one length only
+        smem += (cluster_k - 1) * var->v->res_bytes;
     cudaError_t e = mlkv::launch_decode(*var->v, grid, smem, static_cast<cudaStream_t>(cuda_stream),
                                         &var->tmap, &var->tmap_rows, p, winp, c->pdl != 0);
     if (e != cudaSuccess)
@@ -1133,15 +1134,6 @@ static int issue_step_ml(mlkv_cache_t c, const char *Q, const char *K, const cha
     mlkv_cache::Variant *var = pick_variant(c, mean_len);
     if (var == nullptr || var->v->tc)
         return MLKV_OK;
-    if (!uniform && var->v->smem_bytes + mlkv::table_bytes(c->b) > c->max_smem) {
-        var = nullptr;   // the per-sequence tables need the small-ring variant
-        for (auto &v : c->variants)
-            if (v.v->tile_tokens == 64 && !v.v->tc &&
-                v.v->smem_bytes + mlkv::table_bytes(c->b) <= c->max_smem)
-                var = &v;
-        if (var == nullptr)
-            return MLKV_OK;
-    }
     const long long S = static_cast<long long>(c->b) * c->g;
     // Sequences longest first (stable); items ranked segment-major over them.
     static thread_local std::vector<int> perm;
@@ -1333,7 +1325,7 @@ static int issue_step_ml(mlkv_cache_t c, const char *Q, const char *K, const cha
     if (stage != nullptr && (e = mlkv::launch_stage_copy(*stage, static_cast<cudaStream_t>(stream))) !=
                                 cudaSuccess)
         return fail_cuda(e, "copy-in of the step's inputs");
-    const size_t smem = var->v->smem_bytes + (uniform ? 0 : mlkv::table_bytes(c->b));
+    const size_t smem = mlkv::decode_smem(*var->v, uniform, c->b, &p.raw_bufs);
     e = mlkv::launch_decode(*var->v, grid, smem, static_cast<cudaStream_t>(stream), &var->tmap,
                             &var->tmap_rows, p, nullptr, c->pdl != 0);
     if (e != cudaSuccess)

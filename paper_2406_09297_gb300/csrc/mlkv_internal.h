@@ -53,6 +53,8 @@ struct DecodeParams {
                               // step's first layer: the layers behind it read cache rows, queries
                               // and new tokens before their own wait, so every kernel that came
                               // before the step must have ended); 0: at once
+    int raw_bufs;             // decode_kernel: buffers of raw sums between the consumer warps and the
+                              // epilogue warp, 1 or 2 (decode_smem)
     int newest_ready;         // 1: the segments' newest rows are replaced from K_new/V_new by this
                               // grid: no wait before a segment's last tile
     int store_new;            // with K_new: 1 = also store the new token in the cache (the owner
@@ -192,6 +194,8 @@ struct DecodeVariant {
     size_t res_bytes;         // what cluster mode adds k-1 times (0: the slots lie within smem_bytes)
     const void *fn;
     int tc = 0;               // 1: decode_tc_kernel (tcgen05, TMEM), 0: decode_kernel (mma.sync)
+    size_t raw2_bytes = 0;    // of smem_bytes: the second raw-sum buffer, which a launch may do without
+    int min_blocks = 1;       // CTAs per SM the variant is built for
 };
 
 // The tcgen05 variants (mlkv_decode_tc.cu).
@@ -199,7 +203,18 @@ extern const DecodeVariant kTcVariants[];
 extern const int kNumTcVariants;
 
 // Shared memory a launch adds for the per-sequence tables (only when lengths differ).
-inline size_t table_bytes(int batch) { return ((8 * static_cast<size_t>(batch) + 4) + 15) & ~15ull; }
+constexpr size_t table_bytes(int batch) { return ((8 * static_cast<size_t>(batch) + 4) + 15) & ~15ull; }
+
+// A launch's shared memory (without cluster slots) and raw-sum buffers: one of them where the tables
+// would otherwise cost a resident CTA (an SM's 228 KB, 1 KB of them the system's per CTA).
+inline size_t decode_smem(const DecodeVariant &v, bool uniform, int batch, int *raw_bufs)
+{
+    const size_t tables = uniform ? 0 : table_bytes(batch);
+    const bool two =
+        v.raw2_bytes > 0 && v.min_blocks * (v.smem_bytes + tables + 1024) <= 228 * 1024;
+    *raw_bufs = two ? 2 : 1;
+    return v.smem_bytes - (two ? 0 : v.raw2_bytes) + tables;
+}
 
 // Returns the compiled variant for (head_dim, tile_tokens) of the tcgen05 kernel (tc = 1) or of
 // the mma.sync kernel (tc = 0; for query groups of `group` heads), or nullptr.

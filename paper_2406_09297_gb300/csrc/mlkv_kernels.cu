@@ -77,39 +77,46 @@ struct Plan {
     static constexpr int kRawMeta = kRawO + 2 * 16 * NCW * 4;
     static constexpr int kRawLse = kRawMeta + 32;
     static constexpr int kRawBytes = kRawLse + 64;
-    // Two buffers where shared memory has room for them beside the ring: the epilogue warp takes
-    // ~1.3 us to merge a piece's warps (64 uneven sequences of up to 2048 positions, 12 heads of 64:
-    // 165 us for 12 layers, 172 with one buffer; 145 once the buffer was freed before the counter).
-    static constexpr int kRawBufs = (!kT && T == 256) ? 1 : 2;
-    static constexpr int kRaw = STAGES * kStageBytes;                  // [kRawBufs][kRawBytes]
+    // Two buffers where shared memory has room for them: the epilogue warp takes ~1.3 us to merge a
+    // piece's warps (64 uneven sequences of up to 2048 positions, 12 heads of 64: 165 us for 12
+    // layers, 172 with one buffer; 145 once the buffer was freed before the counter).
+    static constexpr int kMaxRawBufs = (!kT && T == 256) ? 1 : 2;
+    static constexpr int kRaw = STAGES * kStageBytes;                  // the first buffer
     // records an inline merge may take (inline_merge_pieces of the largest group they are 8 for)
     static constexpr int kMaxPieces = kT ? kInlineMergeMaxPieces : inline_merge_pieces(9, D);
-    static constexpr int kEpiW = kRaw + kRawBufs * kRawBytes;   // its weights, f32 [pieces][G]
+    static constexpr int kEpiW = kRaw + kRawBytes;              // its weights, f32 [pieces][G]
     static constexpr int kFlags = kEpiW + kMaxPieces * kRows * 4;   // int [4]
     // u64 full[S], empty[S], res_full[2], res_empty[2], cluster
     static constexpr int kBars = kFlags + 16;
-    // Dynamic tail: per-sequence tables (lengths differ) or, in cluster mode with one raw buffer,
-    // the leader's slots for the other ranks' results ([k-1][kResBytes]).
     // Per-stage query slots: the G rows of the segment whose first tile the stage holds, each row
     // padded by 16 bytes so that the fragment loads (8 rows apart) fall in distinct banks.
     static constexpr int kQRow = D * 2 + 16;
     static constexpr int kQSlot = kRows * kQRow;
     static constexpr int kQ = (kBars + (2 * STAGES + 5) * 8 + 8 + 127) / 128 * 128;
-    static constexpr int kTables = kQ + STAGES * kQSlot;
-    static constexpr int kBytes = kTables;
-    // A cluster's CTAs hold one piece each, so the leader's slots can lie in its second raw buffer.
-    static constexpr bool kClusterInRaw = kRawBufs == 2;
-    static constexpr int kCluster = kClusterInRaw ? kRaw + kRawBytes : kTables;
+    // The tail: the second raw buffer (DecodeParams::raw_bufs == 2) and, lengths differing, the
+    // per-sequence tables.  A cluster's leader keeps the slots for the other ranks' results
+    // ([k-1][kResBytes]) there: its CTAs hold one piece each, so in the second buffer if there is
+    // one.
+    static constexpr int kTail = kQ + STAGES * kQSlot;
+    static constexpr int kBytes = kTail + (kMaxRawBufs - 1) * kRawBytes;
+    static constexpr bool kClusterInRaw = kMaxRawBufs == 2;
     static_assert(!kClusterInRaw || 3 * kResBytes <= kRawBytes, "slots of three ranks");
     static constexpr int kAlloc = kBytes + 1024;      // base aligned up to 1024 in the kernel
     static_assert(kTW % 16 == 0, "each warp takes whole 16-position mma steps");
-    static_assert(NCW == 4 || NCW == 8, "tree merge over 4 or 8 warps");
+    static_assert(NCW == 4, "a statistics row of every warp is one 16-byte load");
     static_assert(D == 64 || D == 128, "head_dim 64 or 128");
     static_assert(T <= 256, "TMA box height");
     static_assert(kResBytes % 16 == 0, "result slots stay 16-byte aligned");
-    static_assert(kMinBlocks * (kAlloc + 1024) <= 228 * 1024, "shared memory of the resident CTAs");
-    static_assert(kRawBufs <= 2, "two pairs of raw-buffer barriers");
-    static_assert(kRawBytes % 16 == 0 && kRawMeta % 16 == 0, "raw buffers stay 16-byte aligned");
+    // Uneven lengths cost a launch no resident CTA and no tile length at any batch: where two raw
+    // buffers and the tables do not fit, one does.  (While they did not, 800 uneven sequences of up
+    // to 3000 positions, 12 layers of one KV head: 926 us, 670 with one.)
+    static constexpr size_t kUneven =
+        kAlloc - (kMaxRawBufs - 1) * kRawBytes + table_bytes(MLKV_MAX_BATCH);
+    static_assert(kMinBlocks * (kAlloc + 1024) <= 228 * 1024 &&
+                      kMinBlocks * (kUneven + 1024) <= 228 * 1024,
+                  "shared memory of the resident CTAs");
+    static_assert(kRawBytes % 16 == 0 && kRawMeta % 16 == 0 && kTail % 16 == 0,
+                  "raw buffers and tables stay 16-byte aligned");
 };
 
 
@@ -177,7 +184,10 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
     const uint32_t bar_res_empty = bar_res_full + 16;        // [2]
     const uint32_t bar_cluster = bar_res_empty + 16;         // leader: k-1 remote arrivals
     volatile int *flags = reinterpret_cast<volatile int *>(smem + PL::kFlags);
-    int *s_len = reinterpret_cast<int *>(smem + PL::kTables);
+    // raw sums: one or two buffers, buffer rb at raw_at(rb)
+    const int two = PL::kMaxRawBufs == 2 ? p.raw_bufs - 1 : 0;
+    auto raw_at = [&](int rb) { return rb ? PL::kTail : PL::kRaw; };
+    int *s_len = reinterpret_cast<int *>(smem + PL::kTail + two * PL::kRawBytes);
     int *s_start = s_len + p.b;
 
     const int warp = threadIdx.x >> 5;
@@ -425,9 +435,9 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
         // m*), o = sum_w 2^(m_w - m*) o_w / l*, lse = m* + log2 l*.
         constexpr int FS = PL::kRawRow;
         for (int k = 0;; ++k) {
-            const int rb = k % PL::kRawBufs;
+            const int rb = k & two;
             int ok = 1;
-            if (lane == 0 && !mbar_wait(bar_res_full + 8 * rb, (k / PL::kRawBufs) & 1)) {
+            if (lane == 0 && !mbar_wait(bar_res_full + 8 * rb, (k >> two) & 1)) {
                 flags[0] = 1;
                 atomicOr(p.err, kErrWaitFull);
                 ok = 0;
@@ -435,7 +445,7 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok)
                 break;
-            uint8_t *slot = smem + PL::kRaw + rb * PL::kRawBytes;
+            uint8_t *slot = smem + raw_at(rb);
             const int *meta = reinterpret_cast<const int *>(slot + PL::kRawMeta);
             if (meta[kMetaStop])
                 break;
@@ -898,10 +908,10 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
         // the next piece (a tree over the warps with a barrier per level held all of them up for
         // ~2 us a piece at head_dim 128).
         constexpr int FS = PL::kRawRow;
-        const int rb = nhand % PL::kRawBufs;
-        uint8_t *slot_raw = smem + PL::kRaw + rb * PL::kRawBytes;
-        if (nhand >= PL::kRawBufs && !flags[0] &&
-            !mbar_wait(bar_res_empty + 8 * rb, ((nhand / PL::kRawBufs) & 1) ^ 1)) {
+        const int rb = nhand & two;
+        uint8_t *slot_raw = smem + raw_at(rb);
+        if (nhand > two && !flags[0] &&
+            !mbar_wait(bar_res_empty + 8 * rb, ((nhand >> two) & 1) ^ 1)) {
             flags[0] = 1;
             atomicOr(p.err, kErrWaitEmpty);
         }
@@ -968,8 +978,8 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
             const int mode = whole ? 0 : (p.cluster_k > 1 ? (rank != 0 ? 1 : 2) : 3);
             if (early && mode == 3)
                 grid_dependency_wait();   // partial records and counters are shared scratch
-            const uint32_t cslots = sbase + PL::kCluster;
-            const uint8_t *cs = smem + PL::kCluster;
+            const uint32_t cslots = sbase + PL::kTail;
+            const uint8_t *cs = smem + PL::kTail;
             uint32_t remote = 0, remote_bar = 0;
             if (mode == 1) {
                 remote = map_to_rank(cslots + (rank - 1) * PL::kResBytes, 0);
@@ -1129,10 +1139,9 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
     // Tell the epilogue warp that no piece follows (the buffer is this piece's own; with no tiles at
     // all it was never used).
     {
-        const int rb = nhand % PL::kRawBufs;
+        const int rb = nhand & two;
         if (warp == 0 && lane == 0)
-            reinterpret_cast<int *>(smem + PL::kRaw + rb * PL::kRawBytes + PL::kRawMeta)[kMetaStop] =
-                1;
+            reinterpret_cast<int *>(smem + raw_at(rb) + PL::kRawMeta)[kMetaStop] = 1;
         __syncwarp();
         if (lane == 0)
             mbar_arrive(bar_res_full + 8 * rb);
@@ -1317,7 +1326,8 @@ constexpr DecodeVariant make_variant()
     using PL = Plan<D, T, STAGES, NCW, kT>;
     return DecodeVariant{D, T, STAGES, PL::kThreads, static_cast<size_t>(PL::kAlloc),
                          PL::kClusterInRaw ? 0 : static_cast<size_t>(PL::kResBytes),
-                         reinterpret_cast<const void *>(&decode_kernel<D, T, STAGES, NCW, kT>)};
+                         reinterpret_cast<const void *>(&decode_kernel<D, T, STAGES, NCW, kT>), 0,
+                         static_cast<size_t>((PL::kMaxRawBufs - 1) * PL::kRawBytes), PL::kMinBlocks};
 }
 
 // (head_dim, positions per tile, ring stages, consumer warps) for groups of more than 8 heads, and

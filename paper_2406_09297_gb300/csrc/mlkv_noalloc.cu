@@ -154,18 +154,12 @@ extern "C" int mlkv_decode_attention_static(const void *kv_slot, int batch, int 
         return fail(st.status, st.error.c_str());
 
     // Tile length by the regular path's default rule (mlkv::default_tile_tokens, over the
-    // batch * kv_heads segments); 64 when the per-sequence tables do not fit beside the ring.
+    // batch * kv_heads segments).
     const double mean_len = static_cast<double>(len_sum) / batch;
-    int T = mlkv::default_tile_tokens(head_dim, mean_len, batch * kv_heads);
+    const int T = mlkv::default_tile_tokens(head_dim, mean_len, batch * kv_heads);
     const mlkv::DecodeVariant *v = mlkv::find_decode_variant(head_dim, T, 0, G);
     if (v == nullptr)
         return fail(MLKV_ERR_UNSUPPORTED, "no decode variant");
-    if (!uniform && v->smem_bytes + mlkv::table_bytes(batch) > st.max_smem) {
-        T = 64;
-        v = mlkv::find_decode_variant(head_dim, T, 0, G);
-        if (v == nullptr || v->smem_bytes + mlkv::table_bytes(batch) > st.max_smem)
-            return fail(MLKV_ERR_UNSUPPORTED, "batch too large for varied lengths");
-    }
 
     static thread_local mlkv::DecodeParams p;
     long long tiles = 0;
@@ -269,7 +263,7 @@ extern "C" int mlkv_decode_attention_static(const void *kv_slot, int batch, int 
     p.Q_next = nullptr;
     p.deferred_merge =
         mlkv::max_pieces_per_segment(p, T, grid) > mlkv::inline_merge_pieces(G, head_dim) ? 1 : 0;
-    const size_t smem = v->smem_bytes + (uniform ? 0 : mlkv::table_bytes(batch));
+    const size_t smem = mlkv::decode_smem(*v, uniform, batch, &p.raw_bufs);
     e = mlkv::launch_decode(*v, grid, smem, stream, &tmap, &tmap_rows, p, nullptr);
     if (e != cudaSuccess)
         return fail(MLKV_ERR_CUDA, "decode launch failed");

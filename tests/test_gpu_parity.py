@@ -265,3 +265,13 @@ def test_split_merges_are_reproducible(h, g, d, b, s, options):
         for out in outs[1:]:
             assert torch.equal(out.view(torch.int16), outs[0].view(torch.int16))
         cache.sync_status()
+
+
+@pytest.mark.parametrize("h", [8, 12, 16])
+@pytest.mark.parametrize("tile", [64, 128, 256])
+def test_largest_uneven_batch_keeps_its_tile(h, tile):
+    # The length tables of the largest batch fit beside every variant's shared memory.
+    b = 1024
+    lens = [1 + (i * 37) % 270 for i in range(b)]
+    run_small_case([0], h, 1, 64, b, lens, 270, seed=36, fused=True,
+                   options={"tile_tokens": tile}, expect={"last_tile_tokens": tile})
