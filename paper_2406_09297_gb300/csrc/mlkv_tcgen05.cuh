@@ -37,9 +37,9 @@ __host__ __device__ constexpr uint32_t umma_idesc(int M, int N, int a_mn, int b_
 
 constexpr uint32_t kLayoutInterleave = 0, kLayoutSw128 = 2;
 
-// True in one thread of the (converged) warp.  A thread picked this way issues tcgen05.mma from
-// uniform registers; one picked by its lane number costs more instructions an MMA (measured: M 128
-// x N 64 x K 16 with P from TMEM 34 cycles against 47 alone and 64 beside busy softmax warps).
+// True in one thread of the (converged) warp.  A thread picked this way issues tcgen05.mma faster
+// than one picked by its lane number (measured, M 128 x N 64 x K 16 with P from TMEM: 34 cycles an
+// MMA against 47 alone and 64 beside busy softmax warps).
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t e;
