@@ -201,16 +201,23 @@ def test_cluster_rule_keeps_a_streaming_grid():
                    expect={"last_cluster_k": 0, "last_deferred_merge": 1})
 
 
-@pytest.mark.parametrize("d,tile", [(64, 64), (64, 128), (64, 256), (128, 64), (128, 128)])
-@pytest.mark.parametrize("pieces,deferred", [(5, 0), (7, 0), (9, 1)])
-def test_merge_of_five_to_nine_pieces(d, tile, pieces, deferred):
-    # One long segment a KV head over `pieces` CTAs: where a segment can meet at most 8 CTAs its
-    # records are merged by the last finisher, else by the merge launch (runs of 2 tiles: a segment
-    # of 2 k tiles meets k CTAs, and the bound for runs that start anywhere is k + 1).
+@pytest.mark.parametrize("d,tile,tc", [(64, 64, 0), (64, 128, 0), (64, 256, 0), (128, 64, 0),
+                                       (128, 128, 0), (64, 128, 1), (64, 256, 1), (128, 128, 1)])
+@pytest.mark.parametrize("pieces,G,deferred", [
+    (5, 3, 0), (7, 3, 0), (9, 3, 1),
+    (7, 512, 0), (3, 513, 0), (4, 513, 1), (7, 513, 1), (3, 16, 0), (4, 16, 1),
+])
+def test_merge_of_few_pieces(d, tile, tc, pieces, G, deferred):
+    # One long segment a KV head over `pieces` CTAs: where a segment can meet at most 8 CTAs (4 for
+    # records of more than 512 floats) its records are merged by the last finisher, else by the merge
+    # launch (runs of 2 tiles: a segment of 2 k tiles meets k CTAs, and the bound for runs that start
+    # anywhere is k + 1).  G of 512 and 513: the largest group of the 8-record bound, one more.
+    if G >= 512:
+        G = 512 // d + G - 512
     nt = 2 * pieces
-    run_small_case([0], 6, 2, d, 1, [nt * tile - 5], nt * tile, seed=31, fused=True,
-                   options={"grid": 2 * pieces, "tile_tokens": tile, "cluster": 0},
-                   expect={"last_deferred_merge": deferred})
+    run_small_case([0], 2 * G, 2, d, 1, [nt * tile - 5], nt * tile, seed=31, fused=True,
+                   options={"grid": 2 * pieces, "tile_tokens": tile, "cluster": 0, "tc": tc},
+                   expect={"last_deferred_merge": deferred, "last_tc": tc})
 
 
 @pytest.mark.parametrize("d,tile", [(64, 64), (64, 128), (64, 256), (128, 64), (128, 128)])

@@ -184,3 +184,103 @@ def test_prefill_out_over_prompt_kv(d, shared):
     for x, y in zip(results[0][0], results[1][0]):
         assert torch.equal(x.view(torch.int16), y.view(torch.int16))
     assert (results[0][1] == results[1][1]).all()
+
+
+@pytest.mark.parametrize("d,h,b", [(64, 12, 520), (128, 24, 520)])
+def test_prefill_more_units_than_one_launch(d, h, b):
+    # More than 6,144 units: an owner layer's several launches over the prompt's K/V in place, then
+    # the store behind the last, and the reader's launches over the slot.
+    import paper_2406_09297_gb300 as mlkv
+    s_max = 130
+    lens = [1 + (i * 61) % s_max for i in range(b)]
+    with mlkv.MLKVCache(2, h, d, [0, 0], 1 if d == 64 else 2, b, s_max) as cache:
+        ref = oracle.OracleCache([0, 0], h, 1 if d == 64 else 2, d, b, s_max)
+        _prefill_model([0, 0], h, 1 if d == 64 else 2, d, b, lens, s_max, s_max, 62, cache, ref,
+                       nthreads=8)
+
+
+@pytest.mark.parametrize("d,h,g", [(64, 12, 3), (128, 16, 4)])
+def test_prefill_among_other_calls_without_a_wait(d, h, g):
+    # A decode of the slot's old contents, the owner's prefill (K/V read in place, stored in its
+    # tail), its reader's prefill over the slot, the owner's and the reader's decode and a whole step,
+    # queued without a host wait: every output and the cache bit for bit as with one after each call.
+    import torch
+
+    import paper_2406_09297_gb300 as mlkv
+    from tests.test_gpu_cache import _read_cache
+    b, S, max_seq = 6, 900, 1000
+    prompts = np.array([900, 1, 333, 128, 650, 257], dtype=np.int32)
+
+    def rand(seed, *shape):
+        gen_ = torch.Generator(device="cuda").manual_seed(seed)
+        return torch.randn(shape, device="cuda", generator=gen_).bfloat16()
+
+    with mlkv.MLKVCache(2, h, d, [0, 0], g, b, max_seq) as cache:
+        q, pq = rand(1, 2, b, h, d), rand(2, 2, b, S, h, d)
+        kn, vn = rand(3, 1, b, g, d), rand(4, 1, b, g, d)
+        prompt_kv = [[rand(10 * r + i, b, g, S, d) for i in range(2)] for r in range(3)]
+        outs = [torch.empty_like(q[0]) for _ in range(4)] + [torch.empty_like(q)]
+        pouts = [torch.zeros_like(pq[0]) for _ in range(2)]
+
+        def run(r, wait):
+            def done():
+                if wait:
+                    torch.cuda.synchronize()
+            K, V = prompt_kv[r]
+            calls = [lambda: cache.decode_attention(1, q[1], outs[0], prompts),
+                     lambda: cache.prefill(0, pq[0], K, V, pouts[0], prompts),
+                     lambda: cache.prefill(1, pq[1], None, None, pouts[1], prompts),
+                     lambda: cache.decode_attention(0, q[0], outs[1], prompts),
+                     lambda: cache.append_decode_attention(0, kn[0], vn[0], q[0], outs[2], prompts + 1),
+                     lambda: cache.decode_attention(1, q[1], outs[3], prompts + 1),
+                     lambda: cache.decode_step(q, vn, kn, outs[4], prompts + 2)]
+            for call in calls:
+                call()
+                done()
+            torch.cuda.synchronize()
+            return [x.clone() for x in outs + pouts] + [
+                torch.from_numpy(_read_cache(cache, b, g, max_seq, d))]
+
+        run(2, True)
+        expect = [run(r, True) for r in range(3)]
+        for rep in range(12):
+            for x, y in zip(run(rep % 3, False), expect[rep % 3]):
+                assert torch.equal(x.view(torch.int16), y.view(torch.int16)), rep
+        cache.sync_status()
+
+
+@pytest.mark.parametrize("what", ["KV", "own KV", "Q"])
+def test_prefill_inputs_in_the_cache(what):
+    # K and V in another slot, in the layer's own slot, and queries in another slot: the prompt is
+    # stored before the attention.  Bits as from separate tensors.
+    import torch
+
+    import paper_2406_09297_gb300 as mlkv
+    from tests.test_gpu_cache import _DevArray, _read_cache
+    h, g, d, b, s = 8, 4, 64, 3, 300
+    prompts = np.array([300, 1, 129], dtype=np.int32)
+    Q = to_dev(gen.gen_q(63, 0, b * s, h, d).reshape(b, s, h, d))
+    K, V = (to_dev(gen.gen_kv(63, 0, i, b, g, s, d)) for i in range(2))
+    results = []
+    for inside in (False, True):
+        with mlkv.MLKVCache(2, h, d, [0, 1], g, b, s) as cache:
+            cache.load_prefix(0, K, V, s)
+            cache.load_prefix(1, K, V, s)
+            n = b * g * s * d
+            q, k, v = Q, K, V
+            if inside and what != "Q":
+                k, v = (torch.as_tensor(_DevArray(x, n), device="cuda").view(torch.bfloat16)
+                        for x in cache.kv_ptr(0 if what == "own KV" else 1)[:2])
+            elif what == "Q":
+                q = torch.as_tensor(_DevArray(cache.kv_ptr(1)[0], 2 * n), device="cuda").view(
+                    torch.bfloat16)[:Q.numel()].view(Q.shape)
+                q.copy_(Q)
+                if not inside:
+                    q = Q
+            out = torch.zeros((b, s, h, d), dtype=torch.bfloat16, device="cuda")
+            cache.prefill(0, q, k, v, out, prompts)
+            torch.cuda.synchronize()
+            cache.sync_status()
+            results.append((out, _read_cache(cache, b, g, s, d)))
+    assert torch.equal(results[0][0].view(torch.int16), results[1][0].view(torch.int16))
+    np.testing.assert_array_equal(results[0][1], results[1][1])
