@@ -54,6 +54,13 @@ namespace {
 // shared-memory plan
 // ------------------------------------------------------------------------------------------------
 
+// Whether CTAs of `bytes` shared memory are `blocks` times resident beside the largest batch's tables
+// (an SM's 228 KB, 1 KB of them the system's per CTA).
+constexpr bool uneven_fits(int blocks, int bytes)
+{
+    return blocks * (bytes + table_bytes(MLKV_MAX_BATCH) + 1024) <= 228 * 1024;
+}
+
 // kRows: query rows the CTA keeps room for, 16 or (groups of at most 8 heads) 8.
 template <int D, int T, int STAGES, int NCW, bool kT>
 struct Plan {
@@ -110,11 +117,11 @@ struct Plan {
     // Uneven lengths cost a launch no resident CTA and no tile length at any batch: where two raw
     // buffers and the tables do not fit, one does.  (While they did not, 800 uneven sequences of up
     // to 3000 positions, 12 layers of one KV head: 926 us, 670 with one.)
-    static constexpr size_t kUneven =
-        kAlloc - (kMaxRawBufs - 1) * kRawBytes + table_bytes(MLKV_MAX_BATCH);
-    static_assert(kMinBlocks * (kAlloc + 1024) <= 228 * 1024 &&
-                      kMinBlocks * (kUneven + 1024) <= 228 * 1024,
+    static_assert(uneven_fits(kMinBlocks, kAlloc - (kMaxRawBufs - 1) * kRawBytes),
                   "shared memory of the resident CTAs");
+    // Two buffers fit at every batch: their number is no run-time value (which cost 2-3% of uneven
+    // layer calls over short sequences, groups of 3 heads).
+    static constexpr bool kTwoFit = kMaxRawBufs == 2 && uneven_fits(kMinBlocks, kAlloc);
     static_assert(kRawBytes % 16 == 0 && kRawMeta % 16 == 0 && kTail % 16 == 0,
                   "raw buffers and tables stay 16-byte aligned");
 };
@@ -185,7 +192,7 @@ __global__ void __launch_bounds__(Plan<D, T, STAGES, NCW, kT>::kThreads,
     const uint32_t bar_cluster = bar_res_empty + 16;         // leader: k-1 remote arrivals
     volatile int *flags = reinterpret_cast<volatile int *>(smem + PL::kFlags);
     // raw sums: one or two buffers, buffer rb at raw_at(rb)
-    const int two = PL::kMaxRawBufs == 2 ? p.raw_bufs - 1 : 0;
+    const int two = PL::kMaxRawBufs == 1 ? 0 : PL::kTwoFit ? 1 : p.raw_bufs - 1;
     auto raw_at = [&](int rb) { return rb ? PL::kTail : PL::kRaw; };
     int *s_len = reinterpret_cast<int *>(smem + PL::kTail + two * PL::kRawBytes);
     int *s_start = s_len + p.b;
