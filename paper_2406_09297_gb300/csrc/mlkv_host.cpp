@@ -520,8 +520,9 @@ static int decode_impl(mlkv_cache_t c, int layer, const void *K_new, const void 
     mean_len /= c->b;
     // Inside a decode step, a layer that is one long segment (d = 64) runs on the 128-position
     // tile (two CTAs per SM) over 64 CTAs, so the next layers' grids stream beside it (measured,
-    // batch 1, 131072 positions, 12 layers: MLKV-2 81.9 us against 96.3 us for the 256-position
-    // tile on the one-wave split, MQA 95.8 against 119.7; 48 or 76 CTAs were slower than 64).
+    // batch 1, 131072 positions, per-layer steps of 12 layers: MLKV-2 63 us against 86 for the
+    // 256-position tile on the one-wave split and 114 for the 128-position one there, MQA 78
+    // against 104 and 129).
     const bool single_long = in_step && c->tile_tokens == 0 && c->grid <= 0 && c->d == 64 &&
                              c->b * c->g == 1 && seq_lens[0] >= 16384;
     mlkv_cache::Variant *var = pick_variant(c, mean_len, single_long ? 128 : 0);
@@ -565,7 +566,7 @@ static int decode_impl(mlkv_cache_t c, int layer, const void *K_new, const void 
     // model in units of one tile's consumer work (~0.5 us on GB300 when the tile is in L2):
     // a DSMEM cluster merge costs ~2 tiles, the last-CTA merge of partial records ~6 (a
     // global write, an atomic and the reads, after the previous layer has finished) and the
-    // separate combine launch ~7.
+    // separate combine launch ~7.  (Fitted before the raw-sum hand-over made merges cheaper.)
     const long long wave = std::min<long long>(
         std::min(var->ctas_per_sm * c->sm_count, c->max_ctas), tiles);
     const long long per_wave = (tiles + wave - 1) / wave;
@@ -580,10 +581,9 @@ static int decode_impl(mlkv_cache_t c, int layer, const void *K_new, const void 
         // the previous layer before writing partials) of at most half the resident slots lets
         // several layers stream at once.  It pays while the one-wave split would cut at least
         // half the segments (S <= 2 waves) and the segments are enough to stream (S >= 32).
-        // Measured per step: 64 segments of 16 tiles of 128, 64 CTAs 59.1 us against 64.8 us
-        // for 2-CTA clusters; 256 segments of 32 tiles of 256, 64 CTAs of 4 segments 872 us
-        // against 917 us; but 3072 segments 13.9 ms against 10.3 ms, and 8 or 24 segments
-        // (batch 8) 2-4% slower than the clusters.
+        // Measured per per-layer step of 12 layers: 32 segments of 16 tiles of 128 35.0 us
+        // against 37.6 for 2-CTA clusters, 64 segments 60.0 against 59.8, 256 segments of 32
+        // tiles of 256 902 against 897 for the one-wave split.
         if (S_all >= 32 && S_all <= 2 * wave) {
             for (long long gw = std::min(S_all, slots / 2); gw >= 1; --gw) {
                 if (S_all % gw == 0) {
@@ -618,12 +618,11 @@ static int decode_impl(mlkv_cache_t c, int layer, const void *K_new, const void 
                 // layer, which the tile-unit model does not see.  So there the largest cluster
                 // size whose grid fits twice wins while each CTA keeps >= 4 tiles and the grid
                 // still holds a quarter of the resident CTAs, enough copies in flight to stream
-                // (measured, 64 segments of 16 tiles of 128: 2-CTA clusters 80.5 us per 12-layer
-                // step against 84.7 us for 4-CTA clusters; with 32 segments 4-CTA clusters, 128
-                // CTAs, stay the better).  A layer that nothing overlaps (a standalone call, the
-                // first layer of a step, a step without early fetch) takes the model's choice:
-                // 4-CTA clusters there, 99.8 against 123.9 us for the default workload's 12
-                // layers one after another.
+                // (measured, 64 segments of 16 tiles of 128: 2-CTA clusters 59.8 us per 12-layer
+                // step against 82.1 us for 4-CTA clusters).  A layer that nothing overlaps (a
+                // standalone call, the first layer of a step, a step without early fetch) takes
+                // the model's choice: 4-CTA clusters there, 90.4 against 119.4 us for 12 such
+                // layer calls.
                 if (c->cluster == 1 && var->ctas_per_sm >= 2 && early_fetch == 1) {
                     for (int k : {4, 2}) {
                         if (cluster_k == 0 && nt % k == 0 && nt / k >= 4 && 2 * S * k <= wave &&
@@ -753,12 +752,12 @@ int mlkv_append_decode_attention(mlkv_cache_t c, int layer, const void *K, const
 
 // The fused decode's context split for nblk blocks: kc key tiles of 128 positions a unit; *units
 // (if given) the units it makes.  Measured on GB300 (batch 64 x 2048 positions, 72 rows a unit):
-// one CTA keeps an SM's softmax and tensor core about as busy as two do, while every unit costs
-// ~5 us outside its key tiles (start, first loads, output) and a split adds the merge launch (16
-// tiles a unit, 128 units: 31 us per step; 8 tiles, 256 units: 39; 4: 43; 1: 63).  So a sequence is
-// split only as far as the units still fit one per SM: the smallest kc whose units number at most
-// the SMs; no split when the (sequence, KV head, block) units alone exceed them.  The unit word
-// holds chunk indices below kFusedMaxChunks.
+// one CTA keeps an SM's softmax and tensor core about as busy as two do, while every unit has its
+// start, first loads and output outside its key tiles and a split adds the merge launch (16 tiles a
+// unit, 128 units: 18.3 us per step; 8 tiles, 256 units: 26.0; 4: 28.0; 2: 30.9; 1: 42.4).  So a
+// sequence is split only as far as the units still fit one per SM: the smallest kc whose units
+// number at most the SMs; no split when the (sequence, KV head, block) units alone exceed them.  The
+// unit word holds chunk indices below kFusedMaxChunks.
 static int fused_plan(const mlkv_cache *c, const int *seq_lens, int nblk, long long *units)
 {
     int n_kt_max = 0;
@@ -979,16 +978,18 @@ static bool fused_step_applies(const mlkv_cache *c, const int *seq_lens, bool ho
         if (c->owner[n] != n - n % L || c->slot[n] != n / L)
             return false;
     if (c->step_fused == 1) {
-        // Where the fused form pays, from measurements on GB300 against the decode kernel's
-        // launch.  A block of one layer shares nothing across layers (MHA, GQA-4, MQA at batch
-        // 256 and 1: 7-16% slower fused); blocks of two saved little or lost (batch 64 x 2000
-        // positions 49 vs 53 us, batch 256 x 8192 535 vs 548, batch 1 x 131072 66 vs 62, batch
-        // 1 x 128 11.6 vs 10.3; with the split-key CTA form 53.2 vs 52.6, 548.9 vs 548.0, 60.3
-        // vs 59.3, 12.5 vs 10.7).  For blocks of >= 3 layers the estimates in us per step, from the
-        // same measurements: the fused form ~1.1 per key tile its busiest SM takes plus ~6 fixed
-        // (+3 for the merge of a split); the decode kernel ~0.55 per (layer, sequence, KV head,
-        // 128 positions) item per SM plus ~3.  They pick the measured winner at batch 8, 64, 128
-        // and 256, batch 1 x 131072 and Llama-2-7B shapes.
+        // Where the fused form pays against the decode kernel's launch.  A block of one layer
+        // shares nothing across layers (MHA, GQA-4 and MQA, batch 8 to 256: 3-50% slower fused;
+        // only one sequence of 16384 gains, 19.8 -> 15.9 us); blocks of two are refused as well.
+        // For blocks of >= 3 layers the estimates in us per step: the fused form ~1.1 per key tile
+        // its busiest SM takes plus ~6 fixed (+3 for the merge of a split); the decode kernel
+        // ~0.55 per (layer, sequence, KV head, 128 positions) item per SM plus ~3.
+        // Both were fitted to former kernels, and the fused one has gained more since.  Now, decode
+        // / fused: right where they are far apart (12 layers in 2 blocks, 64 x 2000: 44.5 / 18.5;
+        // 32 layers in 8, 32 x 2000 positions, 8 KV heads: 735 / 353; one of 128 positions 6.1 /
+        // 8.8), but too careful between: 2 blocks, one of 16384 19.3 / 12.0; 4 blocks, 8 uneven
+        // of up to 16000 38.3 / 19.5; blocks of two, 256 x 2000 179 / 145 and one of 131072 65 /
+        // 41 all go to the decode kernel.
         if (L < 3)
             return false;
         long long units = 0;
@@ -1194,9 +1195,9 @@ static int issue_step_ml(mlkv_cache_t c, const char *Q, const char *K, const cha
         // tiles, plus one tile's worth for each partial record it writes) is taken.  Between the
         // 256-position tile (one CTA per SM, three stages) and the 128-position one (two CTAs per
         // SM) the 256 one is taken unless it gives a CTA more than one item beyond the 128 one's
-        // (measured at batch 1, 131072 positions: MLKV-2 59.4 -> 52.9 us, MLKV-6 71.6 -> 62.8,
-        // MQA 93.4 -> 89.4; GQA-4, 9 items a CTA against 5: 250 -> 260, so 128 there).  A forced
-        // tile size (option "tile") is used as it is.
+        // (measured at batch 1, 131072 positions, with the tile length forced to 128 / 256: MLKV-2
+        // 50.2 / 40.7 us, MLKV-6 51.2 / 45.4, MQA 68.4 / 65.7; GQA-4, 9 items a CTA against 5: 226
+        // / 230, so 128 there).  A forced tile size (option "tile_tokens") is used as it is.
         struct Chunked {
             bool ok = false;
             Plan plan{};

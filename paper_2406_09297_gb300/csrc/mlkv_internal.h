@@ -237,9 +237,11 @@ cudaError_t launch_decode(const DecodeVariant &v, int grid, size_t smem, cudaStr
 // (sequence, KV head) pairs of mean length mean_len.  Longer tiles move more bytes per TMA
 // request and per barrier round trip; shorter ones waste less on short sequences.  For d = 64 the
 // 128-position variant is small enough for two CTAs per SM, so the next layer's CTAs start (and
-// fetch) while this layer's last ones finish: measured faster for many segments of moderate
-// length (64 x 2048: 85 vs 89 us a step; 512 x ~2048: 527 vs 560), slower for few long segments
-// or HBM-bound layers (1 x 131072, 256 x 8192).  mean_len < 0 means "unknown" (reports the
+// fetch) while this layer's last ones finish.  Measured, us of 12 layer calls with tiles of 128 /
+// 256: 512 uneven segments of ~2048 588 / 604, 64 of 2048 90.4 / 89.4, 30 uneven ones of up to 1000
+// 105 / 73, 1 of 131072 174 / 137, 256 of 8192 976 / 995.  d = 128, 32 calls with tiles of 64 / 128:
+// 64 uneven segments of up to 800 258 / 221, 256 of up to 400 484 / 353: the shorter tile below 512
+// does not pay for many uneven segments there.  mean_len < 0 means "unknown" (reports the
 // long-sequence choice).
 inline int default_tile_tokens(int d, double mean_len, int segments)
 {
@@ -265,9 +267,15 @@ cudaError_t launch_combine(const DecodeParams &p, int head_dim, cudaStream_t str
 
 // Pieces per segment above which the decode launch defers its merges to combine_kernel, for records
 // of `group` rows of d floats.  A record of at most 512 floats is one pass of the consumer threads,
-// so up to 8 of them are one round trip to L2, against ~3 us a layer for the separate launch (8
-// sequences of up to 3000 positions, 8 KV heads of 128 with 4 heads each, 6 pieces at most: 529 ->
-// 505 us for 32 layers when the bound went from 4 to 8).  Larger records take several passes: 4.
+// so up to 8 of them are one round trip to L2, against ~3 us a layer for the separate launch.
+// Larger records take several passes: 4.  Measured with a bound of 4 / 8 everywhere, us of layer
+// calls, uneven lengths up to 3000 (equal ones of 3000):
+//   512 floats (8 KV heads of 128, 4 heads each, 8 sequences, 32 layers)    439 / 387
+//   768 (one KV head of 64, 12 heads, 30 sequences, 12 layers)              138 / 119
+//   1024 (4 KV heads of 128, 8 heads each, 8 sequences (10), 32 layers)     361 / 355 (422 / 426)
+//   2048 (2 KV heads of 128, 16 heads each, 16 sequences (20), 32 layers)   442 / 456 (528 / 511)
+// The tcgen05 kernel takes the same bound (4 KV heads of 64, 3 heads each, 8 sequences, 12 layers:
+// 187 / 163).
 constexpr int kInlineMergeMaxPieces = 8;
 constexpr int inline_merge_pieces(int group, int d)
 {

@@ -17,16 +17,15 @@
 //   mbarrier transaction counts.  Each tile is fetched from HBM exactly once and used by all G
 //   query heads of the group.
 //
-//   Math.  NCW consumer warps (4 or 8) split every tile by positions.  Scores S = Q K^T and the
-//   update
-//   O += P V run on the tensor cores (mma.sync m16n8k16, bf16 in, fp32 accumulate) with the
-//   query group padded to M = 16 rows; the softmax is online, in fp32, base 2 with the 1/sqrt(d)
-//   scale folded into the exponent, with quad shuffles for row maxima.  At the end of a piece each
-//   warp leaves its raw sums in shared memory and goes on; the epilogue warp merges them (the
-//   CTA's last piece: all consumer warps, after one barrier).  With the former tree over the
-//   consumer warps, a barrier a level, a piece boundary cost ~2 us at head_dim 128 (measured, 64
-//   uneven segments over 138 CTAs: layer calls 16.2 -> 13.4 us with the merge of up to 8 records
-//   in the launch, below).
+//   Math.  Four consumer warps split every tile by positions.  Scores S = Q K^T and the update
+//   O += P V run on the tensor cores (mma.sync m16n8k16, bf16 in, fp32 accumulate), the query group
+//   padded to 16 rows or (at most 8 heads) to 8 columns; the softmax is online, in fp32, base 2
+//   with the 1/sqrt(d) scale folded into the exponent, with shuffles for the maxima.  At the end of
+//   a piece each warp leaves its raw sums in shared memory and goes on; the epilogue warp merges
+//   them (the CTA's last piece: all consumer warps, after one barrier).  With the former tree over
+//   the consumer warps, a barrier a level, a piece boundary cost ~2 us at head_dim 128 (measured,
+//   64 uneven segments over 138 CTAs: layer calls 16.2 -> 13.4 us with the merge of up to 8 records
+//   in the launch, below; 12.1 now).
 //
 //   Launch.  Programmatic dependent launch: barrier set-up overlaps the previous kernel of the
 //   stream, and no global memory is touched before griddepcontrol.wait.
@@ -1176,8 +1175,10 @@ __global__ void __launch_bounds__(kCombineThreads)
     // The next layer's decode may start at once: it reads neither the partials nor `out`, and it
     // writes partials only after its own dependency wait (after this grid).
     grid_dependents_launch();
-    const bool tables = p.ml_layers <= 0 && p.uniform_len <= 0;   // reads the length tables
-    if (tables)
+    // Uneven lengths wait here, the others behind the divisions (below): there it measured no gain
+    // for them (3 sequences of up to 3,000 positions, 32 layers of 8 KV heads: 323 us here, 325).
+    const bool uneven = p.ml_layers <= 0 && p.uniform_len <= 0;
+    if (uneven)
         grid_dependency_wait();
     const int row = blockIdx.y;
     const int G = p.G;
@@ -1209,7 +1210,7 @@ __global__ void __launch_bounds__(kCombineThreads)
     // Behind the divisions, which overlap the decode grid's tail (one sequence of 5,000 positions, 32
     // layers of 8 KV heads: 304 us with the wait in front of them, 292).  A CTA that returns waits
     // too: this grid ends after the decode grid.
-    if (!tables)
+    if (!uneven)
         grid_dependency_wait();
     if (p.ml_layers <= 0 && np == 1)
         return;   // one CTA held the whole segment and wrote the output itself
@@ -1338,8 +1339,8 @@ constexpr DecodeVariant make_variant()
 }
 
 // (head_dim, positions per tile, ring stages, consumer warps) for groups of more than 8 heads, and
-// for those of at most 8; the first match of a (head_dim, tile) pair is used.  <64, 128, 2, 4> fits
-// twice on an SM (90 KB, 163 registers).
+// for those of at most 8; the first match of a (head_dim, tile) pair is used.  <64, 128, 2, 4> and
+// <64, 64, 4, 4> fit twice on an SM (87 to 112 KB, at most 168 registers).
 const DecodeVariant kVariants[2][5] = {
     {make_variant<64, 128, 2, 4, false>(), make_variant<64, 256, 3, 4, false>(),
      make_variant<64, 64, 4, 4, false>(), make_variant<128, 64, 4, 4, false>(),

@@ -267,8 +267,8 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
     if (threadIdx.x == 0) {
         for (int q = 0; q < NQ; ++q) {
             // the query tiles' barrier: the producer's tensor-map copy, or the loads from host
-            // memory by the last warp (deep form: by every softmax warp); freed by the unit's last S and, where the outputs are staged in
-            // the query tiles, by the softmax warps
+            // memory by the last warp (deep form: by every softmax warp); freed by the unit's last
+            // S and, where the outputs are staged in the query tiles, by the softmax warps
             mbar_init(bar_q + 8 * q,
                       kSplit && kFused && p.q_host != nullptr ? PL::kSoftWarps : 1);
             mbar_init(bar_q_free + 8 * q, 1 + (PL::kStageInQ ? PL::kSoftWarps : 0));
@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
         auto send_q = [&](const Unit &x) {
             const int qb = uc % NQ;
             if (kFused && p.q_host != nullptr) {
-                ++uc;   // the last warp reads the queries from host memory
+                ++uc;   // other warps read the queries from host memory (load_q_host)
                 return true;
             }
             if (uc >= NQ && !flags[0] &&
@@ -980,11 +980,9 @@ __global__ void __launch_bounds__(PrefillPlan<D, kForm>::kThreads,
                 tmem_fence_before();
             }
             if (PL::kStageInQ) {
-                // A warpgroup without a tile in this unit has waited for nothing in it: it must not
-                // run ahead into the barrier's next phase.
-                if (PL::kTiles == 2 && n_g == 0)
-                    wait(bar_q + 8 * qb, n / NQ);
-                // the next queries may be written over the stage
+                // The next queries may be written over the stage.  (Every warpgroup has a tile in
+                // every unit here: two query tiles at head_dim 64 are a fused block of more rows
+                // than one holds.)
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0)

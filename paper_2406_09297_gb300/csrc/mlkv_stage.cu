@@ -4,7 +4,7 @@
 // CPU-GPU link costs a launch.  Used by mlkv_decode_step_host to bring a step's Q and new K/V in
 // (one launch for all three); the decode kernels store the outputs into host memory themselves.
 // Also the store of every owner's new token into its slot for the fused step (one launch for all
-// owners, Sec. 3: only owner layers store K/V).
+// owners, Sec. 3: only owner layers store K/V), and the store of a prompt's K/V.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
