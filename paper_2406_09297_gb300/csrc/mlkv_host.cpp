@@ -985,7 +985,7 @@ static bool fused_step_applies(const mlkv_cache *c, const int *seq_lens, bool ho
         // its busiest SM takes plus ~6 fixed (+3 for the merge of a split); the decode kernel
         // ~0.55 per (layer, sequence, KV head, 128 positions) item per SM plus ~3.
         // Both were fitted to former kernels, and the fused one has gained more since.  Now, decode
-        // / fused: right where they are far apart (12 layers in 2 blocks, 64 x 2000: 44.5 / 18.5;
+        // / fused (steps called back to back, the host's planning included): right where they are far apart (12 layers in 2 blocks, 64 x 2000: 44.5 / 18.5;
         // 32 layers in 8, 32 x 2000 positions, 8 KV heads: 735 / 353; one of 128 positions 6.1 /
         // 8.8), but too careful between: 2 blocks, one of 16384 19.3 / 12.0; 4 blocks, 8 uneven
         // of up to 16000 38.3 / 19.5; blocks of two, 256 x 2000 179 / 145 and one of 131072 65 /
@@ -1195,9 +1195,10 @@ static int issue_step_ml(mlkv_cache_t c, const char *Q, const char *K, const cha
         // tiles, plus one tile's worth for each partial record it writes) is taken.  Between the
         // 256-position tile (one CTA per SM, three stages) and the 128-position one (two CTAs per
         // SM) the 256 one is taken unless it gives a CTA more than one item beyond the 128 one's
-        // (measured at batch 1, 131072 positions, with the tile length forced to 128 / 256: MLKV-2
-        // 50.2 / 40.7 us, MLKV-6 51.2 / 45.4, MQA 68.4 / 65.7; GQA-4, 9 items a CTA against 5: 226
-        // / 230, so 128 there).  A forced tile size (option "tile_tokens") is used as it is.
+        // (measured on the device at batch 1, 131072 positions, with the tile length forced to 128 /
+        // 256: MLKV-2 54.1 / 48.5 us, MLKV-6 64.7 / 57.1, MQA 88.2 / 85.2; GQA-4, 9 items a CTA
+        // against 5: 247 / 255, so 128 there).  Planning both takes the host 70 us a call, the
+        // 256-position one alone 30.  A forced tile size (option "tile_tokens") is used as it is.
         struct Chunked {
             bool ok = false;
             Plan plan{};
