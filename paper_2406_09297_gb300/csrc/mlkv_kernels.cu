@@ -109,7 +109,7 @@ struct Plan {
     static_assert(!kClusterInRaw || 3 * kResBytes <= kRawBytes, "slots of three ranks");
     static constexpr int kAlloc = kBytes + 1024;      // base aligned up to 1024 in the kernel
     static_assert(kTW % 16 == 0, "each warp takes whole 16-position mma steps");
-    static_assert(NCW == 4, "a statistics row of every warp is one 16-byte load");
+    static_assert(NCW == 4, "four consumer warps");
     static_assert(D == 64 || D == 128, "head_dim 64 or 128");
     static_assert(T <= 256, "TMA box height");
     static_assert(kResBytes % 16 == 0, "result slots stay 16-byte aligned");
