@@ -985,11 +985,12 @@ static bool fused_step_applies(const mlkv_cache *c, const int *seq_lens, bool ho
         // its busiest SM takes plus ~6 fixed (+3 for the merge of a split); the decode kernel
         // ~0.55 per (layer, sequence, KV head, 128 positions) item per SM plus ~3.
         // Both were fitted to former kernels, and the fused one has gained more since.  Now, decode
-        // / fused (steps called back to back, the host's planning included): right where they are far apart (12 layers in 2 blocks, 64 x 2000: 44.5 / 18.5;
-        // 32 layers in 8, 32 x 2000 positions, 8 KV heads: 735 / 353; one of 128 positions 6.1 /
-        // 8.8), but too careful between: 2 blocks, one of 16384 19.3 / 12.0; 4 blocks, 8 uneven
-        // of up to 16000 38.3 / 19.5; blocks of two, 256 x 2000 179 / 145 and one of 131072 65 /
-        // 41 all go to the decode kernel.
+        // / fused (steps called back to back, the host's planning included): right where they are
+        // far apart (12 layers in 2 blocks, 64 x 2000: 44.5 / 18.5; 32 layers in 8, 32 x 2000
+        // positions, 8 KV heads: 735 / 353; one of 128 positions 6.1 / 8.8), but too careful
+        // between: 2 blocks, one of 16384 19.3 / 12.0; 4 blocks, 8 uneven of up to 16000 38.3 /
+        // 19.5; blocks of two, 256 x 2000 179 / 145 and one of 131072 65 / 41 all go to the decode
+        // kernel.
         if (L < 3)
             return false;
         long long units = 0;
